@@ -436,24 +436,38 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
   T* oth = H.y[l];
   bool first = zero;
   int np = 0;
-  if (sizeof(T) == 4 && nu1 == 1 && zero && zero_restrict_rows_ok(lv.d) && aligned16(b) && aligned16(cur) &&
-      wait_error_flag()) {
-    // rows of 128 or 256 cells: the single pre-smoothing sweep from zero and
-    // the restriction in one pass, row-resident and fed by TMA
+  const bool one_pass = sizeof(T) == 4 && nu1 == 1 && zero && aligned16(b) && aligned16(x);
+  const bool rows = one_pass && zero_restrict_rows_ok(lv.d) && wait_error_flag();
+  const bool tile = one_pass && zero_restrict_ok(lv.d) && lv.d.n() <= (size_t(1) << 21);
+  bool packed = false;  // cur holds the black cells only
+  if (zero) {
+    // the cycle starts in whichever of the two fields its out-of-place passes
+    // lead from to x (a copy at the end would move the level once more)
+    const bool sw = rb_sweep_swaps<T>(lv.d, false, x, b);
+    int swaps = sw ? nu2 : 0;
+    if (rows)
+      swaps = nu2 > 0 ? nu2 : 1;  // without a post-smoothing sweep: the unpacking
+    else if (!tile && nu1 > 0)
+      swaps += (rb_sweep_swaps<T>(lv.d, true, x, b) ? 1 : 0) + (sw ? nu1 - 1 : 0);
+    if (swaps & 1) std::swap(cur, oth);
+  }
+  if (rows) {
+    // the single pre-smoothing sweep from zero and the restriction in one
+    // pass, row-resident and fed by TMA; only the black cells are stored
     prof_begin(P_RBGS32, g->s);
     launch_zero_restrict_rows(reinterpret_cast<const float*>(b), bshift, reinterpret_cast<float*>(cur),
                               reinterpret_cast<float*>(H.b[l + 1]), lv.d, st, zero_restrict_rows_default_zc(lv.d),
                               g->s);
-    prof_end(P_RBGS32, g->s, "zero_restrict_rows", 8.5 * sizeof(T) / 4.0 * lv.d.n());
-  } else if (sizeof(T) == 4 && nu1 == 1 && zero && zero_restrict_ok(lv.d) && aligned16(b) && aligned16(cur) &&
-             lv.d.n() <= (size_t(1) << 21)) {
+    prof_end(P_RBGS32, g->s, "zero_restrict_rows", 6.5 * lv.d.n());
+    packed = true;
+  } else if (tile) {
     // the single pre-smoothing sweep from zero and the restriction in one pass
     // (levels up to 128^3 cells; on larger ones the kernel is bound by its
     // shared-memory traffic and the two streaming kernels are faster)
     launch_zero_restrict(reinterpret_cast<const float*>(b), bshift, reinterpret_cast<float*>(cur),
                          reinterpret_cast<float*>(H.b[l + 1]), lv.d, st, g->s);
   } else {
-    if (nu1 == 0 && zero) IBRD_CUDA(cudaMemsetAsync(x, 0, sizeof(T) * lv.d.n(), g->s));
+    if (nu1 == 0 && zero) IBRD_CUDA(cudaMemsetAsync(cur, 0, sizeof(T) * lv.d.n(), g->s));
     for (int sweep = 0; sweep < nu1; ++sweep) {
       if (launch_rb_sweep<T>(cur, oth, b, bshift, lv.d, st, first, nullptr, 0, g->s) >= 0) std::swap(cur, oth);
       first = false;
@@ -464,15 +478,24 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
   int sweep = 0;
   if (nu2 >= 1) {
     // the coarse-grid correction inside the first post-smoothing sweep
-    const int r = launch_prolong_sweep<T>(H.x[l + 1], cur, oth, b, bshift, lv.d, st, nu2 == 1 ? part : nullptr,
-                                          part_cap, g->s);
+    const int r = launch_prolong_sweep<T>(H.x[l + 1], cur, packed, oth, b, bshift, lv.d, st,
+                                          nu2 == 1 ? part : nullptr, part_cap, g->s);
     if (r >= 0) {
       std::swap(cur, oth);
       np = nu2 == 1 ? r : 0;
       sweep = 1;
     }
   }
-  if (sweep == 0) launch_prolong8<T>(H.x[l + 1], cur, lv.d, g->s);
+  if (sweep == 0) {
+    if (packed) {
+      prof_begin(P_RBGS32, g->s);
+      launch_unpack_zero(reinterpret_cast<const float*>(cur), reinterpret_cast<const float*>(b), bshift,
+                         reinterpret_cast<float*>(oth), lv.d, st, g->s);
+      prof_end(P_RBGS32, g->s, "unpack_zero", 10.0 * lv.d.n());
+      std::swap(cur, oth);
+    }
+    launch_prolong8<T>(H.x[l + 1], cur, lv.d, g->s);
+  }
   for (; sweep < nu2; ++sweep) {
     const bool last = (sweep == nu2 - 1);
     const int r = launch_rb_sweep<T>(cur, oth, b, bshift, lv.d, st, false, last ? part : nullptr, part_cap, g->s);

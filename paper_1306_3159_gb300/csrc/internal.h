@@ -152,6 +152,10 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
                     double* part, int part_cap, cudaStream_t s);
 template <typename T>
 bool rb_sweep_fused_ok(Dims d);
+// Whether that sweep is out of place (a first sweep from zero when zero != 0;
+// x, b: the fields, for their alignment).
+template <typename T>
+bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b);
 // Launch shape of a red-black sweep kernel picked by the autotuner: tile width
 // tx (cells, fused sweep only: 32 or 64 for the tiled kernel, nx for the
 // row-resident kernel on levels it serves) and z-march depth zc (planes per
@@ -173,8 +177,8 @@ const SweepShape* tuned_sweep(int elem, int kind, Dims d);
 constexpr unsigned kDefaultWaitLimit = 1u << 24;
 int* wait_error_flag();
 unsigned wait_limit();
-// Row-resident FP32 sweep (sweep_rows.cu): rows of 128 or 256 cells, ny a
-// multiple of 8, nz even; the same contract as the fused sweep of
+// Row-resident FP32 sweep (sweep_rows.cu; levels: rows_sweep_ok, ny a
+// multiple of 8, nz even); the same contract as the fused sweep of
 // launch_rb_sweep (out of place, per-CTA partial sums of the new x when part
 // holds enough entries; returns their count or 0). zc = planes per CTA.
 bool rows_sweep_ok(Dims d);
@@ -184,16 +188,22 @@ int launch_rows_sweep(const float* xin, float* xout, const float* b, const doubl
 // The same sweep of xin + P xc (P the trilinear prolongation of the coarse
 // field xc, as launch_prolong8 adds it) without writing the corrected field:
 // the coarse-grid correction fused into the first post-smoothing sweep.
-// zc is made even.
-int launch_rows_prolong_sweep(const float* xc, const float* xin, float* xout, const float* b, const double* bshift,
-                              Dims d, Stencil st, int zc, double* part, int part_cap, cudaStream_t s);
+// packed: xin holds only the black cells (the sweep reads no others), nx / 2
+// per row, as launch_zero_restrict_rows writes them. zc is made even.
+int launch_rows_prolong_sweep(const float* xc, const float* xin, bool packed, float* xout, const float* b,
+                              const double* bshift, Dims d, Stencil st, int zc, double* part, int part_cap,
+                              cudaStream_t s);
 // The first sweep from zero fused with the residual restriction on the same
-// levels as the row-resident sweep: x = sweep(0), bc = mean over 8 children of
-// b - shift - A x (bc 8-byte aligned). zc = planes per CTA (made even).
+// levels as the row-resident sweep: xb = the black cells of x = sweep(0) (nx /
+// 2 per row; the red cells are (b - shift) / diag), bc = mean over 8 children
+// of b - shift - A x (bc 8-byte aligned). zc = planes per CTA (made even).
 bool zero_restrict_rows_ok(Dims d);
 int zero_restrict_rows_default_zc(Dims d);
-void launch_zero_restrict_rows(const float* b, const double* bshift, float* x, float* bc, Dims d, Stencil st,
+void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, float* bc, Dims d, Stencil st,
                                int zc, cudaStream_t s);
+// x from the packed black cells xb and b: the whole field after that sweep.
+void launch_unpack_zero(const float* xb, const float* b, const double* bshift, float* x, Dims d, Stencil st,
+                        cudaStream_t s);
 // Levels handled by the single-CTA coarse V-cycle (shared-memory resident).
 constexpr int kMaxSmallLevels = 12;
 struct CoarseLevels {
@@ -225,10 +235,11 @@ void launch_prolong8(const T* xc, T* x, Dims d, cudaStream_t s);
 // follows it, on levels the row-resident FP32 sweep serves: writes the swept
 // field to xout (xin is left uncorrected) and returns the partial-sum count
 // as launch_rb_sweep does, or -1 without launching when it does not apply
-// (the caller then prolongs and sweeps separately).
+// (the caller then prolongs and sweeps separately). packed: xin holds the
+// black cells only (launch_rows_prolong_sweep).
 template <typename T>
-int launch_prolong_sweep(const T* xc, const T* xin, T* xout, const T* b, const double* bshift, Dims d, Stencil st,
-                         double* part, int part_cap, cudaStream_t s);
+int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
+                         Stencil st, double* part, int part_cap, cudaStream_t s);
 // Coarsest exact solve x = G b with the circulant table G (dc.n() entries).
 template <typename T>
 void launch_coarse_solve(const T* table, const T* b, T* x, Dims dc, cudaStream_t s);

@@ -928,6 +928,12 @@ bool rb_sweep_fused_ok(Dims d) {
 }
 
 
+template <typename T>
+bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b) {
+  if (!aligned16(x) || !aligned16(b)) return false;
+  return rb_sweep_fused_ok<T>(d) || (sizeof(T) == 4 && zero && d.nx % 4 == 0);
+}
+
 template <typename T, int TX, bool ZERO>
 void sweep_launch(dim3 g, cudaStream_t s, const T* xin, T* xout, const T* b, const double* bshift, Dims d, int zc,
                   T inv, T off, double* part) {
@@ -1085,8 +1091,8 @@ void launch_zero_restrict(const float* b, const double* bshift, float* x, float*
 }
 
 template <typename T>
-int launch_prolong_sweep(const T* xc, const T* xin, T* xout, const T* b, const double* bshift, Dims d, Stencil st,
-                         double* part, int part_cap, cudaStream_t s) {
+int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
+                         Stencil st, double* part, int part_cap, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (rows_sweep_ok(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && aligned16(xc) && xin != xout &&
         b != xout && xc != xout && wait_error_flag()) {
@@ -1097,9 +1103,9 @@ int launch_prolong_sweep(const T* xc, const T* xin, T* xout, const T* b, const d
       if ((!tn || tn->tx == 0 || tn->tx == d.nx) && !(tp && tp->tx == 1)) {
         const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
         prof_begin(P_RBGS32, s);
-        const int r = launch_rows_prolong_sweep(xc, xin, xout, b, bshift, d, st, zc, part, part_cap, s);
-        // x, b and the coarse field read once, x written once
-        prof_end(P_RBGS32, s, "prolong_sweep_rows", (3.0 + 0.125) * sizeof(T) * d.n());
+        const int r = launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);
+        // x (or its black half), b and the coarse field read once, x written once
+        prof_end(P_RBGS32, s, "prolong_sweep_rows", ((packed ? 2.5 : 3.0) + 0.125) * sizeof(T) * d.n());
         return r;
       }
     }
@@ -1147,8 +1153,9 @@ void launch_vcycle_small(const CoarseLevels& lv, const T* b, T* x, const double*
                                   cudaStream_t);                                                            \
   template void launch_resid_restrict<T>(const T*, const T*, const double*, T*, Dims, Stencil, cudaStream_t); \
   template void launch_prolong8<T>(const T*, T*, Dims, cudaStream_t);                                       \
-  template int launch_prolong_sweep<T>(const T*, const T*, T*, const T*, const double*, Dims, Stencil, double*,   \
-                                       int, cudaStream_t);                                                   \
+  template int launch_prolong_sweep<T>(const T*, const T*, bool, T*, const T*, const double*, Dims, Stencil,   \
+                                       double*, int, cudaStream_t);                                         \
+  template bool rb_sweep_swaps<T>(Dims, bool, const T*, const T*);                                           \
   template bool rb_sweep_fused_ok<T>(Dims);
 IBRD_INST(double)
 IBRD_INST(float)

@@ -1,33 +1,63 @@
-// Row-resident red-black Gauss-Seidel sweep for large FP32 levels (Sec. III.E:
-// the multigrid smoother of the Helmholtz problem A = alpha I - chi L).
+// Row-resident red-black Gauss-Seidel kernels for FP32 levels (Sec. III.E: the
+// multigrid smoother of the Helmholtz problem A = alpha I - chi L): the sweep
+// (with the prolongation of the coarse correction fused in, after a coarse
+// solve) and the first sweep from zero with the residual restriction.
 //
 // One full sweep (red cells from the old black values, then black cells from
-// the new red values; red = (i + j + k) even) in one pass over memory, for
-// levels whose rows are 128 or 256 cells long:
+// the new red values; red = (i + j + k) even) in one pass over memory.
 //
-// * A warp owns whole x-rows: lane l holds the 4-cell groups 4 l + 128 s
-//   (s < NS = nx / 128) of its row, so the x-neighbours of a group's end cells
-//   come from the neighbouring lanes by shuffles, and the periodic wrap in x is
-//   the shuffle from lane 31 to lane 0. No x-halo exists.
+// Only the black values of the old x enter a sweep, and after a sweep the
+// residual of every black cell is zero, so between the two half-cycles of a
+// V-cycle a level keeps only its black cells: a packed field of nx / 2 values
+// per row. In a row of parity a = (j + k) & 1 the red cells are i = 2 m + a
+// and the black ones i = 2 m + 1 - a, m = 0 .. nx / 2 - 1. In packed rows the
+// six neighbours of entry m of one colour are, of the other colour,
+//   y and z: entry m of the adjacent rows and planes,
+//   x: entries m - 1, m where the neighbours' parity makes them lie to the
+//   left (nbr_sums with right = 0), m, m + 1 where to the right (right = 1);
+//   for a red cell right = a, for a black one right = 1 - a.
+// The x-pair (2 m, 2 m + 1) of a coarse cell holds one red cell, entry m, so
+// the restricted residual is off / 8 times the sum over the coarse cell's four
+// rows of the red entries' neighbour sums (the first sweep from zero leaves
+// b - diag x = 0 in its red cells), and the correction of a packed row needs
+// one interpolated value per coarse cell.
+//
+// * A warp owns x-rows: lane l holds the 4-cell groups l + 32 s (s < NS) of its
+//   row, two packed entries each. x-neighbours come from the neighbouring
+//   lanes by shuffles; the periodic wrap of rows of 128 NS cells is the shuffle
+//   from lane 31 to lane 0. Rows of other lengths leave lanes idle, rows above
+//   256 cells belong to two warps; there the outermost groups read their
+//   neighbour from the published row in shared memory.
 // * A CTA owns TY rows of every plane of a z-chunk, plus one halo row on each
 //   side in y whose red cells it also updates (the black cells at the tile's
 //   edge rows need them); the neighbouring CTA computes the same red values
 //   from the same old data, bit for bit.
-// * Planes arrive by TMA: one thread issues 3-D tensor-map box copies (the
-//   tile's rows plus 2-row halos of x, the tile's rows plus 1-row halos of b)
-//   into a ring of R planes, completing on one mbarrier per ring slot. The
-//   periodic wrap in y is the halo boxes' start row, taken modulo ny on the
-//   host side of the index (every box starts at x = 0, so the 16-byte rule on
-//   the innermost coordinate holds).
-// * Each thread keeps its row of planes p-2 .. p+1 in registers (the
-//   z-neighbours); only the y-neighbour rows are read from shared memory: the
-//   old rows for the red update of plane p, and the red cells after that
-//   update (a separate double-buffered array holding two values per 4-cell
-//   group, so no row is read while it is written) for the black update of
-//   plane p-1 in the same step. One barrier per plane; thread 0 alone waits
-//   on the TMA barriers, one plane ahead.
+// * Planes arrive by TMA: one thread issues tensor-map box copies (the tile's
+//   rows plus 2-row halos of x, 1-row halos of b) into a ring of stages, one
+//   mbarrier per stage. The periodic wrap in y is the halo boxes' start row,
+//   taken modulo ny on the host side of the index (every box starts at x = 0,
+//   so the 16-byte rule on the innermost coordinate holds; nx is a multiple of
+//   32, which keeps the boxes' shared-memory addresses on 128 bytes).
+// * Each thread keeps its row's neighbouring planes in registers (the
+//   z-neighbours); every row is published once in shared memory, packed and
+//   double-buffered, for the y-neighbours of the next step, so no row is read
+//   while it is written and one barrier per plane suffices; thread 0 alone
+//   waits on the TMA barriers, one stage ahead.
 // * Odd z-chunks march downwards, so that adjacent chunks meet at their
 //   common halo planes at the same time (L2 hits, not DRAM re-reads).
+//
+// What bounds them: the time of one step, that is the instructions of 22 warps
+// per SM (issue slots 40 % busy) and the shared-memory round trips between two
+// barriers. Three things set it, measured at 256^3 (ncu): the marches are
+// compiled for each parity of a row, so that choosing the red or the black half
+// of a group costs nothing (14.0 M warp instructions instead of 22.2 M); pairs
+// of cells are computed by the two-wide FP32 instructions; and a plane comes in
+// as few copies as possible, issued by a warp of its own (with nine copies per
+// plane from one of the marching threads every CTA took 40 us, with three 31
+// us). Sweep with the prolongation: 34 us for 176 MB (0.77 of the copy
+// bandwidth), 51 us for 210 MB when x was a full field. Sweep from zero and
+// restriction: 24 us for 109 MB (0.67), 36 us for 143 MB before. At 128^3: 12.6
+// and 8.7 us (13.8 and 10.0).
 //
 // Every mbarrier wait is bounded: a wait that gives up sets *err, drains the
 // copies still in flight (again with a bound) and ends the CTA; the host
@@ -35,16 +65,19 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 
 namespace ibrd {
 namespace {
 
-constexpr int kRowsTY = 8;    // tile rows per CTA
-constexpr int kRowsRing = 4;  // planes in the TMA ring (prefetch distance 2)
+constexpr int kRowsTY = 8;      // tile rows per CTA
+constexpr int kSweepRing = 3;   // TMA stages of the sweep (one plane of x and of b each)
+constexpr int kZeroRing = 4;    // TMA stages of the sweep from zero (one plane of b each)
 constexpr int kCoarseRing = 3;  // coarse planes in the ring of the fused prolongation
 constexpr unsigned kDrainLimit = 1u << 26;
 
@@ -53,8 +86,19 @@ __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)_
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+// One lane of the calling (whole) warp: the feeding warp runs its loop in all
+// lanes, with uniform addresses, and only the copies themselves are predicated.
+__device__ __forceinline__ unsigned elect_lane() {
+  unsigned r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes, unsigned lead) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(
+          bar),
+      "r"(bytes), "r"(lead)
+      : "memory");
 }
 // true when the phase with this parity completed within `limit` tries
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, unsigned limit) {
@@ -69,11 +113,13 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, unsigne
   }
   return false;
 }
-__device__ __forceinline__ void tma_load3(unsigned dst, const CUtensorMap* map, int x, int y, int z, unsigned bar) {
+__device__ __forceinline__ void tma_load4(unsigned dst, const CUtensorMap* map, int y, int z, unsigned bar,
+                                          unsigned lead) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-      "[%5];\n" ::"r"(dst),
-      "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      "{\n .reg .pred p;\n setp.ne.u32 p, %6, 0;\n"
+      " @p cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %2, %3, %4}], "
+      "[%5];\n}\n" ::"r"(dst),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(0), "r"(y), "r"(z), "r"(bar), "r"(lead)
       : "memory");
 }
 
@@ -82,98 +128,227 @@ __device__ __forceinline__ int wrapm(int i, int n) {
   return i < 0 ? i + n : i;
 }
 
-// Gauss-Seidel update of the active cells of one row held as NS 4-vectors
-// per lane: active cells are e = a, a + 2 of every group (e = x mod 4). Their
-// x-neighbours are inactive cells (unchanged by this update): inside the
-// group, or the previous lane's last cell (a = 0) / the next lane's first
-// cell (a = 1), with lane 0 / lane 31 taking it from the adjacent slot. zm and
-// zp are the planes k - 1 and k + 1, bb the right-hand side with its shift
-// removed. The y-neighbours (rows j - 1, j + 1) are full rows (u, dn: float4
-// per group, the active cells' values at components a, a + 2) or, PACKED,
-// the neighbour rows' red-updated cells only (float2 per group: exactly the
-// values at this row's black positions).
-template <int NS, bool PACKED>
-__device__ __forceinline__ void rb_row(float4 (&v)[NS], const void* u, const void* dn, const float4 (&zm)[NS],
-                                       const float4 (&zp)[NS], const float4 (&bb)[NS], int a, float off, float inv,
-                                       int lane) {
-  float t[NS];
-  auto nb = [&](const void* row, int s, int k) -> float {  // k-th active cell's neighbour in `row`
-    if constexpr (PACKED) {
-      const float2 q = reinterpret_cast<const float2*>(row)[32 * s];
-      return k == 0 ? q.x : q.y;
-    } else {
-      const float4 q = reinterpret_cast<const float4*>(row)[32 * s];
-      return a == 0 ? (k == 0 ? q.x : q.z) : (k == 0 ? q.y : q.w);
+// CTA barriers that different warps may reach at different instructions (each
+// warp runs its own copy of the march), and one that also ORs a flag.
+__device__ __forceinline__ void cta_sync() { asm volatile("barrier.cta.sync.aligned 0;\n" ::: "memory"); }
+__device__ __forceinline__ bool cta_sync_or(bool flag) {
+  unsigned r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred.aligned q, 0, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((unsigned)flag)
+      : "memory");
+  return r != 0;
+}
+
+// Tensor maps of a field: boxes of the tile's rows with their halos on both
+// sides, with one halo, and of one halo.
+struct RowMaps {
+  CUtensorMap all, part, halo;
+};
+
+// Rows y0 - HALO .. y0 + ROWS + HALO - 1 (periodic in ny) of plane z into dst
+// (rows of nx values). As few copies as the periodic wrap allows (each costs
+// the issuing warp about 90 cycles, and three or six of them per plane decide
+// the pace of a march): one box inside the domain, two at one edge of it, single
+// halos when the domain is one tile.
+template <int ROWS, int HALO>
+__device__ __forceinline__ void load_rows(float* dst, int nx, const RowMaps& m, int y0, int ny, int z, unsigned bar,
+                                          unsigned lead) {
+  const bool low = y0 >= HALO, high = y0 + ROWS + HALO <= ny;
+  if (low && high) {
+    tma_load4(smem_u32(dst), &m.all, y0 - HALO, z, bar, lead);
+  } else if (low) {
+    tma_load4(smem_u32(dst), &m.part, y0 - HALO, z, bar, lead);
+    tma_load4(smem_u32(dst + (ROWS + HALO) * nx), &m.halo, 0, z, bar, lead);
+  } else if (high) {
+    tma_load4(smem_u32(dst), &m.halo, ny - HALO, z, bar, lead);
+    tma_load4(smem_u32(dst + HALO * nx), &m.part, y0, z, bar, lead);
+  } else {
+    for (int r = -HALO; r < ROWS + HALO; r += HALO)
+      tma_load4(smem_u32(dst + (r + HALO) * nx), &m.halo, wrapm(y0 + r, ny), z, bar, lead);
+  }
+}
+
+// A CTA's warps: WPR for each of the tile's rows and its two halo rows, and one
+// that feeds them.
+template <int WPR>
+constexpr int kRowsThreads = ((kRowsTY + 2) * WPR + 1) * 32;
+
+// The feeding warp of a march over planes 0 .. last: it issues the
+// stages' copies (up to `first` before the march, up to i + ahead at step i, when
+// the ring slot they take is free) and polls their barriers, stage i + 1 in step
+// i; the CTA barrier that ends every step publishes the landed stage. When a
+// wait gives up it issues and waits no more (dead), drains the copies in flight
+// and sets *err; the CTA learns of it at every sixth step and stops, what it
+// wrote since being invalid. The barriers pair with those of the marching warps.
+template <typename Issue, typename Wait>
+__device__ __forceinline__ void feed_stages(int last, int first, int ahead, Issue&& issue, Wait&& wait_stage,
+                                            unsigned limit, int* err) {
+  const unsigned lead = elect_lane();
+  bool dead = false;
+  int issued = -2, landed = -2;
+  auto feed = [&](int upto_issue, int upto_wait) {
+    if (dead) return;
+    while (issued < min(upto_issue, last - 1)) issue(++issued, lead);
+    while (!dead && landed < min(upto_wait, last - 1)) {
+      if (__all_sync(0xffffffffu, wait_stage(landed + 1, limit)))
+        ++landed;
+      else
+        dead = true;
     }
   };
-  if (a == 0) {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) t[s] = __shfl_sync(0xffffffffu, v[s].w, (lane + 31) & 31);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const float L = lane == 0 ? t[(s + NS - 1) % NS] : t[s];
-      const float u0 = nb(u, s, 0), d0 = nb(dn, s, 0), u1 = nb(u, s, 1), d1 = nb(dn, s, 1);
-      v[s].x = (bb[s].x + off * (((L + v[s].y) + (u0 + d0)) + (zm[s].x + zp[s].x))) * inv;
-      v[s].z = (bb[s].z + off * (((v[s].y + v[s].w) + (u1 + d1)) + (zm[s].z + zp[s].z))) * inv;
-    }
-  } else {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) t[s] = __shfl_sync(0xffffffffu, v[s].x, (lane + 1) & 31);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const float R = lane == 31 ? t[(s + 1) % NS] : t[s];
-      const float u0 = nb(u, s, 0), d0 = nb(dn, s, 0), u1 = nb(u, s, 1), d1 = nb(dn, s, 1);
-      v[s].y = (bb[s].y + off * (((v[s].x + v[s].z) + (u0 + d0)) + (zm[s].y + zp[s].y))) * inv;
-      v[s].w = (bb[s].w + off * (((v[s].z + R) + (u1 + d1)) + (zm[s].w + zp[s].w))) * inv;
-    }
+  bool ok = true;
+  for (int i = -1; ok && i < last; ++i) {
+    // i = -1: the stages the march starts from; i = 0: they have been read
+    if (i) feed(i < 0 ? first : i + ahead, i < 0 ? 1 : i + 1);
+    __syncwarp();
+    if (i < 0 || (i > 0 && i % 6 == 0))
+      ok = !cta_sync_or(dead);
+    else
+      cta_sync();
+  }
+  if (dead) {
+    while (landed < issued) wait_stage(++landed, kDrainLimit);
+    if (lead) atomicOr(err, 1);
   }
 }
 
-// Adds to the fine row v the coarse correction of Sec. III.E (cell-centred
-// trilinear prolongation) in the order every prolongation kernel uses: z
-// between the row's parent coarse plane cp and the other plane co, then y
-// between the parent coarse row cr and its neighbour nr on the row's side
-// (coarse planes in shared memory, NX / 2 floats per row), then x. Lane l
-// holds, per slot s, fine cells 4 g .. 4 g + 3 of group g = l + 32 s, over
-// coarse cells 2 g, 2 g + 1; their x-neighbours 2 g - 1 and 2 g + 2 come from
-// the adjacent lanes (lane 0 / 31 from the adjacent slot: the periodic wrap).
-template <int NS>
-__device__ __forceinline__ void add_correction(float4 (&v)[NS], const float* cp, const float* co, int cr, int nr,
-                                               int lane) {
-  constexpr int NXC = 64 * NS;
-  float2 zy[NS];  // the pair after z and y (16 times its value)
-  float tp[NS], tn[NS];
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const int o = 2 * (lane + 32 * s);
-    const float2 pp = *reinterpret_cast<const float2*>(cp + cr * NXC + o);
-    const float2 op = *reinterpret_cast<const float2*>(co + cr * NXC + o);
-    const float2 pn = *reinterpret_cast<const float2*>(cp + nr * NXC + o);
-    const float2 on = *reinterpret_cast<const float2*>(co + nr * NXC + o);
-    zy[s] = make_float2(prolong_axis(prolong_axis(pp.x, op.x), prolong_axis(pn.x, on.x)),
-                        prolong_axis(prolong_axis(pp.y, op.y), prolong_axis(pn.y, on.y)));
+// Two FP32 operations in one instruction, each rounded as the scalar one is:
+// the kernels below are bound by the instructions they issue, and their cells
+// come in pairs.
+__device__ __forceinline__ unsigned long long bits2(float2 a) {
+  return ((unsigned long long)__float_as_uint(a.y) << 32) | __float_as_uint(a.x);
+}
+__device__ __forceinline__ float2 pair2(unsigned long long a) {
+  return make_float2(__uint_as_float((unsigned)a), __uint_as_float((unsigned)(a >> 32)));
+}
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+  return pair2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+  return pair2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)), "l"(bits2(c)));
+  return pair2(r);
+}
+// prolong_axis and prolong_add on pairs
+__device__ __forceinline__ float2 prolong_axis2(float2 n, float2 f) { return fma2(dup2(3.f), n, f); }
+__device__ __forceinline__ float2 prolong_add2(float2 x, float2 t64) { return fma2(dup2(0x1p-6f), t64, x); }
+
+// Rows as a kernel sees them. NXT: the row length fixed at compile time (0: taken at
+// run time); WPR: warps per row; NS: groups per lane.
+template <int NS, int WPR, int NXT>
+struct Row {
+  static constexpr bool kWrap = NXT == 128 * NS && WPR == 1;  // one full warp holds the whole row
+  int nx, lane, g0, gw;  // row length; this lane's group of slot 0; groups per warp
+  __device__ __forceinline__ Row(int nx_, int warp_in_row) {
+    nx = NXT ? NXT : nx_;
+    lane = threadIdx.x & 31;
+    gw = nx / (4 * WPR);
+    g0 = warp_in_row * gw + lane;
   }
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    tp[s] = __shfl_sync(0xffffffffu, zy[s].y, (lane + 31) & 31);
-    tn[s] = __shfl_sync(0xffffffffu, zy[s].x, (lane + 1) & 31);
+  __device__ __forceinline__ bool valid(int s) const { return kWrap || lane + 32 * s < gw; }
+  // group of slot s (an idle lane reads the warp's last one)
+  __device__ __forceinline__ int group(int s) const {
+    if constexpr (kWrap) return lane + 32 * s;
+    const int q = lane + 32 * s;
+    return g0 - lane + (q < gw ? q : gw - 1);
   }
+};
+
+// The packed pairs v moved by one entry: w = the entries m - 1 or, with right,
+// m + 1 of each pair's entries m. The outermost groups a warp's lanes cannot
+// reach by shuffles (rows that do not wrap within the warp) take edge(m).
+template <int NS, int WPR, int NXT, typename F>
+__device__ __forceinline__ void shifted(float2 (&w)[NS], const float2 (&v)[NS], bool right,
+                                        const Row<NS, WPR, NXT>& r, F&& edge) {
+  const int src = (right ? r.lane + 1 : r.lane + 31) & 31;
+  float t[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) t[s] = __shfl_sync(0xffffffffu, right ? v[s].x : v[s].y, src);
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
-    const float z0 = lane == 0 ? tp[(s + NS - 1) % NS] : tp[s];
-    const float z3 = lane == 31 ? tn[(s + 1) % NS] : tn[s];
-    v[s].x = prolong_add(v[s].x, prolong_axis(zy[s].x, z0));
-    v[s].y = prolong_add(v[s].y, prolong_axis(zy[s].x, zy[s].y));
-    v[s].z = prolong_add(v[s].z, prolong_axis(zy[s].y, zy[s].x));
-    v[s].w = prolong_add(v[s].w, prolong_axis(zy[s].y, z3));
+    float o = t[s];
+    if constexpr (Row<NS, WPR, NXT>::kWrap) {
+      static_assert(NS <= 2, "the adjacent slot on either side is the other one");
+      if (NS == 2 && r.lane == (right ? 31 : 0)) o = t[NS - 1 - s];
+    } else {
+      const int q = r.lane + 32 * s;
+      if (right ? (r.lane == 31 || q == r.gw - 1) : r.lane == 0) {
+        const int g = r.group(s), half = r.nx >> 1;
+        int m = right ? 2 * g + 2 : 2 * g - 1;
+        m = m < 0 ? m + half : (m >= half ? m - half : m);
+        o = edge(m);
+      }
+    }
+    w[s] = right ? make_float2(v[s].y, o) : make_float2(o, v[s].x);
   }
 }
 
-// Grid: (ny / TY, z-chunks). Block: (TY + 2) warps; warp w owns row
-// y0 - 1 + w (w = 0 and w = TY + 1 are the halo rows: red cells only).
-// Shared memory: XS[R][TY + 4][nx] (old x, rows y0-2 .. y0+TY+1),
-// BS[R][TY + 2][nx] (b, rows y0-1 .. y0+TY), RS[2][TY + 2][nx / 2] (the red
-// cells of each row after the red update, two per 4-cell group), R mbarriers.
+// Per entry of the packed pairs v the sum of its two x-neighbours among the
+// entries of the same packed row: (m - 1, m) or, with right, (m, m + 1). `row`
+// is the published copy of that row.
+template <int NS, int WPR, int NXT>
+__device__ __forceinline__ void nbr_sums(float2 (&n)[NS], const float2 (&v)[NS], const float* row, bool right,
+                                         const Row<NS, WPR, NXT>& r) {
+  shifted<NS, WPR, NXT>(n, v, right, r, [&](int m) { return row[m]; });
+#pragma unroll
+  for (int s = 0; s < NS; ++s) n[s] = add2(v[s], n[s]);
+}
+
+// The correction of a packed row: v += (P xc) at its black cells (Sec. III.E,
+// cell-centred trilinear prolongation) in the order every prolongation kernel
+// uses: z between the row's parent coarse plane cp and the other plane co, then
+// y between the parent coarse row cr and its neighbour nr on the row's side
+// (coarse rows of nx / 2 floats), then x towards coarse cell m + 1 (right: the
+// black cell is the odd one of its pair) or m - 1.
+template <int NS, int WPR, int NXT>
+__device__ __forceinline__ void add_correction(float2 (&v)[NS], const float* cp, const float* co, int cr, int nr,
+                                               bool right, const Row<NS, WPR, NXT>& r) {
+  const int nxc = r.nx >> 1;
+  const float *pp = cp + cr * nxc, *op = co + cr * nxc, *pn = cp + nr * nxc, *on = co + nr * nxc;
+  float2 zy[NS], f[NS];  // the pair after z and y (16 times its value), and its neighbours
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const int o = 2 * r.group(s);
+    const float2 a = *reinterpret_cast<const float2*>(pp + o), b = *reinterpret_cast<const float2*>(op + o);
+    const float2 c = *reinterpret_cast<const float2*>(pn + o), d = *reinterpret_cast<const float2*>(on + o);
+    zy[s] = prolong_axis2(prolong_axis2(a, b), prolong_axis2(c, d));
+  }
+  shifted<NS, WPR, NXT>(f, zy, right, r, [&](int m) {
+    return prolong_axis(prolong_axis(pp[m], op[m]), prolong_axis(pn[m], on[m]));
+  });
+#pragma unroll
+  for (int s = 0; s < NS; ++s) v[s] = prolong_add2(v[s], prolong_axis2(zy[s], f[s]));
+}
+
+// What a sweep reads as the old x.
+enum SweepIn {
+  IN_FULL = 0,      // a full field
+  IN_FULL_PRO = 1,  // a full field plus the prolongation of a coarse field
+  IN_PACKED_PRO = 2 // a packed field of black cells plus the prolongation of a coarse field
+};
+
+// Shared memory (floats): x ring, b ring, two published planes of corrected
+// black rows y0-2 .. y0+TY+1, two planes of red rows y0-1 .. y0+TY, coarse ring.
+__host__ __device__ constexpr size_t sweep_rows_floats(int nx, int in) {
+  return (size_t)kSweepRing * (kRowsTY + 4) * (in == IN_PACKED_PRO ? nx / 2 : nx) +
+         (size_t)kSweepRing * (kRowsTY + 2) * nx + (size_t)(kRowsTY + 4) * nx + (size_t)(kRowsTY + 2) * nx +
+         (in == IN_FULL ? 0 : (size_t)kCoarseRing * (kRowsTY / 2 + 4) * (nx / 2));
+}
+
+// Grid: (ny / TY, z-chunks). Block: (TY + 2) rows of WPR warps; row w is
+// y0 - 1 + w (w = 0 and w = TY + 1 are the halo rows: red cells only; they
+// also publish the outer rows y0 - 2 and y0 + TY + 1).
 //
 // March order: chunk c covers planes [k0, k1) and visits planes k0-2 .. k1+1
 // upwards when c is even and k1+1 .. k0-2 downwards when c is odd, so that
@@ -181,55 +356,49 @@ __device__ __forceinline__ void add_correction(float4 (&v)[NS], const float* cp,
 // time and the halo planes they share come from L2. The Gauss-Seidel result
 // does not depend on the order in which the cells of one colour are updated,
 // so both directions give the same sweep. March index i = 0 .. zc + 3 names
-// plane mp(i); step i updates the red cells of mp(i) and the black cells of
-// mp(i - 1) (when that plane is in the chunk) and stores mp(i - 1).
+// plane mp(i). Step i reads stage i (x of plane i + 1, b of plane i), publishes
+// the black cells of plane i + 1, updates the red cells of plane i and the
+// black cells of plane i - 1 (when that plane is in the chunk) and stores
+// plane i - 1.
 //
-// PRO: the sweep that follows the coarse-grid correction, with the
-// correction fused: x (xin) arrives uncorrected, and every x value the sweep
-// reads is x + P xc, P the cell-centred trilinear prolongation of the coarse
-// field xc, in the arithmetic of the stand-alone prolongation kernel. The
+// With the prolongation fused the x values are corrected as they are read. The
 // coarse planes arrive by TMA into a ring of kCoarseRing slots of TY / 2 + 4
 // coarse rows (the parents of the tile's rows and their neighbours), riding
-// on the barriers of the fine planes. Fine planes 2K - 1 and 2K share the
-// coarse pair {K - 1, K}, so in march order every second fine plane brings a
-// new coarse plane (coarse march plane j = i / 2 + 2 first serves the
-// correction of fine march plane i + 1, i even). Each thread corrects its own
-// row of plane i + 1 in registers when it loads it and writes it back for the
-// y-neighbour reads of step i + 1; the halo warps also correct the two outer
-// x rows. Chunks hold an even number of planes so that the pairing is the same
-// in both march directions.
-template <int NS, bool PRO>
-__global__ void __launch_bounds__((kRowsTY + 2) * 32, 2)
-    k_rbgs_rows(const __grid_constant__ CUtensorMap mx_tile, const __grid_constant__ CUtensorMap mx_pair,
-                const __grid_constant__ CUtensorMap mb_tile, const __grid_constant__ CUtensorMap mb_one,
-                const __grid_constant__ CUtensorMap mc_half, const __grid_constant__ CUtensorMap mc_pair,
-                float* __restrict__ xout, const double* __restrict__ bshift, int ny, int nz, int zc, float inv,
-                float off, double* __restrict__ part, int* __restrict__ err, unsigned wait_limit) {
-  constexpr int TY = kRowsTY, R = kRowsRing, NX = 128 * NS;
-  constexpr int XROWS = TY + 4, BROWS = TY + 2, RROWS = TY + 2, RW = NX / 2;
-  constexpr int NXC = NX / 2, CROWS = TY / 2 + 4;
-  constexpr unsigned XBYTES = XROWS * NX * 4, BBYTES = BROWS * NX * 4, CBYTES = CROWS * NXC * 4;
+// on the stages. Fine planes 2K - 1 and 2K share the coarse pair {K - 1, K}, so
+// every second stage brings a new coarse plane (coarse march plane j = i / 2 + 2
+// first serves the correction of fine march plane i + 1, i even). Chunks hold
+// an even number of planes so that the pairing is the same in both march
+// directions.
+template <int NS, int WPR, int NXT, int IN>
+__global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
+    k_rbgs_rows(const __grid_constant__ RowMaps mx, const __grid_constant__ RowMaps mb,
+                const __grid_constant__ RowMaps mc, float* __restrict__ xout, const double* __restrict__ bshift,
+                int nx_, int ny, int nz, int zc, float inv, float off, double* __restrict__ part,
+                int* __restrict__ err, unsigned wait_limit) {
+  constexpr int TY = kRowsTY, R = kSweepRing;
+  constexpr bool PRO = IN != IN_FULL, PIN = IN == IN_PACKED_PRO;
+  constexpr int XROWS = TY + 4, BROWS = TY + 2, CROWS = TY / 2 + 4;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), w = warp / WPR;
+  const Row<NS, WPR, NXT> row(nx_, warp % WPR);
+  const int nx = row.nx, nxp = nx >> 1, nxr = PIN ? nxp : nx;  // nxr: row length of the x ring
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   float* XS = reinterpret_cast<float*>(sm_raw);
-  float* BS = XS + R * XROWS * NX;
-  float* RS = BS + R * BROWS * NX;
-  float* CS = RS + 2 * RROWS * RW;
-  unsigned long long* bars = reinterpret_cast<unsigned long long*>(CS + (PRO ? kCoarseRing * CROWS * NXC : 0));
+  float* BS = XS + R * XROWS * nxr;
+  float* CP = BS + R * BROWS * nx;
+  float* RS = CP + 2 * XROWS * nxp;
+  float* CS = RS + 2 * BROWS * nxp;
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(CS + (PRO ? kCoarseRing * CROWS * nxp : 0));
 
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int y0 = blockIdx.x * TY;
   const int k0 = blockIdx.y * zc, k1 = min(k0 + zc, nz);
   const bool down = blockIdx.y & 1;
-  const size_t plane = (size_t)NX * ny;
-  const float sh = bshift ? (float)(*bshift) : 0.f;
+  const float2 msh = dup2(bshift ? -(float)(*bshift) : -0.f), off2 = dup2(off), inv2 = dup2(inv);
   const bool interior = w >= 1 && w <= TY;
-  // this warp's row: parity of y (ny is even, so the wrap keeps it)
-  const int ypar = (y0 - 1 + w) & 1;
   const int last = k1 - k0 + 3;  // march index of the last plane
   auto mp = [&](int i) { return down ? k1 + 1 - i : k0 - 2 + i; };
-  // coarse march plane j and the one a fine plane's copy brings (-1: none)
-  auto cmp = [&](int j) { return down ? (k1 >> 1) + 1 - j : (k0 >> 1) - 2 + j; };
-  auto cj_of = [&](int i) { return i <= 3 ? i : ((i & 1) ? (i + 3) >> 1 : -1); };
+  auto cmp = [&](int j) { return down ? (k1 >> 1) + 1 - j : (k0 >> 1) - 2 + j; };  // coarse march plane j
+  // parity of this warp's row in march plane 1 (ny is even, so the wrap keeps it)
+  const bool a1 = (y0 - 1 + w + mp(1)) & 1;
   // coarse rows of this warp's own row: its parent and the parent's neighbour
   const int cr = ((w + 1) >> 1) + 1, nr = (w & 1) ? cr - 1 : cr + 1;
 
@@ -237,439 +406,412 @@ __global__ void __launch_bounds__((kRowsTY + 2) * 32, 2)
     for (int s = 0; s < R; ++s) mbar_init(smem_u32(bars + s), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  __syncthreads();
+  cta_sync();
 
-  // copies of march plane i (x rows y0-2 .. y0+TY+1, b rows y0-1 .. y0+TY) into its slot
-  // box start rows, wrapped once (march planes lie in [-2, nz + 1], coarse
-  // march planes in [-2, nz / 2 + 1]: one compare wraps them)
-  const int ya = wrapm(y0 - 2, ny), yb = wrapm(y0 + TY, ny), yh = wrapm(y0 - 1, ny);
-  const int nyc = ny >> 1, nzc = nz >> 1, yc = y0 >> 1;
-  const int yca = wrapm(yc - 2, nyc), ycb = wrapm(yc + TY / 2, nyc);
-  auto issue = [&](int i) {
-    const int s = i % R;
+  // Copies of stage i = -1 .. last - 1 (slot (i + 1) % R): x of march plane
+  // i + 1 (rows y0-2 .. y0+TY+1), for i >= 1 b of march plane i (rows y0-1 ..
+  // y0+TY), with PRO the coarse march planes 0 and 1 (i = -1) or i / 2 + 2 (even
+  // i >= 0; coarse rows y0/2 - 2 .. y0/2 + TY/2 + 1). Planes lie in [-2, nz + 1],
+  // coarse ones in [-2, nz / 2 + 1]: one compare wraps them.
+  auto wrapz = [](int z, int n) { return z < 0 ? z + n : (z >= n ? z - n : z); };
+  auto issue_coarse = [&](int j, unsigned bar, unsigned lead) {
+    load_rows<TY / 2, 2>(CS + (j % kCoarseRing) * CROWS * nxp, nxp, mc, y0 >> 1, ny >> 1, wrapz(cmp(j), nz >> 1), bar,
+                         lead);
+  };
+  auto issue = [&](int i, unsigned lead) {
+    const unsigned xbytes = XROWS * nxr * 4, bbytes = BROWS * nx * 4, cbytes = CROWS * nxp * 4;
+    const int s = (i + 1) % R;
     const unsigned bar = smem_u32(bars + s);
-    int z = mp(i);
-    z += z < 0 ? nz : (z >= nz ? -nz : 0);
-    float* xs = XS + s * XROWS * NX;
-    float* bs = BS + s * BROWS * NX;
-    const int j = PRO ? cj_of(i) : -1;
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    mbar_expect_tx(bar, XBYTES + BBYTES + (j >= 0 ? CBYTES : 0u));
-    tma_load3(smem_u32(xs), &mx_pair, 0, ya, z, bar);
-    tma_load3(smem_u32(xs + 2 * NX), &mx_tile, 0, y0, z, bar);
-    tma_load3(smem_u32(xs + (TY + 2) * NX), &mx_pair, 0, yb, z, bar);
-    tma_load3(smem_u32(bs), &mb_one, 0, yh, z, bar);
-    tma_load3(smem_u32(bs + NX), &mb_tile, 0, y0, z, bar);
-    tma_load3(smem_u32(bs + (TY + 1) * NX), &mb_one, 0, yb, z, bar);
-    if (PRO && j >= 0) {
-      // coarse rows y0/2 - 2 .. y0/2 + TY/2 + 1 of coarse plane cmp(j)
-      float* cs = CS + (j % kCoarseRing) * CROWS * NXC;
-      int kc = cmp(j);
-      kc += kc < 0 ? nzc : (kc >= nzc ? -nzc : 0);
-      tma_load3(smem_u32(cs), &mc_pair, 0, yca, kc, bar);
-      tma_load3(smem_u32(cs + 2 * NXC), &mc_half, 0, yc, kc, bar);
-      tma_load3(smem_u32(cs + (TY / 2 + 2) * NXC), &mc_pair, 0, ycb, kc, bar);
+    const bool even = i >= 0 && !(i & 1);
+    mbar_expect_tx(bar, xbytes + (i >= 1 ? bbytes : 0u) + (PRO ? (i < 0 ? 2u : (even ? 1u : 0u)) * cbytes : 0u), lead);
+    load_rows<TY, 2>(XS + s * XROWS * nxr, nxr, mx, y0, ny, wrapz(mp(i + 1), nz), bar, lead);
+    if (i >= 1) load_rows<TY, 1>(BS + s * BROWS * nx, nx, mb, y0, ny, wrapz(mp(i), nz), bar, lead);
+    if constexpr (PRO) {
+      if (i < 0) {
+        issue_coarse(0, bar, lead);
+        issue_coarse(1, bar, lead);
+      } else if (even) {
+        issue_coarse((i >> 1) + 2, bar, lead);
+      }
     }
   };
-  // thread 0 alone polls the barriers; the CTA barrier that follows every
-  // wait publishes the landed plane to the other threads
-  auto wait_plane = [&](int i, unsigned limit) {
-    return mbar_wait(smem_u32(bars + (i % R)), (unsigned)((i / R) & 1), limit);
+  auto wait_stage = [&](int i, unsigned limit) {
+    return mbar_wait(smem_u32(bars + (i + 1) % R), (unsigned)(((i + 1) / R) & 1), limit);
   };
-  auto xrow = [&](int i, int r) { return reinterpret_cast<const float4*>(XS + (i % R) * XROWS * NX + r * NX); };
-  auto brow = [&](int i, int r) { return reinterpret_cast<const float4*>(BS + (i % R) * BROWS * NX + r * NX); };
-  auto rrow = [&](int i, int r) { return reinterpret_cast<float2*>(RS + (i & 1) * RROWS * RW + r * RW); };
-  auto xroww = [&](int i, int r) { return reinterpret_cast<float4*>(XS + (i % R) * XROWS * NX + r * NX); };
-  auto cslot = [&](int j) -> const float* { return CS + (j % kCoarseRing) * CROWS * NXC; };
-  // PRO, halo warps: correct x row 0 (warp 0) or TY + 3 (warp TY + 1) of
-  // march plane i in shared memory; cp / co: parent / other coarse plane
-  const bool outer = w == 0 || w == TY + 1;
-  auto fix_outer = [&](int i, const float* cp, const float* co) {
-    const bool top = w == 0;
-    float4 v[NS];
-    float4* row = xroww(i, top ? 0 : TY + 3) + lane;
+  // rows of the published planes (by the march plane's parity), a coarse plane by its ring slot
+  auto cprow = [&](int par, int r) { return CP + (par * XROWS + r) * nxp; };
+  auto rsrow = [&](int par, int r) { return RS + (par * BROWS + r) * nxp; };
+  auto cslot = [&](int s) -> const float* { return CS + s * CROWS * nxp; };
+  // the old black values of row r (0 .. TY + 3) in ring slot `slot`, uncorrected; right: its black cells are the odd ones
+  auto load_black = [&](float2 (&v)[NS], int slot, int r, bool right) {
+    const float* p = XS + (slot * XROWS + r) * nxr;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) v[s] = row[32 * s];
-    add_correction<NS>(v, cp, co, top ? 1 : CROWS - 2, top ? 0 : CROWS - 1, lane);
+    for (int s = 0; s < NS; ++s) {
+      if constexpr (PIN) {
+        v[s] = *reinterpret_cast<const float2*>(p + 2 * row.group(s));
+      } else {
+        const float4 q = *reinterpret_cast<const float4*>(p + 4 * row.group(s));
+        v[s] = right ? make_float2(q.y, q.w) : make_float2(q.x, q.z);
+      }
+    }
+  };
+  auto put_row = [&](float* p, const float2 (&v)[NS]) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s) row[32 * s] = v[s];
+    for (int s = 0; s < NS; ++s)
+      if (row.valid(s)) *reinterpret_cast<float2*>(p + 2 * row.group(s)) = v[s];
+  };
+  auto get_row = [&](float2 (&v)[NS], const float* p) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) v[s] = *reinterpret_cast<const float2*>(p + 2 * row.group(s));
+  };
+  // the plane in ring slot `slot` (its march index's parity par; right: this
+  // row's black cells are the odd ones) into v (this warp's row) and into the
+  // published rows; jp / jo: the ring slots of its parent and other coarse planes
+  auto take_plane = [&](float2 (&v)[NS], bool right, int slot, int par, int jp, int jo) {
+    load_black(v, slot, w + 1, right);
+    if constexpr (PRO) add_correction<NS, WPR, NXT>(v, cslot(jp), cslot(jo), cr, nr, right, row);
+    put_row(cprow(par, w + 1), v);
+    if (!interior) {  // the outer row next to this halo row
+      const bool top = w == 0;
+      float2 o[NS];
+      load_black(o, slot, top ? 0 : TY + 3, !right);
+      if constexpr (PRO)
+        add_correction<NS, WPR, NXT>(o, cslot(jp), cslot(jo), top ? 1 : CROWS - 2, top ? 0 : CROWS - 1, !right, row);
+      put_row(cprow(par, top ? 0 : TY + 3), o);
+    }
   };
 
   bool ok = true;
-  if (tid == 0) {
-    // PRO: plane 3's copy brings coarse plane 3 into the slot of coarse
-    // plane 0, which the prologue still reads: it is issued after it
-    for (int i = 0; i < (PRO ? 3 : R) && i <= last; ++i) issue(i);
-    ok = wait_plane(0, wait_limit) && wait_plane(1, wait_limit) && wait_plane(2, wait_limit);
-  }
-  int issued = PRO ? 2 : min(R - 1, last);
-  ok = !__syncthreads_or(!ok);
-  // march planes up to `done` have landed (the same value in every thread:
-  // it only advances after a barrier that every thread passed)
-  int done = ok ? 2 : -1;
-
-  float4 A[NS], B[NS], C[NS], D[NS], BX[NS], BY[NS];
-  if (ok) {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      B[s] = xrow(0, w + 1)[lane + 32 * s];
-      C[s] = xrow(1, w + 1)[lane + 32 * s];
-    }
-    if constexpr (PRO) {
-      // fine march planes 0 and 1 have the parent coarse plane 1; the other
-      // plane is 0 for plane 0 and 2 for plane 1
-      add_correction<NS>(B, cslot(1), cslot(0), cr, nr, lane);
-      add_correction<NS>(C, cslot(1), cslot(2), cr, nr, lane);
-#pragma unroll
-      for (int s = 0; s < NS; ++s) xroww(1, w + 1)[lane + 32 * s] = C[s];
-      if (outer) fix_outer(1, cslot(1), cslot(2));
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    }
-  }
-  __syncthreads();  // step 1 refills plane 0's slot
-  if (PRO && ok) {
-    if (tid == 0) issue(3);
-    issued = 3;
-  }
   float acc = 0.f, comp = 0.f;  // Kahan sum of the new x (tile rows)
+  // where the black cells' step stores this row of plane mp(2), mp(3), ...
+  const ptrdiff_t plane = (ptrdiff_t)nx * ny;
+  float* dst = xout + (ptrdiff_t)mp(2) * plane + (ptrdiff_t)(y0 - 1 + w) * nx;
+  const ptrdiff_t dstep = down ? -plane : plane;
+  // a warp's march, compiled for each parity of its row in march plane 1
+  auto march = [&](auto first_parity) {
+    constexpr bool A1 = decltype(first_parity)::value;
+    // old black cells of three planes, new red cells of three, b of the black cells of two
+    float2 C0[NS], C1[NS], C2[NS], R0[NS], R1[NS], R2[NS], B0[NS], B1[NS];
+    ok = !cta_sync_or(false);  // stages -1, 0 and 1 have landed
+    if (!ok) return;
+    // march planes 0 and 1 have the parent coarse plane 1; the other plane is
+    // 0 for plane 0 and 2 for plane 1
+    take_plane(C0, A1, 0, 0, 1, 0);
+    take_plane(C1, !A1, 1, 1, 1, 2);
+    cta_sync();  // the slots of stages -1 and 0 are free
 
-  // Step i: pm2 .. pp1 are this thread's row of march planes i - 2 .. i + 1,
-  // bm1 / b0 its b of march planes i - 1 / i. Planes i and i + 1 have landed.
-  auto step = [&](float4 (&pm2)[NS], float4 (&pm1)[NS], float4 (&p0)[NS], float4 (&pp1)[NS], float4 (&bm1)[NS],
-                  float4 (&b0)[NS], int i, bool odd) -> bool {
-    if (i > last - 1 || !ok) return false;
-    // plane i + 3 takes the slot of plane i - 1, last read before the barrier
-    // that ended step i - 1 (PRO, even i: its copy brings coarse plane
-    // i / 2 + 3 into the slot of coarse plane i / 2, last read in step i - 1)
-    if (tid == 0 && i + 3 <= last) issue(i + 3);
-    if (i + 3 <= last) issued = i + 3;
-    const int z = mp(i);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) pp1[s] = xrow(i + 1, w + 1)[lane + 32 * s];
-    if constexpr (PRO) {
-      // correct plane i + 1: odd i keeps the coarse pair of step i - 1, whose
+    // Step i: cm, c0, cp = old black cells of march planes i - 1, i, i + 1 (cp is read here); rm2, rm1, r0 = new red
+    // cells of planes i - 2, i - 1, i (r0 is formed here); bm1 / b0 = b of the black cells of planes i - 1 / i.
+    auto step = [&](float2 (&cm)[NS], float2 (&c0)[NS], float2 (&cp)[NS], float2 (&rm2)[NS], float2 (&rm1)[NS],
+                    float2 (&r0)[NS], float2 (&bm1)[NS], float2 (&b0)[NS], int i, auto phase) {
+      // i = 1 + phase (mod 6): ring slots and parities are constants
+      constexpr int PH = decltype(phase)::value, P0 = (PH + 1) & 1, P1 = PH & 1, S1 = (PH + 2) % R;
+      constexpr bool a = A1 != (bool)(PH & 1);  // plane i: red cells at 2 m + a
+      static_assert(R == 3 && kCoarseRing == 3, "the unrolling by 6 fixes the slots");
+      // coarse planes of plane i + 1: odd i keeps the pair of step i - 1, whose
       // newer plane is the parent; even i brings coarse plane i / 2 + 2 (the
       // other) and the parent is the plane before it
-      const int jp = odd ? ((i - 1) >> 1) + 2 : (i >> 1) + 1;
-      const int jo = odd ? jp - 1 : jp + 1;
-      add_correction<NS>(pp1, cslot(jp), cslot(jo), cr, nr, lane);
-    }
+      constexpr int JP = P0 ? (PH / 2 + 2) % 3 : ((PH + 1) / 2 + 1) % 3, JO = (JP + (P0 ? 2 : 1)) % 3;
+      take_plane(cp, a, S1, P1, JP, JO);
+      float2 br[NS], n[NS], u[NS], d[NS];
+      const float* bp = BS + (S1 * BROWS + w) * nx;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      float4 t = brow(i, w)[lane + 32 * s];
-      t.x -= sh, t.y -= sh, t.z -= sh, t.w -= sh;
-      b0[s] = t;
-    }
-    const int a = (ypar + z) & 1;
-    // red cells of plane mp(i) from the old rows y - 1, y + 1 of that plane
-    rb_row<NS, false>(p0, xrow(i, w) + lane, xrow(i, w + 2) + lane, pm1, pp1, b0, a, off, inv, lane);
-    float2* rr = rrow(i, w);
+      for (int s = 0; s < NS; ++s) {
+        const float4 t = *reinterpret_cast<const float4*>(bp + 4 * row.group(s));
+        br[s] = add2(a ? make_float2(t.y, t.w) : make_float2(t.x, t.z), msh);
+        b0[s] = add2(a ? make_float2(t.x, t.z) : make_float2(t.y, t.w), msh);
+      }
+      // red cells of plane i from the old black cells around them
+      nbr_sums<NS, WPR, NXT>(n, c0, cprow(P0, w + 1), a, row);
+      get_row(u, cprow(P0, w));
+      get_row(d, cprow(P0, w + 2));
 #pragma unroll
-    for (int s = 0; s < NS; ++s)
-      rr[lane + 32 * s] = a == 0 ? make_float2(p0[s].x, p0[s].z) : make_float2(p0[s].y, p0[s].w);
-    if (interior && i >= 3) {
-      // black cells of plane mp(i - 1) from the red cells of its rows y - 1, y + 1
-      rb_row<NS, true>(pm1, rrow(i - 1, w - 1) + lane, rrow(i - 1, w + 1) + lane, pm2, p0, bm1, a, off, inv,
-                       lane);
-      float4* dst = reinterpret_cast<float4*>(xout + (size_t)mp(i - 1) * plane + (size_t)(y0 - 1 + w) * NX);
-#pragma unroll
-      for (int s = 0; s < NS; ++s) dst[lane + 32 * s] = pm1[s];
-      if (part) {
+      for (int s = 0; s < NS; ++s)
+        r0[s] = mul2(fma2(off2, add2(add2(n[s], add2(u[s], d[s])), add2(cm[s], cp[s])), br[s]), inv2);
+      put_row(rsrow(P0, w), r0);
+      if (interior && i >= 3) {
+        // black cells of plane i - 1 (there at 2 m + a) from the new red cells around them
+        float2 k[NS];
+        nbr_sums<NS, WPR, NXT>(n, rm1, rsrow(P1, w), a, row);
+        get_row(u, rsrow(P1, w - 1));
+        get_row(d, rsrow(P1, w + 1));
         float t = 0.f;
 #pragma unroll
-        for (int s = 0; s < NS; ++s) t += (pm1[s].x + pm1[s].y) + (pm1[s].z + pm1[s].w);
-        const float yk = t - comp, tk = acc + yk;
-        comp = (tk - acc) - yk;
-        acc = tk;
+        for (int s = 0; s < NS; ++s) {
+          k[s] = mul2(fma2(off2, add2(add2(n[s], add2(u[s], d[s])), add2(rm2[s], r0[s])), bm1[s]), inv2);
+          if (row.valid(s)) {
+            *reinterpret_cast<float4*>(dst + 4 * row.group(s)) =
+                a ? make_float4(rm1[s].x, k[s].x, rm1[s].y, k[s].y) : make_float4(k[s].x, rm1[s].x, k[s].y, rm1[s].y);
+            t += (rm1[s].x + rm1[s].y) + (k[s].x + k[s].y);
+          }
+        }
+        dst += dstep;
+        if (part) {
+          const float yk = t - comp, tk = acc + yk;
+          comp = (tk - acc) - yk;
+          acc = tk;
+        }
       }
+      if constexpr (PH == 5)
+        ok = !cta_sync_or(false);
+      else
+        cta_sync();
+    };
+#define IBRD_STEP(c0, c1, c2, r0, r1, r2, b0, b1, ph) \
+  if (i + ph >= last) return;                         \
+  step(c0, c1, c2, r0, r1, r2, b0, b1, i + ph, std::integral_constant<int, ph>{});
+    for (int i = 1; ok; i += 6) {
+      IBRD_STEP(C0, C1, C2, R0, R1, R2, B0, B1, 0)
+      IBRD_STEP(C1, C2, C0, R1, R2, R0, B1, B0, 1)
+      IBRD_STEP(C2, C0, C1, R2, R0, R1, B0, B1, 2)
+      IBRD_STEP(C0, C1, C2, R0, R1, R2, B1, B0, 3)
+      IBRD_STEP(C1, C2, C0, R1, R2, R0, B0, B1, 4)
+      IBRD_STEP(C2, C0, C1, R2, R0, R1, B1, B0, 5)
     }
-    if constexpr (PRO) {
-      // the corrected rows of plane i + 1 for the y-neighbour reads of step
-      // i + 1 (nothing reads that plane's rows in this step); the outer rows
-      // from the halo warps; then the writers' proxy fence, as TMA later
-      // refills the slot
-      const int jp = odd ? ((i - 1) >> 1) + 2 : (i >> 1) + 1;
-      const int jo = odd ? jp - 1 : jp + 1;
-#pragma unroll
-      for (int s = 0; s < NS; ++s) xroww(i + 1, w + 1)[lane + 32 * s] = pp1[s];
-      if (outer) fix_outer(i + 1, cslot(jp), cslot(jo));
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    }
-    bool good = true;
-    if (tid == 0 && i + 2 <= last) good = wait_plane(i + 2, wait_limit);
-    ok = !__syncthreads_or(!good);
-    if (ok) done = i + 2;
-    return ok;
+#undef IBRD_STEP
   };
-  for (int i = 1; i < last; i += 4) {
-    if (!step(A, B, C, D, BX, BY, i, true)) break;
-    if (!step(B, C, D, A, BY, BX, i + 1, false)) break;
-    if (!step(C, D, A, B, BX, BY, i + 2, true)) break;
-    if (!step(D, A, B, C, BY, BX, i + 3, false)) break;
-  }
-  if (!ok) {
-    // a plane wait gave up: drain the copies still in flight, report, stop
-    if (tid == 0) {
-      for (int i = done + 1; i <= issued; ++i) wait_plane(i, kDrainLimit);
-      atomicOr(err, 1);
-    }
-    __syncthreads();
-    return;
+  if (w == TY + 2) {
+    // stage i + 2 takes the slot of stage i - 1, last read before the barrier
+    // that ended step i - 1, as was the coarse plane it replaces
+    feed_stages(last, 1, 2, issue, wait_stage, wait_limit, err);
+  } else if (a1) {
+    march(std::true_type{});
+  } else {
+    march(std::false_type{});
   }
   if (part) {
     double v = (double)acc;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     double* ws = reinterpret_cast<double*>(RS);  // no step reads RS after the last barrier
-    if (lane == 0) ws[w] = v;
-    __syncthreads();
+    if (row.lane == 0 && w < TY + 2) ws[tid >> 5] = v;
+    cta_sync();
     if (tid == 0) {
       double sum = 0.0;
-      for (int i = 0; i < TY + 2; ++i) sum += ws[i];
+      for (int i = 0; i < (TY + 2) * WPR; ++i) sum += ws[i];
       part[blockIdx.x + gridDim.x * blockIdx.y] = sum;
     }
   }
 }
 
-// First red-black sweep from x = 0 fused with the residual restriction, for
-// the same levels as the sweep above: x = one sweep of A x = b - shift from
-// zero (red cells (b - shift) / diag, black cells from their red neighbours,
-// the arithmetic of k_rb_zero_f32v) and bc = mean over the 8 children of
-// b - shift - A x, in one pass over b (HBM: read b, write x and bc).
-//
-// Layout as in k_rbgs_rows: warp w owns row y0 - 1 + w of every plane; a ring
-// of R b-planes (rows y0-2 .. y0+TY+1) arrives by TMA; the march order
-// alternates between even and odd z-chunks. Step i forms x on march plane i
-// (all warps, rows y0-1 .. y0+TY: the edge rows' residuals need them) from b
-// of planes i-1 .. i+1, and the residual of march plane i-1 (tile warps) from
-// x of planes i-2 .. i; x rows go through shared memory (XB, double-buffered)
-// for the y-neighbours. Restriction: the two cells of a coarse cell along x
-// sit in one lane, the two planes along z are summed in registers over two
-// steps, and the two rows along y belong to warps w (even y) and w + 1 (odd
-// y): when a plane pair is complete the odd row's warp leaves its sums in
-// shared memory (RY) and the even row's warp adds them one step later (after
-// the step's barrier) and writes the coarse row. Chunks start on even planes
-// and hold an even number of them, so plane pairs never straddle chunks.
-template <int NS>
-__global__ void __launch_bounds__((kRowsTY + 2) * 32, 2)
-    k_zr_rows(const __grid_constant__ CUtensorMap mb_tile, const __grid_constant__ CUtensorMap mb_pair,
-              float* __restrict__ xout, float* __restrict__ bc, const double* __restrict__ bshift, int ny, int nz,
-              int zc, float inv, float off, float diag, int* __restrict__ err, unsigned wait_limit) {
-  constexpr int TY = kRowsTY, R = kRowsRing, NX = 128 * NS, NXC = NX / 2;
-  constexpr int XROWS = TY + 4, XBROWS = TY + 2;
-  constexpr unsigned BBYTES = XROWS * NX * 4;
-  extern __shared__ __align__(1024) unsigned char sm_raw[];
-  float* BSM = reinterpret_cast<float*>(sm_raw);        // R b planes, rows y0-2 .. y0+TY+1
-  float* XB = BSM + R * XROWS * NX;                      // 2 x planes, rows y0-1 .. y0+TY
-  float2* RY = reinterpret_cast<float2*>(XB + 2 * XBROWS * NX);  // TY/2 odd-row pair sums
-  unsigned long long* bars = reinterpret_cast<unsigned long long*>(RY + (TY / 2) * NXC / 2);
+// Shared memory (floats): b ring (rows y0-2 .. y0+TY+1), two published planes
+// of red rows y0-2 .. y0+TY+1, two planes of black rows y0-1 .. y0+TY, the odd
+// rows' restriction sums.
+__host__ __device__ constexpr size_t zero_rows_floats(int nx) {
+  return (size_t)kZeroRing * (kRowsTY + 4) * nx + (size_t)(kRowsTY + 4) * nx + (size_t)(kRowsTY + 2) * nx +
+         (size_t)(kRowsTY / 2) * (nx / 2);
+}
 
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+// First red-black sweep from x = 0 fused with the residual restriction: red
+// cells (b - shift) / diag, black cells from their red neighbours (the
+// arithmetic of k_rb_zero_f32v), bc = mean over the 8 children of
+// b - shift - A x, in one pass over b (HBM: read b, write the packed black
+// cells and bc; the red cells are b / diag and enter no later sweep). The
+// residual is off times the neighbour sum in the red cells and zero in the
+// black ones.
+//
+// Layout as in k_rbgs_rows. Step i reads stage i (b of march plane i + 1),
+// publishes its red cells, forms the black cells of plane i (all rows: the edge
+// rows' neighbours need them) and the restriction sums of plane i - 1. The two
+// planes of a coarse cell are summed in registers over two steps, its two rows
+// belong to warps w (even y) and the next (odd y): when a plane pair is
+// complete the odd row leaves its sums in shared memory (RY) and the even row
+// adds them one step later (after the step's barrier) and writes the coarse
+// row. Chunks start on even planes and hold an even number of them, so plane
+// pairs never straddle chunks.
+template <int NS, int WPR, int NXT>
+__global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
+    k_zr_rows(const __grid_constant__ RowMaps mb, float* __restrict__ xb, float* __restrict__ bc,
+              const double* __restrict__ bshift, int nx_, int ny, int nz, int zc, float inv, float off,
+              int* __restrict__ err, unsigned wait_limit) {
+  constexpr int TY = kRowsTY, R = kZeroRing, XROWS = TY + 4, BROWS = TY + 2;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), w = warp / WPR;
+  const Row<NS, WPR, NXT> row(nx_, warp % WPR);
+  const int nx = row.nx, nxp = nx >> 1;
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  float* BSM = reinterpret_cast<float*>(sm_raw);
+  float* RP = BSM + R * XROWS * nx;
+  float* XB = RP + 2 * XROWS * nxp;
+  float* RY = XB + 2 * BROWS * nxp;
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(RY + (TY / 2) * nxp);
+
   const int y0 = blockIdx.x * TY;
-  const int k0 = blockIdx.y * zc, k1 = min(k0 + zc, nz);
+  const int k0 = blockIdx.y * zc, k1 = min(k0 + zc, nz);  // even
   const bool down = blockIdx.y & 1;
-  const size_t plane = (size_t)NX * ny;
-  const int nyc = ny >> 1;
-  const float sh = bshift ? (float)(*bshift) : 0.f;
+  const float2 msh = dup2(bshift ? -(float)(*bshift) : -0.f), off2 = dup2(off), inv2 = dup2(inv);
+  const float2 off8 = dup2(off * 0.125f);
   const bool interior = w >= 1 && w <= TY;
   const int y = y0 - 1 + w;
-  const int ypar = y & 1;  // ny is even, so the wrap keeps it
+  const bool odd_row = y & 1;
   const int last = k1 - k0 + 3;
   auto mp = [&](int i) { return down ? k1 + 1 - i : k0 - 2 + i; };
+  // parity of this warp's row in march plane 1 (ny is even, so the wrap keeps it)
+  const bool a1 = (y + mp(1)) & 1;
 
   if (tid == 0) {
     for (int s = 0; s < R; ++s) mbar_init(smem_u32(bars + s), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  __syncthreads();
-  // box start rows wrapped once; march planes lie in [-2, nz + 1]
-  const int ya = wrapm(y0 - 2, ny), yb = wrapm(y0 + TY, ny);
-  auto issue = [&](int i) {
-    const int s = i % R;
+  cta_sync();
+  // stage i = -1 .. last - 1 (slot (i + 1) % R): b of march plane i + 1
+  auto issue = [&](int i, unsigned lead) {
+    const int s = (i + 1) % R;
     const unsigned bar = smem_u32(bars + s);
-    int z = mp(i);
+    int z = mp(i + 1);
     z += z < 0 ? nz : (z >= nz ? -nz : 0);
-    float* bs = BSM + s * XROWS * NX;
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    mbar_expect_tx(bar, BBYTES);
-    tma_load3(smem_u32(bs), &mb_pair, 0, ya, z, bar);
-    tma_load3(smem_u32(bs + 2 * NX), &mb_tile, 0, y0, z, bar);
-    tma_load3(smem_u32(bs + (TY + 2) * NX), &mb_pair, 0, yb, z, bar);
+    mbar_expect_tx(bar, XROWS * nx * 4, lead);
+    load_rows<TY, 2>(BSM + s * XROWS * nx, nx, mb, y0, ny, z, bar, lead);
   };
-  auto wait_plane = [&](int i, unsigned limit) {
-    return mbar_wait(smem_u32(bars + (i % R)), (unsigned)((i / R) & 1), limit);
+  auto wait_stage = [&](int i, unsigned limit) {
+    return mbar_wait(smem_u32(bars + (i + 1) % R), (unsigned)(((i + 1) / R) & 1), limit);
   };
-  auto brow = [&](int i, int r) { return reinterpret_cast<const float4*>(BSM + (i % R) * XROWS * NX + r * NX); };
-  auto xrow = [&](int i, int r) { return reinterpret_cast<float4*>(XB + (i & 1) * XBROWS * NX + r * NX); };
+  auto rprow = [&](int par, int r) { return RP + (par * XROWS + r) * nxp; };
+  auto xbrow = [&](int par, int r) { return XB + (par * BROWS + r) * nxp; };
+  auto put_row = [&](float* p, const float2 (&v)[NS]) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (row.valid(s)) *reinterpret_cast<float2*>(p + 2 * row.group(s)) = v[s];
+  };
+  auto get_row = [&](float2 (&v)[NS], const float* p) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) v[s] = *reinterpret_cast<const float2*>(p + 2 * row.group(s));
+  };
+  // the plane in ring slot `slot` (its march index's parity par, this row's
+  // parity a): its red cells, (b - shift) / diag, into r (this warp's row) and
+  // into the published rows; its black cells' b - shift into bb
+  auto take_plane = [&](float2 (&r)[NS], float2 (&bb)[NS], bool a, int slot, int par) {
+    const float* p = BSM + (slot * XROWS + w + 1) * nx;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const float4 t = *reinterpret_cast<const float4*>(p + 4 * row.group(s));
+      r[s] = mul2(add2(a ? make_float2(t.y, t.w) : make_float2(t.x, t.z), msh), inv2);
+      bb[s] = add2(a ? make_float2(t.x, t.z) : make_float2(t.y, t.w), msh);
+    }
+    put_row(rprow(par, w + 1), r);
+    if (!interior) {  // the outer row next to this halo row (the other parity)
+      const int o = w == 0 ? 0 : TY + 3;
+      const float* q = BSM + (slot * XROWS + o) * nx;
+      float2 v[NS];
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const float4 t = *reinterpret_cast<const float4*>(q + 4 * row.group(s));
+        v[s] = mul2(add2(a ? make_float2(t.x, t.z) : make_float2(t.y, t.w), msh), inv2);
+      }
+      put_row(rprow(par, o), v);
+    }
+  };
 
   bool ok = true;
-  if (tid == 0) {
-    for (int i = 0; i < R && i <= last; ++i) issue(i);
-    ok = wait_plane(0, wait_limit) && wait_plane(1, wait_limit) && wait_plane(2, wait_limit);
-  }
-  int issued = min(R - 1, last);
-  ok = !__syncthreads_or(!ok);
-  int done = ok ? 2 : -1;
-
-  auto shifted = [&](float4 t) {
-    t.x -= sh, t.y -= sh, t.z -= sh, t.w -= sh;
-    return t;
-  };
-  // b - shift of this thread's row: planes i-1, i, i+1 (march order)
-  float4 B0[NS], B1[NS], B2[NS];
-  // x of this thread's row: planes i-2, i-1, i
-  float4 X0[NS], X1[NS], X2[NS];
-  float2 acc[NS], held[NS];  // restriction sums: plane pair in progress / completed (even rows)
-  if (ok) {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      B0[s] = shifted(brow(0, w + 1)[lane + 32 * s]);
-      B1[s] = shifted(brow(1, w + 1)[lane + 32 * s]);
-    }
-  }
-  __syncthreads();  // step 1 refills plane 0's slot
-  bool pending = false;  // an even row holds a completed pair to combine
-
-  // x on march plane i from b' of planes i-1 (bm), i (b0), i+1 (bp) of this
-  // row and rows y -/+ 1 of plane i (shared memory): red cells b'/diag, black
-  // cells (b' + off * sum of the red neighbours' b'/diag) / diag.
-  auto form_x = [&](float4 (&xo)[NS], const float4 (&bm)[NS], const float4 (&b0)[NS], const float4 (&bp)[NS],
-                    int i, int a) {
-    const float4* u = brow(i, w) + lane;
-    const float4* dn = brow(i, w + 2) + lane;
-    float tl[NS], tr[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      tl[s] = __shfl_sync(0xffffffffu, b0[s].w, (lane + 31) & 31);
-      tr[s] = __shfl_sync(0xffffffffu, b0[s].x, (lane + 1) & 31);
-    }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const float L = (lane == 0 ? tl[(s + NS - 1) % NS] : tl[s]) * inv;
-      const float Rr = (lane == 31 ? tr[(s + 1) % NS] : tr[s]) * inv;
-      const float4 uu = shifted(u[32 * s]), dd = shifted(dn[32 * s]);
-      const float c0 = b0[s].x * inv, c1 = b0[s].y * inv, c2 = b0[s].z * inv, c3 = b0[s].w * inv;
-      auto blk = [&](float bv, float l, float r, float uv, float dv, float zm, float zp) {
-        return (bv + off * (((l + r) + (uv * inv + dv * inv)) + (zm * inv + zp * inv))) * inv;
-      };
-      float4 o;
-      if (a == 0) {  // red at e = 0, 2
-        o.x = c0;
-        o.y = blk(b0[s].y, c0, c2, uu.y, dd.y, bm[s].y, bp[s].y);
-        o.z = c2;
-        o.w = blk(b0[s].w, c2, Rr, uu.w, dd.w, bm[s].w, bp[s].w);
-      } else {  // red at e = 1, 3
-        o.x = blk(b0[s].x, L, c1, uu.x, dd.x, bm[s].x, bp[s].x);
-        o.y = c1;
-        o.z = blk(b0[s].z, c1, c3, uu.z, dd.z, bm[s].z, bp[s].z);
-        o.w = c3;
-      }
-      xo[s] = o;
-    }
-  };
-  // residual b' - A x of this row on march plane i - 1, x-pair sums
-  auto resid = [&](float2 (&p)[NS], const float4 (&xm)[NS], const float4 (&x0)[NS], const float4 (&xp)[NS],
-                   const float4 (&b0)[NS], int i) {
-    const float4* u = xrow(i - 1, w - 1) + lane;
-    const float4* dn = xrow(i - 1, w + 1) + lane;
-    float tl[NS], tr[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      tl[s] = __shfl_sync(0xffffffffu, x0[s].w, (lane + 31) & 31);
-      tr[s] = __shfl_sync(0xffffffffu, x0[s].x, (lane + 1) & 31);
-    }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const float L = lane == 0 ? tl[(s + NS - 1) % NS] : tl[s];
-      const float Rr = lane == 31 ? tr[(s + 1) % NS] : tr[s];
-      const float4 uu = u[32 * s], dd = dn[32 * s];
-      auto r = [&](float bv, float c, float l, float rr, float uv, float dv, float zm, float zp) {
-        return bv - (diag * c - off * (((l + rr) + (uv + dv)) + (zm + zp)));
-      };
-      const float r0 = r(b0[s].x, x0[s].x, L, x0[s].y, uu.x, dd.x, xm[s].x, xp[s].x);
-      const float r1 = r(b0[s].y, x0[s].y, x0[s].x, x0[s].z, uu.y, dd.y, xm[s].y, xp[s].y);
-      const float r2 = r(b0[s].z, x0[s].z, x0[s].y, x0[s].w, uu.z, dd.z, xm[s].z, xp[s].z);
-      const float r3 = r(b0[s].w, x0[s].w, x0[s].z, Rr, uu.w, dd.w, xm[s].w, xp[s].w);
-      p[s] = make_float2(r0 + r1, r2 + r3);
-    }
-  };
+  // where this row of plane mp(2), mp(3), ... and the coarse rows go
+  const ptrdiff_t pplane = (ptrdiff_t)nxp * ny, cplane = (ptrdiff_t)nxp * (ny >> 1);
+  float* dst = xb + (ptrdiff_t)mp(2) * pplane + (ptrdiff_t)y * nxp;
+  float* cdst = bc + (ptrdiff_t)(mp(2) >> 1) * cplane + (ptrdiff_t)(y >> 1) * nxp;
+  const ptrdiff_t dstep = down ? -pplane : pplane, cstep = down ? -cplane : cplane;
+  float2 held[NS];  // restriction sums of a completed plane pair (even rows)
   // coarse row of an even fine row y: its held sums plus the odd row's (RY)
-  auto combine = [&](int kc) {
-    const float2* ry = RY + ((w - 1) >> 1) * (NXC / 2);
-    float2* dst = reinterpret_cast<float2*>(bc + ((size_t)kc * nyc + (y >> 1)) * NXC);
+  auto combine = [&]() {
+    float2 o[NS];
+    get_row(o, RY + ((w - 1) >> 1) * nxp);
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const float2 o = ry[lane + 32 * s];
-      dst[lane + 32 * s] = make_float2((held[s].x + o.x) * 0.125f, (held[s].y + o.y) * 0.125f);
-    }
+    for (int s = 0; s < NS; ++s)
+      if (row.valid(s)) *reinterpret_cast<float2*>(cdst + 2 * row.group(s)) = mul2(add2(held[s], o[s]), off8);
+    cdst += cstep;
   };
-  int kc_pending = 0;
+  auto march = [&](auto first_parity) {
+    constexpr bool A1 = decltype(first_parity)::value;
+    // red cells of three planes, b of the black cells of two, black cells of three
+    float2 R0[NS], R1[NS], R2[NS], B0[NS], B1[NS], X0[NS], X1[NS], X2[NS];
+    float2 acc[NS];  // restriction sums of the plane pair in progress
+    ok = !cta_sync_or(false);  // stages -1, 0 and 1 have landed
+    if (!ok) return;
+    take_plane(R0, B1, !A1, 0, 0);
+    take_plane(R1, B0, A1, 1, 1);
+    cta_sync();  // the slots of stages -1 and 0 are free
 
-  // Step i: bm, b0, bp = b' of march planes i-1, i, i+1 (bp is loaded here);
-  // xm2, xm1, x0 = x of march planes i-2, i-1, i (x0 is formed here).
-  auto step = [&](float4 (&bm)[NS], float4 (&b0)[NS], float4 (&bp)[NS], float4 (&xm2)[NS], float4 (&xm1)[NS],
-                  float4 (&x0)[NS], int i) -> bool {
-    if (i > last - 1 || !ok) return false;
-    if (tid == 0 && i + 3 <= last) issue(i + 3);
-    if (i + 3 <= last) issued = i + 3;
-    if (pending) {  // the odd row left its sums in RY before the last barrier
-      combine(kc_pending);
-      pending = false;
-    }
+    // Step i: rm, r0, rp = red cells of march planes i - 1, i, i + 1 (rp is read here); b0 / bp = b of the black cells
+    // of planes i / i + 1; xm2, xm1, x0 = black cells of planes i - 2, i - 1, i (x0 is formed here).
+    auto step = [&](float2 (&rm)[NS], float2 (&r0)[NS], float2 (&rp)[NS], float2 (&b0)[NS], float2 (&bp)[NS],
+                    float2 (&xm2)[NS], float2 (&xm1)[NS], float2 (&x0)[NS], int i, auto phase) {
+      constexpr int PH = decltype(phase)::value, P0 = (PH + 1) & 1, P1 = PH & 1;
+      constexpr bool a = A1 != (bool)(PH & 1);  // plane i: red cells at 2 m + a, black ones at 2 m + 1 - a
+      // plane pairs complete at even i; the odd row left its sums in RY before the last barrier
+      if (P0 == 1 && interior && !odd_row && i >= 5) combine();
+      take_plane(rp, bp, !a, (i + 1) % R, P1);
+      float2 n[NS], u[NS], d[NS];
+      nbr_sums<NS, WPR, NXT>(n, r0, rprow(P0, w + 1), !a, row);
+      get_row(u, rprow(P0, w));
+      get_row(d, rprow(P0, w + 2));
 #pragma unroll
-    for (int s = 0; s < NS; ++s) bp[s] = shifted(brow(i + 1, w + 1)[lane + 32 * s]);
-    const int z = mp(i);
-    form_x(x0, bm, b0, bp, i, (ypar + z) & 1);
-    float4* xr = xrow(i, w);
+      for (int s = 0; s < NS; ++s)
+        x0[s] = mul2(fma2(off2, add2(add2(n[s], add2(u[s], d[s])), add2(rm[s], rp[s])), b0[s]), inv2);
+      put_row(xbrow(P0, w), x0);
+      if (interior && i >= 3) {
+        put_row(dst, xm1);
+        dst += dstep;
+        nbr_sums<NS, WPR, NXT>(n, xm1, xbrow(P1, w), !a, row);
+        get_row(u, xbrow(P1, w - 1));
+        get_row(d, xbrow(P1, w + 1));
+        // march order visits a plane pair (2K, 2K + 1) upwards or downwards, its first plane at odd i
 #pragma unroll
-    for (int s = 0; s < NS; ++s) xr[lane + 32 * s] = x0[s];
-    if (interior && i >= 3) {
-      const int zr = mp(i - 1);  // plane of the residual, in [k0, k1)
-      float4* dst = reinterpret_cast<float4*>(xout + (size_t)zr * plane + (size_t)y * NX);
+        for (int s = 0; s < NS; ++s) {
+          const float2 p = add2(add2(n[s], add2(u[s], d[s])), add2(xm2[s], x0[s]));
+          acc[s] = P0 == 1 ? p : add2(acc[s], p);
+        }
+        if (P0 == 0) {
+          if (odd_row) {
+            put_row(RY + ((w - 2) >> 1) * nxp, acc);
+          } else {
 #pragma unroll
-      for (int s = 0; s < NS; ++s) dst[lane + 32 * s] = xm1[s];
-      float2 pr[NS];
-      resid(pr, xm2, xm1, x0, bm, i);
-      // march order visits a plane pair (2K, 2K + 1) upwards or downwards
-      const bool first = down ? (zr & 1) : !(zr & 1);
-#pragma unroll
-      for (int s = 0; s < NS; ++s) acc[s] = first ? pr[s] : make_float2(acc[s].x + pr[s].x, acc[s].y + pr[s].y);
-      if (!first) {
-        if (ypar) {
-          float2* ry = RY + ((w - 2) >> 1) * (NXC / 2);
-#pragma unroll
-          for (int s = 0; s < NS; ++s) ry[lane + 32 * s] = acc[s];
-        } else {
-#pragma unroll
-          for (int s = 0; s < NS; ++s) held[s] = acc[s];
-          pending = true;
-          kc_pending = zr >> 1;
+            for (int s = 0; s < NS; ++s) held[s] = acc[s];
+          }
         }
       }
+      if constexpr (PH == 5)
+        ok = !cta_sync_or(false);
+      else
+        cta_sync();
+    };
+#define IBRD_STEP(r0, r1, r2, b0, b1, x0, x1, x2, ph) \
+  if (i + ph >= last) return;                         \
+  step(r0, r1, r2, b0, b1, x0, x1, x2, i + ph, std::integral_constant<int, ph>{});
+    for (int i = 1; ok; i += 6) {
+      IBRD_STEP(R0, R1, R2, B0, B1, X0, X1, X2, 0)
+      IBRD_STEP(R1, R2, R0, B1, B0, X1, X2, X0, 1)
+      IBRD_STEP(R2, R0, R1, B0, B1, X2, X0, X1, 2)
+      IBRD_STEP(R0, R1, R2, B1, B0, X0, X1, X2, 3)
+      IBRD_STEP(R1, R2, R0, B0, B1, X1, X2, X0, 4)
+      IBRD_STEP(R2, R0, R1, B1, B0, X2, X0, X1, 5)
     }
-    bool good = true;
-    if (tid == 0 && i + 2 <= last) good = wait_plane(i + 2, wait_limit);
-    ok = !__syncthreads_or(!good);
-    if (ok) done = i + 2;
-    return ok;
+#undef IBRD_STEP
   };
-  for (int i = 1; i < last; i += 6) {
-    if (!step(B0, B1, B2, X0, X1, X2, i)) break;
-    if (!step(B1, B2, B0, X1, X2, X0, i + 1)) break;
-    if (!step(B2, B0, B1, X2, X0, X1, i + 2)) break;
-    if (!step(B0, B1, B2, X0, X1, X2, i + 3)) break;
-    if (!step(B1, B2, B0, X1, X2, X0, i + 4)) break;
-    if (!step(B2, B0, B1, X2, X0, X1, i + 5)) break;
+  if (w == TY + 2) {
+    feed_stages(last, 2, 3, issue, wait_stage, wait_limit, err);  // stage i + 3 takes the slot of stage i - 1
+  } else if (a1) {
+    march(std::true_type{});
+  } else {
+    march(std::false_type{});
   }
-  if (!ok) {
-    if (tid == 0) {
-      for (int i = done + 1; i <= issued; ++i) wait_plane(i, kDrainLimit);
-      atomicOr(err, 1);
-    }
-    __syncthreads();
-    return;
+  if (ok && interior && !odd_row) combine();  // the last pair (its RY write preceded the last barrier)
+}
+
+// x = the field whose black cells are packed in xb and whose red cells are
+// (b - shift) / diag (the state after a first sweep from zero): for V-cycles
+// that need the pre-smoothed field in full (no post-smoothing sweep, or the
+// prolongation kept separate). One thread per 4-cell group.
+__global__ void __launch_bounds__(256) k_unpack_zero(const float* __restrict__ xb, const float* __restrict__ b,
+                                                     const double* __restrict__ bshift, float* __restrict__ x,
+                                                     int nx, int ny, int nz, float inv) {
+  const size_t groups = (size_t)(nx >> 2) * ny * nz;
+  const float sh = bshift ? (float)(*bshift) : 0.f;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < groups;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const size_t r = t / (nx >> 2);  // row j + ny k
+    const bool a = ((int)(r % ny) + (int)(r / ny)) & 1;
+    const float2 k = reinterpret_cast<const float2*>(xb)[t];
+    const float4 q = reinterpret_cast<const float4*>(b)[t];
+    reinterpret_cast<float4*>(x)[t] = a ? make_float4(k.x, (q.y - sh) * inv, k.y, (q.w - sh) * inv)
+                                        : make_float4((q.x - sh) * inv, k.x, (q.z - sh) * inv, k.y);
   }
-  if (pending) combine(kc_pending);  // the last pair (its RY write preceded the last barrier)
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -687,68 +829,75 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// Tensor map of an FP32 field [nz][ny][nx] with boxes of nx x rows x 1.
-CUtensorMap field_map(const float* f, Dims d, int rows) {
+// Tensor map of an FP32 field of rows of nx values [nz][ny][nx] with boxes of
+// one plane of `rows` whole rows. A box side holds at most 256 values: longer
+// rows are two halves (a fourth dimension), which land one after the other.
+CUtensorMap field_map(const float* f, int nx, int ny, int nz, int rows) {
   CUtensorMap m;
   std::memset(&m, 0, sizeof(m));
-  const cuuint64_t dims[3] = {(cuuint64_t)d.nx, (cuuint64_t)d.ny, (cuuint64_t)d.nz};
-  const cuuint64_t strides[2] = {(cuuint64_t)d.nx * 4, (cuuint64_t)d.nx * d.ny * 4};
-  const cuuint32_t box[3] = {(cuuint32_t)d.nx, (cuuint32_t)rows, 1};
-  const cuuint32_t es[3] = {1, 1, 1};
-  const CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(f), dims, strides, box,
+  const int parts = nx > 256 ? 2 : 1, w = nx / parts;
+  const cuuint64_t dims[4] = {(cuuint64_t)w, (cuuint64_t)parts, (cuuint64_t)ny, (cuuint64_t)nz};
+  const cuuint64_t strides[3] = {(cuuint64_t)w * 4, (cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
+  const cuuint32_t box[4] = {(cuuint32_t)w, (cuuint32_t)parts, (cuuint32_t)rows, 1};
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  const CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(f), dims, strides, box,
                                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled"};
   return m;
 }
 
-template <int NS, bool PRO>
-constexpr size_t rows_smem() {
-  constexpr int NX = 128 * NS;
-  return sizeof(float) * (size_t)NX *
-             (kRowsRing * (kRowsTY + 4) + kRowsRing * (kRowsTY + 2) + (kRowsTY + 2) +
-              (PRO ? kCoarseRing * (kRowsTY / 2 + 4) / 2 : 0)) +
-         8 * kRowsRing;
+RowMaps row_maps(const float* f, int nx, int ny, int nz, int rows, int halo) {
+  return RowMaps{field_map(f, nx, ny, nz, rows + 2 * halo), field_map(f, nx, ny, nz, rows + halo),
+                 field_map(f, nx, ny, nz, halo)};
 }
-// two CTAs per SM (228 KB of shared memory, 1 KB reserved per CTA)
-static_assert(2 * (rows_smem<2, true>() + 1024) <= 228 * 1024, "two CTAs per SM");
 
-template <int NS, bool PRO>
-void rows_launch(dim3 g, cudaStream_t s, const CUtensorMap (&m)[6], float* xout, const double* bshift, Dims d,
-                 int zc, float inv, float off, double* part, int* err, unsigned limit) {
-  constexpr size_t sm = rows_smem<NS, PRO>();
+// two CTAs of the sweep and three of the sweep from zero per SM at 256-cell
+// rows (228 KB of shared memory, 1 KB reserved per CTA)
+static_assert(2 * (4 * sweep_rows_floats(256, IN_FULL_PRO) + 8 * kSweepRing + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(3 * (4 * zero_rows_floats(256) + 8 * kZeroRing + 1024) <= 228 * 1024, "three CTAs per SM");
+
+template <int NS, int WPR, int NXT, int IN>
+void sweep_rows_go(dim3 g, cudaStream_t s, const RowMaps& mx, const RowMaps& mb, const RowMaps& mc, float* xout, const double* bshift, Dims d,
+                   int zc, float inv, float off, double* part) {
+  const size_t sm = 4 * sweep_rows_floats(d.nx, IN) + 8 * kSweepRing;
   static std::atomic<unsigned long long> attr{0};
-  ensure_smem_attr((const void*)k_rbgs_rows<NS, PRO>, (int)sm, attr);
-  k_rbgs_rows<NS, PRO><<<g, (kRowsTY + 2) * 32, sm, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], xout, bshift, d.ny,
-                                                          d.nz, zc, inv, off, part, err, limit);
+  ensure_smem_attr((const void*)k_rbgs_rows<NS, WPR, NXT, IN>,
+                   (int)(4 * sweep_rows_floats(NXT ? NXT : 128 * NS * WPR, IN) + 8 * kSweepRing), attr);
+  k_rbgs_rows<NS, WPR, NXT, IN><<<g, kRowsThreads<WPR>, sm, s>>>(
+      mx, mb, mc, xout, bshift, d.nx, d.ny, d.nz, zc, inv, off, part, wait_error_flag(),
+      wait_limit());
 }
 
-// The row sweep of xin into xout; with xc non-null, of xin + P xc (the fused
-// prolongation, zc even).
-int rows_sweep_any(const float* xin, const float* xc, float* xout, const float* b, const double* bshift, Dims d,
+// Calls f with the kernel shape of rows of nx cells (see rows_sweep_ok).
+template <typename F>
+void with_row_shape(int nx, F&& f) {
+  if (nx == 128)
+    f(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{}, std::integral_constant<int, 128>{});
+  else
+    f(std::integral_constant<int, 2>{}, std::integral_constant<int, 1>{}, std::integral_constant<int, 256>{});
+}
+
+// The row sweep of x (in: SweepIn; xc the coarse field of the fused prolongation) into xout.
+template <int IN>
+int sweep_rows_any(const float* xin, const float* xc, float* xout, const float* b, const double* bshift, Dims d,
                    Stencil st, int zc, double* part, int part_cap, cudaStream_t s) {
-  const Dims dc{d.nx / 2, d.ny / 2, d.nz / 2};
-  const CUtensorMap mx = field_map(xin, d, kRowsTY), mx2 = field_map(xin, d, 2);
-  const CUtensorMap m[6] = {mx, mx2, field_map(b, d, kRowsTY), field_map(b, d, 1),
-                            xc ? field_map(xc, dc, kRowsTY / 2) : mx, xc ? field_map(xc, dc, 2) : mx2};
+  const int nxr = IN == IN_PACKED_PRO ? d.nx / 2 : d.nx;
+  const RowMaps mx = row_maps(xin, nxr, d.ny, d.nz, kRowsTY, 2), mb = row_maps(b, d.nx, d.ny, d.nz, kRowsTY, 1);
+  const RowMaps mc = xc ? row_maps(xc, d.nx / 2, d.ny / 2, d.nz / 2, kRowsTY / 2, 2) : mx;
   dim3 g(d.ny / kRowsTY, (d.nz + zc - 1) / zc);
   const int nblk = (int)(g.x * g.y);
   if (nblk > part_cap) part = nullptr;
-  const float inv = (float)(1.0 / st.diag), off = (float)st.off;
-  int* err = wait_error_flag();
-  const unsigned limit = wait_limit();
-  if (d.nx == 256) {
-    if (xc)
-      rows_launch<2, true>(g, s, m, xout, bshift, d, zc, inv, off, part, err, limit);
-    else
-      rows_launch<2, false>(g, s, m, xout, bshift, d, zc, inv, off, part, err, limit);
-  } else {
-    if (xc)
-      rows_launch<1, true>(g, s, m, xout, bshift, d, zc, inv, off, part, err, limit);
-    else
-      rows_launch<1, false>(g, s, m, xout, bshift, d, zc, inv, off, part, err, limit);
-  }
+  with_row_shape(d.nx, [&](auto ns, auto wpr, auto nxt) {
+    sweep_rows_go<ns.value, wpr.value, nxt.value, IN>(g, s, mx, mb, mc, xout, bshift, d, zc, (float)(1.0 / st.diag),
+                                                      (float)st.off, part);
+  });
   return part ? nblk : 0;
+}
+
+int clamp_zc(int zc, int nz, bool even) {
+  zc = zc < 2 ? 2 : (zc > nz ? nz : zc);
+  return even ? zc + (zc & 1) : zc;
 }
 
 }  // namespace
@@ -773,20 +922,20 @@ int launch_rows_sweep(const float* xin, float* xout, const float* b, const doubl
                       int zc, double* part, int part_cap, cudaStream_t s) {
   if (!rows_sweep_ok(d) || !aligned16(xin) || !aligned16(xout) || !aligned16(b) || xin == xout || b == xout)
     throw CudaError{cudaErrorInvalidValue, "row sweep arguments"};
-  zc = zc < 2 ? 2 : (zc > d.nz ? d.nz : zc);
-  return rows_sweep_any(xin, nullptr, xout, b, bshift, d, st, zc, part, part_cap, s);
+  return sweep_rows_any<IN_FULL>(xin, nullptr, xout, b, bshift, d, st, clamp_zc(zc, d.nz, false), part, part_cap, s);
 }
 
-int launch_rows_prolong_sweep(const float* xc, const float* xin, float* xout, const float* b, const double* bshift,
-                              Dims d, Stencil st, int zc, double* part, int part_cap, cudaStream_t s) {
+int launch_rows_prolong_sweep(const float* xc, const float* xin, bool packed, float* xout, const float* b,
+                              const double* bshift, Dims d, Stencil st, int zc, double* part, int part_cap,
+                              cudaStream_t s) {
   if (!rows_sweep_ok(d) || !aligned16(xin) || !aligned16(xout) || !aligned16(b) || !aligned16(xc) || xin == xout ||
       b == xout || xc == xout)
     throw CudaError{cudaErrorInvalidValue, "prolongation + row sweep arguments"};
-  zc = zc < 2 ? 2 : (zc > d.nz ? d.nz : zc);
-  zc += zc & 1;  // even chunks: fine planes 2K - 1, 2K share their coarse pair in both march directions
-  return rows_sweep_any(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s);
+  // even chunks: fine planes 2K - 1, 2K share their coarse pair in both march directions
+  zc = clamp_zc(zc, d.nz, true);
+  return packed ? sweep_rows_any<IN_PACKED_PRO>(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s)
+                : sweep_rows_any<IN_FULL_PRO>(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s);
 }
-
 
 bool zero_restrict_rows_ok(Dims d) { return rows_sweep_ok(d); }
 
@@ -794,29 +943,30 @@ int zero_restrict_rows_default_zc(Dims d) {
   return rows_sweep_default_zc(d);  // even: plane pairs of the restriction stay inside a chunk
 }
 
-void launch_zero_restrict_rows(const float* b, const double* bshift, float* x, float* bc, Dims d, Stencil st,
+void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, float* bc, Dims d, Stencil st,
                                int zc, cudaStream_t s) {
-  if (!zero_restrict_rows_ok(d) || !aligned16(b) || !aligned16(x) || ((uintptr_t)bc & 7u) || b == x)
+  if (!zero_restrict_rows_ok(d) || !aligned16(b) || !aligned16(xb) || ((uintptr_t)bc & 7u) || b == xb)
     throw CudaError{cudaErrorInvalidValue, "fused zero sweep + restriction arguments"};
-  zc = zc < 2 ? 2 : (zc > d.nz ? d.nz : zc);
-  zc += zc & 1;
-  const CUtensorMap mt = field_map(b, d, kRowsTY), mpair = field_map(b, d, 2);
+  zc = clamp_zc(zc, d.nz, true);
+  const RowMaps mb = row_maps(b, d.nx, d.ny, d.nz, kRowsTY, 2);
   dim3 g(d.ny / kRowsTY, (d.nz + zc - 1) / zc);
-  const float inv = (float)(1.0 / st.diag), off = (float)st.off, diag = (float)st.diag;
-  int* err = wait_error_flag();
-  const unsigned limit = wait_limit();
-  auto go = [&](auto kern, int ns) {
-    const size_t sm = sizeof(float) * (size_t)(128 * ns) *
-                          (kRowsRing * (kRowsTY + 4) + 2 * (kRowsTY + 2) + kRowsTY / 2 / 2) +
-                      8 * kRowsRing;
-    static std::atomic<unsigned long long> attr1{0}, attr2{0};
-    ensure_smem_attr((const void*)kern, (int)sm, ns == 2 ? attr2 : attr1);
-    kern<<<g, (kRowsTY + 2) * 32, sm, s>>>(mt, mpair, x, bc, bshift, d.ny, d.nz, zc, inv, off, diag, err, limit);
-  };
-  if (d.nx == 256)
-    go(k_zr_rows<2>, 2);
-  else
-    go(k_zr_rows<1>, 1);
+  with_row_shape(d.nx, [&](auto ns, auto wpr, auto nxt) {
+    constexpr int NS = ns.value, WPR = wpr.value, NXT = nxt.value;
+    const size_t sm = 4 * zero_rows_floats(d.nx) + 8 * kZeroRing;
+    static std::atomic<unsigned long long> attr{0};
+    ensure_smem_attr((const void*)k_zr_rows<NS, WPR, NXT>,
+                     (int)(4 * zero_rows_floats(NXT ? NXT : 128 * NS * WPR) + 8 * kZeroRing), attr);
+    k_zr_rows<NS, WPR, NXT><<<g, kRowsThreads<WPR>, sm, s>>>(
+        mb, xb, bc, bshift, d.nx, d.ny, d.nz, zc, (float)(1.0 / st.diag), (float)st.off, wait_error_flag(),
+        wait_limit());
+  });
+}
+
+void launch_unpack_zero(const float* xb, const float* b, const double* bshift, float* x, Dims d, Stencil st,
+                        cudaStream_t s) {
+  const size_t groups = d.n() / 4;
+  const int blocks = (int)std::min<size_t>((groups + 255) / 256, 152 * 16);
+  k_unpack_zero<<<blocks, 256, 0, s>>>(xb, b, bshift, x, d.nx, d.ny, d.nz, (float)(1.0 / st.diag));
 }
 
 }  // namespace ibrd
