@@ -365,9 +365,9 @@ ibrd_status ibrd_solve_many(int count, const ibrd_solve_item* items, int threads
 /* Autotuner (not in the paper: launch-shape selection for this library's
    kernels). For every multigrid level whose red-black sweeps (Sec. III.E) run
    as a fused one-pass sweep kernel, times candidate launch shapes of the
-   sweep -- the row-resident FP32 kernel (levels whose rows are 128 or 256
-   cells; tx = nx) or the tiled kernel with tile width 32 or 64 cells (FP32)
-   or 32 (FP64), each with z-march depths (planes per CTA, 2 to 512) -- and
+   sweep -- the row-resident FP32 kernel (levels whose rows are a multiple of
+   32 of at most 512 cells; tx = nx at 128 and 256 cells, else 0) or the tiled
+   kernel with tile width 32 or 64 cells (FP32) or 32 (FP64), each with z-march depths (planes per CTA, 2 to 512) -- and
    the z-march depth of the stencil pass that forms the first
    sweep from a zero guess (FP32), on scratch fields of the level's size with
    CUDA events, and keeps a shape only when it is at least 3 % faster than the
@@ -407,7 +407,8 @@ double ibrd_periodic_constant(double lx, double ly, double lz);
    handle's hierarchy, tx in {0, 32, 64} or tx = nx (0 for kind 1; 64 only
    for FP32 and when 64 divides nx, else ignored; nx selects the row-resident
    FP32 sweep on levels whose rows are 128 or 256 cells, ny a multiple of 8
-   and nz even), zc >= 0 (0 = built-in; clamped to the level's nz).
+   and nz even; 0, the built-in rule, selects it wherever it serves the level),
+   zc >= 0 (0 = built-in; clamped to the level's nz).
    kind 2 (FP32 only, zc = 0) is the coarse-grid correction of the level: on
    levels the row-resident sweep serves, the V-cycle adds the prolongation of
    the coarse correction inside the first post-smoothing sweep (one pass over

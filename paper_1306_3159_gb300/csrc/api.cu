@@ -2161,6 +2161,10 @@ double time_sweep(ibrd_grid g, int kind, Dims d, Stencil st, T* const set[2][3],
   return best;
 }
 
+// Levels whose row-resident sweep a shape names by its row length (the others
+// have it as their built-in shape).
+bool rows_named(Dims d) { return d.nx == 128 || d.nx == 256; }
+
 // Tunes the sweep kernels of element type T on the levels that run them.
 template <typename T>
 void autotune_levels(ibrd_grid g, bool retune, std::vector<ibrd_tune_entry>& rep) {
@@ -2216,7 +2220,7 @@ void autotune_levels(ibrd_grid g, bool retune, std::vector<ibrd_tune_entry>& rep
           if (kind == TUNE_SWEEP) {
             txs = {32};
             if (elem == 4 && d.nx % 64 == 0) txs.push_back(64);
-            if (elem == 4 && rows_sweep_ok(d)) txs.push_back(d.nx);
+            if (elem == 4 && rows_sweep_ok(d)) txs.push_back(rows_named(d) ? d.nx : 0);
           }
           static const int zcs[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
           for (int tx : txs)
@@ -3070,7 +3074,8 @@ ibrd_status ibrd_autotune(ibrd_grid g, int precision, int retune, ibrd_tune_entr
 
 ibrd_status ibrd_tune_set(ibrd_grid g, int elem_bytes, int kind, int nx, int ny, int nz, int tx, int zc) {
   return guarded(g, "ibrd_tune_set", [&]() {
-    const bool rows = elem_bytes == 4 && kind == TUNE_SWEEP && tx == nx && rows_sweep_ok(Dims{nx, ny, nz});
+    const bool rows =
+        elem_bytes == 4 && kind == TUNE_SWEEP && tx == nx && rows_sweep_ok(Dims{nx, ny, nz}) && rows_named(Dims{nx, ny, nz});
     const bool pro = kind == TUNE_PROLONG;
     if ((elem_bytes != 4 && elem_bytes != 8) || (kind != TUNE_SWEEP && kind != TUNE_ZERO && !pro) || zc < 0 ||
         (!pro && tx != 0 && tx != 32 && tx != 64 && !rows) || (kind == TUNE_ZERO && tx != 0) ||

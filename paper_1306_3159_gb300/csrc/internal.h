@@ -157,8 +157,8 @@ bool rb_sweep_fused_ok(Dims d);
 template <typename T>
 bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b);
 // Launch shape of a red-black sweep kernel picked by the autotuner: tile width
-// tx (cells, fused sweep only: 32 or 64 for the tiled kernel, nx for the
-// row-resident kernel on levels it serves) and z-march depth zc (planes per
+// tx (cells, fused sweep only: 32 or 64 for the tiled kernel, nx = 128 or 256
+// for the row-resident kernel there) and z-march depth zc (planes per
 // CTA); 0 keeps the built-in rule (the row-resident kernel where it applies).
 struct SweepShape {
   int tx = 0;

@@ -928,6 +928,13 @@ bool rb_sweep_fused_ok(Dims d) {
 }
 
 
+// Whether a tuned shape (or none) means the row-resident kernel on a level it
+// serves: the built-in width, or the row length where it is 128 or 256 (widths
+// of 32 and 64 name the tiled kernel).
+static bool rows_shape(const SweepShape* tn, Dims d) {
+  return !tn || tn->tx == 0 || (tn->tx == d.nx && d.nx > 64);
+}
+
 template <typename T>
 bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b) {
   if (!aligned16(x) || !aligned16(b)) return false;
@@ -969,12 +976,12 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
     }
   }
   if constexpr (sizeof(T) == 4) {
-    // rows of 128 or 256 cells: the row-resident kernel unless a tiled shape
-    // was chosen for this level
+    // rows of up to 512 cells: the row-resident kernel unless a tiled shape was
+    // chosen for this level
     if (!zero && rows_sweep_ok(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && xin != xout &&
         b != xout && wait_error_flag()) {
       const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
-      if (!tn || tn->tx == 0 || tn->tx == d.nx) {
+      if (rows_shape(tn, d)) {
         const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
         prof_begin(c, s);
         const int r = launch_rows_sweep(xin, xout, b, bshift, d, st, zc, part, part_cap, s);
@@ -1100,7 +1107,7 @@ int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const 
       // chosen or the fusion was switched off for it
       const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
       const SweepShape* tp = tuned_sweep(4, TUNE_PROLONG, d);
-      if ((!tn || tn->tx == 0 || tn->tx == d.nx) && !(tp && tp->tx == 1)) {
+      if (rows_shape(tn, d) && !(tp && tp->tx == 1)) {
         const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
         prof_begin(P_RBGS32, s);
         const int r = launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);

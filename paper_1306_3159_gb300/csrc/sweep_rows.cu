@@ -25,9 +25,14 @@
 // * A warp owns x-rows: lane l holds the 4-cell groups l + 32 s (s < NS) of its
 //   row, two packed entries each. x-neighbours come from the neighbouring
 //   lanes by shuffles; the periodic wrap of rows of 128 NS cells is the shuffle
-//   from lane 31 to lane 0. Rows of other lengths leave lanes idle, rows above
-//   256 cells belong to two warps; there the outermost groups read their
-//   neighbour from the published row in shared memory.
+//   from lane 31 to lane 0. Rows of other lengths (multiples of 32) leave lanes
+//   idle and take one more shuffle for the wrap; rows above 256 cells belong to
+//   two warps, whose outermost groups read their neighbour from the published
+//   row in shared memory. The tiled sweep (smoother.cu), which served these
+//   lengths, is the slower one at all of them: FP32 V-cycles of one pre- and one
+//   post-sweep at 96^3, 160^3, 224^3, 320^3 and 512^3 take 73, 117, 157, 361 and
+//   537 us, with the tiled sweep and separate transfers 88, 151, 222, 446 and
+//   1330 us (512^3 is the largest cube a CTA's shared memory holds rows of).
 // * A CTA owns TY rows of every plane of a z-chunk, plus one halo row on each
 //   side in y whose red cells it also updates (the black cells at the tile's
 //   edge rows need them); the neighbouring CTA computes the same red values
@@ -249,47 +254,47 @@ __device__ __forceinline__ float2 prolong_add2(float2 x, float2 t64) { return fm
 template <int NS, int WPR, int NXT>
 struct Row {
   static constexpr bool kWrap = NXT == 128 * NS && WPR == 1;  // one full warp holds the whole row
-  int nx, lane, g0, gw;  // row length; this lane's group of slot 0; groups per warp
+  int nx, lane, g0, gw;  // row length; the warp's first group and its number of groups (at most 32 in all slots but the last)
   __device__ __forceinline__ Row(int nx_, int warp_in_row) {
     nx = NXT ? NXT : nx_;
     lane = threadIdx.x & 31;
     gw = nx / (4 * WPR);
-    g0 = warp_in_row * gw + lane;
+    g0 = WPR == 1 ? 0 : warp_in_row * gw;
   }
-  __device__ __forceinline__ bool valid(int s) const { return kWrap || lane + 32 * s < gw; }
+  __device__ __forceinline__ bool valid(int s) const { return kWrap || s < NS - 1 || lane + 32 * s < gw; }
   // group of slot s (an idle lane reads the warp's last one)
   __device__ __forceinline__ int group(int s) const {
     if constexpr (kWrap) return lane + 32 * s;
     const int q = lane + 32 * s;
-    return g0 - lane + (q < gw ? q : gw - 1);
+    return g0 + (s < NS - 1 || q < gw ? q : gw - 1);
   }
+  __device__ __forceinline__ int last_lane() const { return (gw - 1) & 31; }  // of the warp's last group, in the last slot
 };
 
 // The packed pairs v moved by one entry: w = the entries m - 1 or, with right,
-// m + 1 of each pair's entries m. The outermost groups a warp's lanes cannot
-// reach by shuffles (rows that do not wrap within the warp) take edge(m).
+// m + 1 of each pair's entries m. Inside a row they are the adjacent lane's, or
+// at lane 0 / 31 the adjacent slot's. Beyond the warp's ends: of a row that is
+// one warp's, the row's other end (the next shuffle target where the row fills
+// the lanes, one more shuffle where it does not); of a row of two warps, edge(m).
 template <int NS, int WPR, int NXT, typename F>
 __device__ __forceinline__ void shifted(float2 (&w)[NS], const float2 (&v)[NS], bool right,
                                         const Row<NS, WPR, NXT>& r, F&& edge) {
+  static_assert(NS <= 2, "the adjacent slot on either side is the other one");
+  constexpr bool kWrap = Row<NS, WPR, NXT>::kWrap;
   const int src = (right ? r.lane + 1 : r.lane + 31) & 31;
-  float t[NS];
+  float t[NS], e = 0.f;
 #pragma unroll
   for (int s = 0; s < NS; ++s) t[s] = __shfl_sync(0xffffffffu, right ? v[s].x : v[s].y, src);
+  if constexpr (!kWrap && WPR == 1) e = __shfl_sync(0xffffffffu, right ? v[0].x : v[NS - 1].y, right ? 0 : r.last_lane());
+  if constexpr (!kWrap && WPR > 1) {
+    const int half = r.nx >> 1, m = right ? 2 * (r.g0 + r.gw) : 2 * r.g0 - 1;
+    e = edge(m < 0 ? m + half : (m >= half ? m - half : m));
+  }
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     float o = t[s];
-    if constexpr (Row<NS, WPR, NXT>::kWrap) {
-      static_assert(NS <= 2, "the adjacent slot on either side is the other one");
-      if (NS == 2 && r.lane == (right ? 31 : 0)) o = t[NS - 1 - s];
-    } else {
-      const int q = r.lane + 32 * s;
-      if (right ? (r.lane == 31 || q == r.gw - 1) : r.lane == 0) {
-        const int g = r.group(s), half = r.nx >> 1;
-        int m = right ? 2 * g + 2 : 2 * g - 1;
-        m = m < 0 ? m + half : (m >= half ? m - half : m);
-        o = edge(m);
-      }
-    }
+    if (NS == 2 && (kWrap || s == (right ? 0 : 1)) && r.lane == (right ? 31 : 0)) o = t[NS - 1 - s];
+    if (!kWrap && s == (right ? NS - 1 : 0) && r.lane == (right ? r.last_lane() : 0)) o = e;
     w[s] = right ? make_float2(v[s].y, o) : make_float2(o, v[s].x);
   }
 }
@@ -606,9 +611,11 @@ __host__ __device__ constexpr size_t zero_rows_floats(int nx) {
 // cells (b - shift) / diag, black cells from their red neighbours (the
 // arithmetic of k_rb_zero_f32v), bc = mean over the 8 children of
 // b - shift - A x, in one pass over b (HBM: read b, write the packed black
-// cells and bc; the red cells are b / diag and enter no later sweep). The
-// residual is off times the neighbour sum in the red cells and zero in the
-// black ones.
+// cells and bc; the red cells are b / diag and enter no later sweep). In exact
+// arithmetic the residual is off times the neighbour sum in the red cells and
+// zero in the black ones; inv = 1 / diag in FP32 leaves a common relative error
+// of up to 3e-8 in every x, which adds (1 - diag inv) diag x to every residual
+// (off times slack x): small, but the coarse levels would not average it out.
 //
 // Layout as in k_rbgs_rows. Step i reads stage i (b of march plane i + 1),
 // publishes its red cells, forms the black cells of plane i (all rows: the edge
@@ -622,7 +629,7 @@ __host__ __device__ constexpr size_t zero_rows_floats(int nx) {
 template <int NS, int WPR, int NXT>
 __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
     k_zr_rows(const __grid_constant__ RowMaps mb, float* __restrict__ xb, float* __restrict__ bc,
-              const double* __restrict__ bshift, int nx_, int ny, int nz, int zc, float inv, float off,
+              const double* __restrict__ bshift, int nx_, int ny, int nz, int zc, float inv, float off, float slack,
               int* __restrict__ err, unsigned wait_limit) {
   constexpr int TY = kRowsTY, R = kZeroRing, XROWS = TY + 4, BROWS = TY + 2;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), w = warp / WPR;
@@ -639,7 +646,7 @@ __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
   const int k0 = blockIdx.y * zc, k1 = min(k0 + zc, nz);  // even
   const bool down = blockIdx.y & 1;
   const float2 msh = dup2(bshift ? -(float)(*bshift) : -0.f), off2 = dup2(off), inv2 = dup2(inv);
-  const float2 off8 = dup2(off * 0.125f);
+  const float2 off8 = dup2(off * 0.125f), slack2 = dup2(slack);
   const bool interior = w >= 1 && w <= TY;
   const int y = y0 - 1 + w;
   const bool odd_row = y & 1;
@@ -754,7 +761,7 @@ __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
         // march order visits a plane pair (2K, 2K + 1) upwards or downwards, its first plane at odd i
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
-          const float2 p = add2(add2(n[s], add2(u[s], d[s])), add2(xm2[s], x0[s]));
+          const float2 p = fma2(slack2, add2(rm[s], xm1[s]), add2(add2(n[s], add2(u[s], d[s])), add2(xm2[s], x0[s])));
           acc[s] = P0 == 1 ? p : add2(acc[s], p);
         }
         if (P0 == 0) {
@@ -872,10 +879,21 @@ void sweep_rows_go(dim3 g, cudaStream_t s, const RowMaps& mx, const RowMaps& mb,
 // Calls f with the kernel shape of rows of nx cells (see rows_sweep_ok).
 template <typename F>
 void with_row_shape(int nx, F&& f) {
+  constexpr std::integral_constant<int, 0> any{};
+  constexpr std::integral_constant<int, 1> one{};
+  constexpr std::integral_constant<int, 2> two{};
   if (nx == 128)
-    f(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{}, std::integral_constant<int, 128>{});
+    f(one, one, std::integral_constant<int, 128>{});
+  else if (nx == 256)
+    f(two, one, std::integral_constant<int, 256>{});
+  else if (nx == 512)
+    f(two, two, std::integral_constant<int, 512>{});
+  else if (nx < 128)
+    f(one, one, any);
+  else if (nx < 256)
+    f(two, one, any);
   else
-    f(std::integral_constant<int, 2>{}, std::integral_constant<int, 1>{}, std::integral_constant<int, 256>{});
+    f(two, two, any);
 }
 
 // The row sweep of x (in: SweepIn; xc the coarse field of the fused prolongation) into xout.
@@ -903,15 +921,15 @@ int clamp_zc(int zc, int nz, bool even) {
 }  // namespace
 
 bool rows_sweep_ok(Dims d) {
-  return (d.nx == 128 || d.nx == 256) && d.ny % kRowsTY == 0 && d.ny >= kRowsTY && d.nz % 2 == 0 && d.nz >= 4;
+  return d.nx % 32 == 0 && d.nx <= 512 && d.ny % kRowsTY == 0 && d.ny >= kRowsTY && d.nz % 2 == 0 && d.nz >= 4;
 }
 
 int rows_sweep_default_zc(Dims d) {
-  // about one wave of two resident CTAs per SM; an even number of planes, as
-  // the sweep with the prolongation fused needs, so that both kernels split
-  // a level into the same CTAs (and per-CTA partial sums)
+  // about one wave of two resident CTAs per SM (one with two warps per row); an
+  // even number of planes, as the sweep with the prolongation fused needs, so
+  // that both kernels split a level into the same CTAs (and per-CTA partial sums)
   const int cols = d.ny / kRowsTY;
-  int chunks = (2 * 152) / cols;
+  int chunks = ((d.nx > 256 ? 1 : 2) * 152) / cols;
   chunks = chunks < 1 ? 1 : chunks;
   int zc = (d.nz + chunks - 1) / chunks;
   zc += zc & 1;
@@ -950,6 +968,7 @@ void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, 
   zc = clamp_zc(zc, d.nz, true);
   const RowMaps mb = row_maps(b, d.nx, d.ny, d.nz, kRowsTY, 2);
   dim3 g(d.ny / kRowsTY, (d.nz + zc - 1) / zc);
+  const float inv = (float)(1.0 / st.diag), slack = (float)((1.0 - st.diag * (double)inv) * st.diag / st.off);
   with_row_shape(d.nx, [&](auto ns, auto wpr, auto nxt) {
     constexpr int NS = ns.value, WPR = wpr.value, NXT = nxt.value;
     const size_t sm = 4 * zero_rows_floats(d.nx) + 8 * kZeroRing;
@@ -957,8 +976,7 @@ void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, 
     ensure_smem_attr((const void*)k_zr_rows<NS, WPR, NXT>,
                      (int)(4 * zero_rows_floats(NXT ? NXT : 128 * NS * WPR) + 8 * kZeroRing), attr);
     k_zr_rows<NS, WPR, NXT><<<g, kRowsThreads<WPR>, sm, s>>>(
-        mb, xb, bc, bshift, d.nx, d.ny, d.nz, zc, (float)(1.0 / st.diag), (float)st.off, wait_error_flag(),
-        wait_limit());
+        mb, xb, bc, bshift, d.nx, d.ny, d.nz, zc, inv, (float)st.off, slack, wait_error_flag(), wait_limit());
   });
 }
 
