@@ -720,7 +720,7 @@ size_t ensure_krylov(ibrd_grid g, size_t n, int restart) {
 
 // w (= V[j+1]) <- w - sum_{i<=j} h_i v_i, the projections h written into
 // H[:, j], h_{j+1,j} (the norm of w after) into H[j+1, j], ||w||^2 before into
-// S_TMP and h_{j+1,j}^2 into S_SQ; then V[j+1] is the new basis vector. Stored
+// S_TMP, h_{j+1,j}^2 into S_SQ, and the Givens step of column j. Stored
 // basis vectors need not have norm 1: V[i] = v_i / vsc[i], vsc[i] its inverse
 // norm, and every projection and coefficient carries that factor. Classical
 // Gram-Schmidt. Without a second pass (eta <= 0) the pass that subtracts the
@@ -729,36 +729,55 @@ size_t ensure_krylov(ibrd_grid g, size_t n, int restart) {
 // pass, fixes h_{j+1,j} and vsc[j+1] (no separate normalisation pass). With the
 // DGKS second pass (threshold eta, decided on the device, its kernels
 // returning at once when it is not needed) the vector is normalised after it.
-// Without the second pass and with at most kDotGroup - 1 basis vectors the
-// reductions of both passes, the norm bookkeeping and the Givens step of
-// column j run in the last CTA of the multi-dot and multi-axpy launches;
-// returns true when the Givens step is done.
+// The reductions, the norm bookkeeping, the decision and the Givens step run in
+// the last CTA of the multi-dot and multi-axpy launches (groups of kDotGroup
+// vectors) or in the normalising pass: no launch of their own.
 template <typename E>
-bool orthogonalize(ibrd_grid g, int j, size_t n, size_t ld, int ldh, double eta) {
+void orthogonalize(ibrd_grid g, int j, size_t n, size_t ld, int ldh, double eta) {
   E* V = reinterpret_cast<E*>(g->V);
   E* w = V + (size_t)(j + 1) * ld;
   double* hcol = g->H + (size_t)j * ldh;
   double* vs = g->vsc;
   double* sc = g->scal;
   const int nb = j + 1;  // basis vectors V[0..j]
-  if (eta <= 0.0 && nb + 1 <= kDotGroup) {
-    DotTail dt;
-    dt.ticket = g->ticket;
-    dt.out = hcol;
-    dt.scale = vs;
-    dt.nscale = nb;
-    dt.nb = nb;
-    dt.ww = sc + S_TMP;
-    dt.hhat = sc + S_HHAT;
-    dt.hinv = sc + S_HINV;
-    launch_multidot(V, ld, nb + 1, w, n, g->partial, g->s, nullptr, &dt);
-    AxpyTail at;
-    at.ticket = g->ticket;
+  const bool second = eta > 0.0;
+  // projections onto `cnt` vectors from V[0] on into out, the first nb of them scaled
+  auto dots = [&](int cnt, double* out, const double* gate, bool estimate) {
+    for (int g0 = 0; g0 < cnt; g0 += kDotGroup) {
+      const int m = std::min(kDotGroup, cnt - g0);
+      DotTail dt;
+      dt.ticket = g->ticket;
+      dt.out = out + g0;
+      dt.scale = vs + g0;
+      dt.nscale = std::max(0, std::min(m, nb - g0));
+      if (estimate && g0 + m >= cnt) {
+        dt.nb = nb;
+        dt.h = out;
+        dt.ww = sc + S_TMP;
+        dt.hhat = sc + S_HHAT;
+        dt.hinv = sc + S_HINV;
+      }
+      launch_multidot(V + (size_t)g0 * ld, ld, m, w, n, g->partial, g->s, gate, &dt);
+    }
+  };
+  // w -= sum coef_i V[i] / vsc; the last group's tail does `at`'s work
+  auto subtract = [&](const double* coef, const double* gate, const double* post, const AxpyTail& at) {
+    for (int g0 = 0; g0 < nb; g0 += kDotGroup) {
+      const int m = std::min(kDotGroup, nb - g0);
+      const bool last = g0 + m >= nb;
+      launch_multi_axpy(w, V + (size_t)g0 * ld, ld, m, coef + g0, -1.0, n, last ? g->partial : nullptr, g->s, gate,
+                        vs + g0, last ? post : nullptr, last ? &at : nullptr);
+    }
+  };
+  dots(nb + 1, hcol, nullptr, !second);  // the last is <w, w>, unscaled
+  AxpyTail at;
+  at.ticket = g->ticket;
+  at.sq = sc + S_SQ;
+  if (!second) {
     at.rho2 = sc + S_RHO2;
     at.hhat = sc + S_HHAT;
     at.hsub = hcol + nb;
     at.vscale = vs + nb;
-    at.sq = sc + S_SQ;
     at.H = g->H;
     at.ldh = ldh;
     at.j = j;
@@ -766,53 +785,23 @@ bool orthogonalize(ibrd_grid g, int j, size_t n, size_t ld, int ldh, double eta)
     at.sn = g->sn;
     at.gvec = g->gvec;
     at.res = sc + S_RES;
-    launch_multi_axpy(w, V, ld, nb, hcol, -1.0, n, g->partial, g->s, nullptr, vs, sc + S_HINV, &at);
-    return true;
+    subtract(hcol, nullptr, sc + S_HINV, at);
+    return;
   }
-  // pass 1: dots of V[0..j+1] (the last is <w, w>, unscaled)
-  for (int g0 = 0; g0 < nb + 1; g0 += kDotGroup) {
-    const int m = std::min(kDotGroup, nb + 1 - g0);
-    launch_multidot(V + (size_t)g0 * ld, ld, m, w, n, g->partial, g->s);
-    launch_reduce_partials(g->partial, m, hcol + g0, g->s, nullptr, vs + g0, std::max(0, std::min(m, nb - g0)));
-  }
-  if (eta <= 0.0) {
-    launch_gs_norm_estimate(hcol, nb, sc + S_TMP, sc + S_HHAT, sc + S_HINV, g->s);
-    for (int g0 = 0; g0 < nb; g0 += kDotGroup) {
-      const int m = std::min(kDotGroup, nb - g0);
-      const bool last = g0 + m >= nb;
-      launch_multi_axpy(w, V + (size_t)g0 * ld, ld, m, hcol + g0, -1.0, n, last ? g->partial : nullptr, g->s,
-                        nullptr, vs + g0, last ? sc + S_HINV : nullptr);
-    }
-    launch_reduce_partials(g->partial, 1, sc + S_RHO2, g->s);
-    launch_gs_norm_fix(sc + S_RHO2, sc + S_HHAT, hcol + nb, vs + nb, sc + S_SQ, g->s);
-    return false;
-  }
-  IBRD_CUDA(cudaMemcpyAsync(sc + S_TMP, hcol + nb, sizeof(double), cudaMemcpyDeviceToDevice, g->s));
-  for (int g0 = 0; g0 < nb; g0 += kDotGroup) {
-    const int m = std::min(kDotGroup, nb - g0);
-    const bool last = g0 + m >= nb;
-    launch_multi_axpy(w, V + (size_t)g0 * ld, ld, m, hcol + g0, -1.0, n, last ? g->partial : nullptr, g->s,
-                      nullptr, vs + g0);
-  }
-  launch_reduce_partials(g->partial, 1, sc + S_SQ, g->s);
+  AxpyTail first = at;
+  first.flag = sc + S_RFLAG;
+  first.count = sc + S_RCOUNT;
+  first.eta = eta;
+  first.before = hcol + nb;
+  first.ww = sc + S_TMP;
+  subtract(hcol, nullptr, nullptr, first);
   const double* gate = sc + S_RFLAG;
-  launch_reorth_flag(sc + S_TMP, sc + S_SQ, eta, sc + S_RFLAG, sc + S_RCOUNT, g->s);
-  for (int g0 = 0; g0 < nb; g0 += kDotGroup) {
-    const int m = std::min(kDotGroup, nb - g0);
-    launch_multidot(V + (size_t)g0 * ld, ld, m, w, n, g->partial, g->s, gate);
-    launch_reduce_partials(g->partial, m, g->hb2 + g0, g->s, gate, vs + g0, m);
-  }
-  for (int g0 = 0; g0 < nb; g0 += kDotGroup) {
-    const int m = std::min(kDotGroup, nb - g0);
-    const bool last = g0 + m >= nb;
-    launch_multi_axpy(w, V + (size_t)g0 * ld, ld, m, g->hb2 + g0, -1.0, n, last ? g->partial : nullptr, g->s,
-                      gate, vs + g0);
-  }
-  launch_reduce_partials(g->partial, 1, sc + S_SQ, g->s, gate);
-  launch_vec_add_small(hcol, g->hb2, nb, g->s, gate);
-  launch_gs_norm_unit(sc + S_SQ, hcol + nb, vs + nb, g->s);
-  launch_scale_by_inv<E>(w, w, n, hcol + nb, 1.0, g->s);
-  return false;
+  dots(nb, g->hb2, gate, false);
+  at.add = g->hb2;
+  at.nadd = nb;
+  at.hcol = hcol;
+  subtract(g->hb2, gate, nullptr, at);
+  launch_gs_finish<E>(w, n, sc + S_SQ, hcol + nb, vs + nb, g->H, ldh, j, g->cs, g->sn, g->gvec, sc + S_RES, g->s);
 }
 
 struct SolveResult {
@@ -911,8 +900,7 @@ SolveResult fgmres(ibrd_grid g, LinOp<E>& op, const E* b, E* x, size_t n, const 
       E* w = V + (size_t)(j + 1) * ld;
       run_precond<E>(g, op, j, vj, zj, o.graphs != 0);
       op.apply(zj, w);
-      if (!orthogonalize<E>(g, j, n, ld, ldh, o.reorth_eta))
-        launch_givens(g->H, ldh, j, g->cs, g->sn, g->gvec, g->scal + S_RES, g->s);
+      orthogonalize<E>(g, j, n, ld, ldh, o.reorth_eta);
       // one host read per iteration: residual estimate and the norms
       IBRD_CUDA(cudaMemcpyAsync(g->host, g->scal, sizeof(double) * (S_WAIT + 1), cudaMemcpyDeviceToHost, g->s));
       IBRD_CUDA(cudaStreamSynchronize(g->s));
@@ -1405,8 +1393,7 @@ void capture_refine(ibrd_grid g, LinOp<double>& op64, LinOp<float>& op32, const 
               SG.inner_per_app = g->inner - ia;
             }
             op32.apply(zj, w);
-            if (!orthogonalize<float>(g, j, n, ld, ldh, o.reorth_eta))
-              launch_givens(g->H, ldh, j, g->cs, g->sn, g->gvec, sc + S_RES, g->s);
+            orthogonalize<float>(g, j, n, ld, ldh, o.reorth_eta);
             k_g_it_ctrl<<<1, 32, 0, g->s>>>(st, sc, g->ghist, j, m, j + 1 < m ? hs.h[j + 1] : hs.h[j], h_k);
             SG.l_it[j] = mark() - a0 + 1;
           });

@@ -9,6 +9,7 @@
 // bound by HBM and keep one read of each input and one write per output.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -100,9 +101,18 @@ __global__ void __launch_bounds__(256) k_absmax_bits(const double* __restrict__ 
     const unsigned long long a = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
     m = a > m ? a : m;
   };
-  if (vec) {  // 16-byte aligned: pairs, then the odd last entry
-    for (size_t i = t; i < n / 2; i += stride) {
-      const double2 v = reinterpret_cast<const double2*>(x)[i];
+  if (vec) {  // 16-byte aligned: pairs, two in flight, then the odd last entry
+    const double2* x2 = reinterpret_cast<const double2*>(x);
+    size_t i = t;
+    for (; i + stride < n / 2; i += 2 * stride) {
+      const double2 v = x2[i], w = x2[i + stride];
+      take(v.x);
+      take(v.y);
+      take(w.x);
+      take(w.y);
+    }
+    if (i < n / 2) {
+      const double2 v = x2[i];
       take(v.x);
       take(v.y);
     }
@@ -668,20 +678,50 @@ __device__ void fin_tail(const double* partial, const FinTail& t) {
   if (threadIdx.x == 0) *t.ticket = 0u;
 }
 
-// Sum of x: each thread folds 8-element runs (FP32 inputs summed in FP32 within
-// a run, then in FP64) from a grid-stride loop with 4 independent runs in flight.
+// Sum of x. 16-byte vectors, four in flight per thread (vec; the last n % V
+// entries one by one): FP32 values are summed in FP32 over runs of 8 and the
+// runs in FP64 (two FP64 instructions per run, hidden behind the loads). 19 us
+// for a 256^3 FP32 field (67 MB) and 84 us at 512^3 (0.94 of the copy bandwidth);
+// 28 and 156 us with scalar loads and runs of 4.
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict__ x, size_t n,
+__global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict__ x, size_t n, int vec,
                                                              double* __restrict__ partial, FinTail tail) {
   double acc = 0.0;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  size_t i = t;
-  for (; i + 3 * stride < n; i += 4 * stride) {
-    const T a0 = x[i], a1 = x[i + stride], a2 = x[i + 2 * stride], a3 = x[i + 3 * stride];
-    acc += (double)((a0 + a1) + (a2 + a3));
+  size_t done = 0;
+  if (vec) {
+    if constexpr (sizeof(T) == 4) {
+      const size_t n4 = n >> 2;
+      auto at = [&](size_t i) { return reinterpret_cast<const float4*>(x)[i]; };
+      auto run = [](float4 v) { return (v.x + v.y) + (v.z + v.w); };
+      size_t i = t;
+      for (; i + 3 * stride < n4; i += 4 * stride) {
+        const float4 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
+        acc += (double)(run(a) + run(b));
+        acc += (double)(run(c) + run(d));
+      }
+      for (; i < n4; i += stride) acc += (double)run(at(i));
+      done = 4 * n4;
+    } else {
+      const size_t n2 = n >> 1;
+      auto at = [&](size_t i) { return reinterpret_cast<const double2*>(x)[i]; };
+      double acc1 = 0.0;
+      size_t i = t;
+      for (; i + 3 * stride < n2; i += 4 * stride) {
+        const double2 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
+        acc += (a.x + a.y) + (b.x + b.y);
+        acc1 += (c.x + c.y) + (d.x + d.y);
+      }
+      for (; i < n2; i += stride) {
+        const double2 a = at(i);
+        acc += a.x + a.y;
+      }
+      acc += acc1;
+      done = 2 * n2;
+    }
   }
-  for (; i < n; i += stride) acc += (double)x[i];
+  for (size_t i = done + t; i < n; i += stride) acc += (double)x[i];
   acc = block_sum(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
   if (tail.ticket) fin_tail(partial, tail);
@@ -711,7 +751,20 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_partial(const E* __restrict
     const double s = block_sum_f(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
   } else {
-    double acc = 0.0;
+    double acc = 0.0, acc1 = 0.0;
+    if (vec) {
+      const size_t n2 = n >> 1, t = i;
+      const double2 *x2 = reinterpret_cast<const double2*>(x), *y2 = reinterpret_cast<const double2*>(y);
+      size_t v = t;
+      for (; v + stride < n2; v += 2 * stride) {
+        const double2 a = x2[v], b = y2[v], c = x2[v + stride], d = y2[v + stride];
+        acc = fma(a.x, b.x, fma(a.y, b.y, acc));
+        acc1 = fma(c.x, d.x, fma(c.y, d.y, acc1));
+      }
+      if (v < n2) acc = fma(x2[v].x, y2[v].x, fma(x2[v].y, y2[v].y, acc));
+      acc += acc1;
+      i = 2 * n2 + t;
+    }
     for (; i < n; i += stride) acc = fma(x[i], y[i], acc);
     acc = block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
@@ -772,11 +825,33 @@ __global__ void k_nvec_affine(const double* __restrict__ in, double* __restrict_
   }
 }
 
+// 16-byte vectors, two in flight per thread (vec), the rest one by one: 17 us at
+// 256^3 FP32 and 153 us at 512^3 (1074 MB); 29 and 254 us with scalar accesses.
 template <typename T>
-__global__ void k_sub_scalar(T* __restrict__ x, size_t n, const double* __restrict__ m) {
+__global__ void __launch_bounds__(256) k_sub_scalar(T* __restrict__ x, size_t n, int vec, const double* __restrict__ m) {
   const T v = (T)(*m);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    x[i] -= v;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  size_t done = 0;
+  if (vec) {
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int W = 16 / sizeof(T);
+    V* xv = reinterpret_cast<V*>(x);
+    auto less = [&](V a) {
+      a.x -= v, a.y -= v;
+      if constexpr (W == 4) a.z -= v, a.w -= v;
+      return a;
+    };
+    const size_t nv = n / W;
+    size_t i = t;
+    for (; i + stride < nv; i += 2 * stride) {
+      const V a = xv[i], b = xv[i + stride];
+      xv[i] = less(a);
+      xv[i + stride] = less(b);
+    }
+    if (i < nv) xv[i] = less(xv[i]);
+    done = nv * W;
+  }
+  for (size_t i = done + t; i < n; i += stride) x[i] -= v;
 }
 
 // FP32 to FP32 with 16-byte aligned fields: 4-vectors.
@@ -904,15 +979,36 @@ __global__ void k_scale_by_inv(const E* __restrict__ x, E* __restrict__ y, size_
 
 // y = (float) x * sigma, with the sum of squares of y: per thread and across
 // a warp in FP32 (terms of one sign; a thread holds about a hundred of a
-// 256^3 field), across warps and blocks in FP64.
+// 256^3 field), across warps and blocks in FP64. vec: 16-byte aligned, four
+// values per thread and step, two steps in flight; 34 us at 256^3 (201 MB, 0.87 of
+// the copy bandwidth), 70 us with scalar loads.
 __global__ void __launch_bounds__(kRedThreads) k_convert_sq(const double* __restrict__ x, float* __restrict__ y,
-                                                            size_t n, float sigma, const double* __restrict__ sigma_dev,
+                                                            size_t n, int vec, float sigma,
+                                                            const double* __restrict__ sigma_dev,
                                                             double* __restrict__ partial, FinTail tail) {
   if (sigma_dev) sigma = (float)*sigma_dev;
   float acc = 0.f;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-#pragma unroll 4
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
+  const size_t stride = (size_t)gridDim.x * blockDim.x, t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  size_t done = 0;
+  if (vec) {
+    const size_t n4 = n >> 2;
+    auto put = [&](size_t i, double2 a, double2 b) {
+      const float4 v = make_float4(d2f_bits(a.x) * sigma, d2f_bits(a.y) * sigma, d2f_bits(b.x) * sigma,
+                                   d2f_bits(b.y) * sigma);
+      reinterpret_cast<float4*>(y)[i] = v;
+      acc = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, acc))));
+    };
+    const double2* x2 = reinterpret_cast<const double2*>(x);
+    size_t i = t;
+    for (; i + stride < n4; i += 2 * stride) {
+      const double2 a = x2[2 * i], b = x2[2 * i + 1], c = x2[2 * (i + stride)], d = x2[2 * (i + stride) + 1];
+      put(i, a, b);
+      put(i + stride, c, d);
+    }
+    if (i < n4) put(i, x2[2 * i], x2[2 * i + 1]);
+    done = 4 * n4;
+  }
+  for (size_t i = done + t; i < n; i += stride) {
     const float v = d2f_bits(x[i]) * sigma;
     y[i] = v;
     acc = fmaf(v, v, acc);
@@ -1093,12 +1189,13 @@ template <typename T>
 void launch_sum(const T* x, size_t n, double* partial, double* out, double scale, cudaStream_t s, unsigned* ticket) {
   FinTail t;
   if (ticket) t = FinTail{ticket, out, scale, nullptr, 1.0};
+  const int nb = red_blocks(n);
   prof_begin(P_DOT, s);
-  k_sum_partial<T><<<kRedBlocks, kRedThreads, 0, s>>>(x, n, partial, t);
+  k_sum_partial<T><<<nb, kRedThreads, 0, s>>>(x, n, aligned16(x), partial, t);
   prof_end(P_DOT, s, "sum_partial", 1.0 * sizeof(T) * n);
   if (ticket) return;
   prof_begin(P_REDUCE, s);
-  k_finalize<<<1, kRedThreads, 0, s>>>(partial, kRedBlocks, out, scale);
+  k_finalize<<<1, kRedThreads, 0, s>>>(partial, nb, out, scale);
   prof_end(P_REDUCE, s, "finalize");
 }
 
@@ -1113,19 +1210,20 @@ void launch_convert_sum(const X* x, T* y, size_t n, double* partial, double* out
                         cudaStream_t s, unsigned* ticket) {
   FinTail t;
   if (ticket) t = FinTail{ticket, out_in, 1.0, out_out, 1.0};
+  const int nb = red_blocks(n);
   prof_begin(P_VEC, s);
   if constexpr (sizeof(X) == 4 && sizeof(T) == 4) {
     if (aligned16(x) && aligned16(y))
-      k_copy_sum_f32v<<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, partial, partial + kRedBlocks, t);
+      k_copy_sum_f32v<<<nb, kRedThreads, 0, s>>>(x, y, n, partial, partial + nb, t);
     else
-      k_convert_sum<X, T><<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, partial, partial + kRedBlocks, t);
+      k_convert_sum<X, T><<<nb, kRedThreads, 0, s>>>(x, y, n, partial, partial + nb, t);
   } else {
-    k_convert_sum<X, T><<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, partial, partial + kRedBlocks, t);
+    k_convert_sum<X, T><<<nb, kRedThreads, 0, s>>>(x, y, n, partial, partial + nb, t);
   }
   prof_end(P_VEC, s, "convert_sum", (double)(sizeof(X) + sizeof(T)) * n);
   if (ticket) return;
-  launch_finalize(partial, kRedBlocks, out_in, 1.0, s);
-  launch_finalize(partial + kRedBlocks, kRedBlocks, out_out, 1.0, s);
+  launch_finalize(partial, nb, out_in, 1.0, s);
+  launch_finalize(partial + nb, nb, out_out, 1.0, s);
 }
 
 template <typename F>
@@ -1143,18 +1241,20 @@ void launch_dot(const E* x, const E* y, size_t n, double* partial, double* out, 
   FinTail t;
   if (ticket) t = FinTail{ticket, out, scale, nullptr, 1.0};
   prof_begin(P_DOT, s);
-  k_dot_partial<E><<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, partial, aligned16(x) && aligned16(y), t);
+  const int nb = red_blocks(n);
+  k_dot_partial<E><<<nb, kRedThreads, 0, s>>>(x, y, n, partial, aligned16(x) && aligned16(y), t);
   prof_end(P_DOT, s, "dot_partial", 2.0 * sizeof(E) * n);
   if (ticket) return;
   prof_begin(P_REDUCE, s);
-  k_finalize<<<1, kRedThreads, 0, s>>>(partial, kRedBlocks, out, scale);
+  k_finalize<<<1, kRedThreads, 0, s>>>(partial, nb, out, scale);
   prof_end(P_REDUCE, s, "finalize");
 }
 
 template <typename T>
 void launch_sub_scalar(T* x, size_t n, const double* mean, cudaStream_t s) {
   prof_begin(P_VEC, s);
-  k_sub_scalar<T><<<stream_blocks(n, 256), 256, 0, s>>>(x, n, mean);
+  const int vec = aligned16(x);
+  k_sub_scalar<T><<<stream_blocks(vec ? n / (16 / sizeof(T)) + 1 : n, 256), 256, 0, s>>>(x, n, vec, mean);
   prof_end(P_VEC, s, "sub_scalar", 2.0 * sizeof(T) * n);
 }
 
@@ -1194,10 +1294,11 @@ void launch_convert_sq(const double* x, float* y, size_t n, double sigma, double
   FinTail t;
   if (ticket) t = FinTail{ticket, out, 1.0, nullptr, 1.0};
   prof_begin(P_VEC, s);
-  k_convert_sq<<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, (float)sigma, nullptr, partial, t);
+  const int nb = red_blocks(n);
+  k_convert_sq<<<nb, kRedThreads, 0, s>>>(x, y, n, aligned16(x) && aligned16(y), (float)sigma, nullptr, partial, t);
   prof_end(P_VEC, s, "convert_sq", 12.0 * n);
   if (ticket) return;
-  launch_finalize(partial, kRedBlocks, out, 1.0, s);
+  launch_finalize(partial, nb, out, 1.0, s);
 }
 
 void launch_convert_sq(const double* x, float* y, size_t n, const double* sigma_dev, double* partial, double* out,
@@ -1205,10 +1306,11 @@ void launch_convert_sq(const double* x, float* y, size_t n, const double* sigma_
   FinTail t;
   if (ticket) t = FinTail{ticket, out, 1.0, nullptr, 1.0};
   prof_begin(P_VEC, s);
-  k_convert_sq<<<kRedBlocks, kRedThreads, 0, s>>>(x, y, n, 1.f, sigma_dev, partial, t);
+  const int nb = red_blocks(n);
+  k_convert_sq<<<nb, kRedThreads, 0, s>>>(x, y, n, aligned16(x) && aligned16(y), 1.f, sigma_dev, partial, t);
   prof_end(P_VEC, s, "convert_sq", 12.0 * n);
   if (ticket) return;
-  launch_finalize(partial, kRedBlocks, out, 1.0, s);
+  launch_finalize(partial, nb, out, 1.0, s);
 }
 
 void launch_add_scaled(double a, const float* d, double* x, size_t n, cudaStream_t s) {

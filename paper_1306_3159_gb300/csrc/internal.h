@@ -125,9 +125,16 @@ __device__ __forceinline__ double f2d_bits(float f) {
 #endif
 
 // ---------------------------------------------------------------- reductions
-// Deterministic two-stage reductions use a fixed grid of kRedBlocks blocks.
+// Deterministic two-stage reductions of n entries run red_blocks(n) blocks: one
+// per 512 entries (2 per thread) up to kRedBlocks. A block costs its block-wide
+// sums and one partial for the last block to read whether it holds entries or
+// not; entries a thread takes one after the other cost a memory latency each.
 constexpr int kRedBlocks = 608;   // 4 x 152 SMs
 constexpr int kRedThreads = 256;
+inline int red_blocks(size_t n) {
+  const size_t b = (n + 511) / 512;
+  return b < 1 ? 1 : (b > (size_t)kRedBlocks ? kRedBlocks : (int)b);
+}
 
 // ---------------------------------------------------------------- grid kernels
 // All launchers enqueue on `s` and check the launch.
@@ -356,35 +363,55 @@ constexpr int kDotGroup = 8;
 // after the others (it takes the last ticket of a per-handle counter after a
 // fence; no CTA waits for another), so that an FGMRES iteration needs no
 // separate single-CTA launches for it. ticket: 0 between uses, reset by that
-// CTA. The arithmetic is that of the separate kernels it replaces.
+// CTA.
 struct DotTail {
   unsigned* ticket = nullptr;
   double* out = nullptr;  // out[g] = the sum of partial row g, times scale[g] for g < nscale
   const double* scale = nullptr;
   int nscale = 0;
-  int nb = 0;  // > 0: then launch_gs_norm_estimate's work on out[0..nb]
+  // nb > 0: the norm of the vector after one classical Gram-Schmidt pass,
+  // estimated before the pass from its projections h[0..nb) and h[nb] = ||w||^2:
+  // ||w||^2 - sum h_i^2, floored at 1e-8 ||w||^2 (where cancellation leaves no
+  // digits the floor only changes the stored vector's scale, which the exact
+  // norm taken in the same pass then records); writes ||w||^2, the estimate and
+  // its reciprocal (0 for w = 0)
+  int nb = 0;
+  const double* h = nullptr;
   double *ww = nullptr, *hhat = nullptr, *hinv = nullptr;
 };
 struct AxpyTail {
   unsigned* ticket = nullptr;
-  double* rho2 = nullptr;  // the sum of the squares partials, then launch_gs_norm_fix's work
+  double* sq = nullptr;  // the sum of the squares partials (with hhat: h_{j+1,j}^2)
+  // hhat: the pass stored the new basis vector scaled by 1 / *hhat; the sum is
+  // its squared norm *rho2, h_{j+1,j} = hhat sqrt(rho2) (the norm of the unscaled
+  // vector) goes to *hsub, the stored vector's inverse norm to *vscale, and the
+  // Givens step of column j follows
+  double* rho2 = nullptr;
   const double* hhat = nullptr;
-  double *hsub = nullptr, *vscale = nullptr, *sq = nullptr;
-  double* H = nullptr;  // then launch_givens' work on column j
+  double *hsub = nullptr, *vscale = nullptr;
+  double* H = nullptr;
   int ldh = 0, j = 0;
   double *cs = nullptr, *sn = nullptr, *gvec = nullptr, *res = nullptr;
+  // flag: whether a second Gram-Schmidt pass is needed (eta >= 1 or sq < eta^2
+  // *before, the squared norm before the pass, which also goes to *ww); counted
+  // in *count
+  double* flag = nullptr;
+  double* count = nullptr;
+  double eta = 0.0;
+  const double* before = nullptr;
+  double* ww = nullptr;
+  // add: a second pass' projections add[0..nadd) join hcol[0..nadd)
+  const double* add = nullptr;
+  int nadd = 0;
+  double* hcol = nullptr;
 };
-// partial[g * kRedBlocks + blk] for g < nvec (nvec <= kDotGroup)
+// partial[g * kRedBlocks + blk], blk < red_blocks(n), for g < nvec (nvec <= kDotGroup)
 // gate (nullable device scalar): the kernel does nothing when *gate == 0.
 void launch_multidot(const double* V, size_t ldv, int nvec, const double* w, size_t n, double* partial,
                      cudaStream_t s, const double* gate = nullptr, const DotTail* tail = nullptr);
 // FP32 basis: V and w 16-byte aligned, ldv % 4 == 0.
 void launch_multidot(const float* V, size_t ldv, int nvec, const float* w, size_t n, double* partial,
                      cudaStream_t s, const double* gate = nullptr, const DotTail* tail = nullptr);
-// out[g] = sum_blk partial[g*kRedBlocks + blk]   (g < nvec), times scale[g]
-// for g < nscale when scale is given
-void launch_reduce_partials(const double* partial, int nvec, double* out, cudaStream_t s,
-                            const double* gate = nullptr, const double* scale = nullptr, int nscale = 0);
 // w += sign * sum_g coef[g] cscale[g] V[g] (cscale optional), then w *= *post
 // (optional); optional partial sums of squares of the new w.
 void launch_multi_axpy(double* w, const double* V, size_t ldv, int nvec, const double* coef, double sign,
@@ -396,26 +423,14 @@ void launch_multi_axpy(float* w, const float* V, size_t ldv, int nvec, const dou
                        double* partial_sq, cudaStream_t s, const double* gate = nullptr,
                        const double* cscale = nullptr, const double* post = nullptr,
                        const AxpyTail* tail = nullptr);
-// Gram-Schmidt norm bookkeeping (one-warp kernels): the estimate of the norm
-// after one pass from the projections h[0..nb) and h[nb] = ||w||^2 (writes
-// ||w||^2, the estimate and its reciprocal); after a pass that stored the
-// vector scaled by the estimate's reciprocal, with squared norm *rho2:
-// h_{j+1,j}, the stored vector's inverse norm and h_{j+1,j}^2; for a vector
-// normalised exactly afterwards: h_{j+1,j} = sqrt(*sq) and scale 1.
-void launch_gs_norm_estimate(const double* h, int nb, double* ww, double* hhat, double* hinv, cudaStream_t s);
-void launch_gs_norm_fix(const double* rho2, const double* hhat, double* hsub, double* vscale, double* sq,
-                        cudaStream_t s);
-void launch_gs_norm_unit(const double* sq, double* hsub, double* vscale, cudaStream_t s);
-// Givens step j on column H[:, j] (ldh = restart + 1): rotations cs/sn,
-// residual vector gvec; writes |gvec[j+1]| to *res.
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* gvec, double* res,
-                   cudaStream_t s);
+// w, of squared norm *sq, normalised in place; *hsub = its norm, *vscale = 1, and
+// the Givens step j on column H[:, j] (ldh = restart + 1): rotations cs/sn,
+// residual vector gvec; |gvec[j+1]| into *res.
+template <typename E>
+void launch_gs_finish(E* w, size_t n, const double* sq, double* hsub, double* vscale, double* H, int ldh, int j,
+                      double* cs, double* sn, double* gvec, double* res, cudaStream_t s);
 // Back substitution y = R^{-1} g for the leading k x k block.
 void launch_backsolve(const double* H, int ldh, int k, const double* gvec, double* y, cudaStream_t s);
-// Combine two dot results: h[i] += h2[i] for i < n (device).
-void launch_vec_add_small(double* h, const double* h2, int n, cudaStream_t s, const double* gate = nullptr);
-// *flag = (eta >= 1 || *sq < eta^2 *ww); *count += *flag
-void launch_reorth_flag(const double* ww, const double* sq, double eta, double* flag, double* count, cudaStream_t s);
 // *dst = sqrt(*src)
 void launch_sqrt_scalar(const double* src, double* dst, cudaStream_t s);
 

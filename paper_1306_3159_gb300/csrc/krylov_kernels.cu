@@ -9,47 +9,55 @@
 // The Hessenberg matrix, Givens rotations and the least-squares update stay on
 // the device; the host only reads the residual estimate.
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 
 namespace ibrd {
 namespace {
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block sum, result valid in thread 0 of the block. Safe to call repeatedly.
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double sw[32];
-  v = warp_sum(v);
+// Block sums of NV per-thread values at once (kRedThreads threads); thread g <
+// NV of the block returns value g's sum. Within a warp a butterfly halves the
+// values a lane carries while it folds the lanes: 9 additions per lane for eight
+// values instead of 40 (FP64's pipe is about 64 times narrower than FP32's, and
+// the eight separate trees were half of a launch over 0.9 M entries); the warps'
+// totals are added in FP64 by warp 0. FP32 values are folded within a warp in FP32.
+template <int NV, typename A>
+__device__ __forceinline__ double block_sums(const A (&in)[NV]) {
+  constexpr int P = NV <= 1 ? 1 : (NV <= 2 ? 2 : (NV <= 4 ? 4 : 8));
+  constexpr int B = P == 1 ? 0 : (P == 2 ? 1 : (P == 4 ? 2 : 3));  // log2
+  constexpr int NW = kRedThreads / 32;
+  __shared__ double sw[NW][P];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sw[wid] = v;
-  __syncthreads();
-  v = (threadIdx.x < (blockDim.x >> 5)) ? sw[threadIdx.x] : 0.0;
-  if (wid == 0) v = warp_sum(v);
-  return v;
-}
-
-// Block sum of FP32 per-thread values, result valid in thread 0: each warp
-// adds its 32 values in FP32, the block adds the warps' totals in FP64. The
-// FP64 pipe of GB300 is about 64 times narrower than the FP32 one, so five
-// FP64 shuffle levels over every warp of every block cost microseconds at the
-// end of a reduction over a 256^3 field; this keeps them to one warp per block.
-__device__ __forceinline__ double block_sum_f(float v) {
-  __shared__ double sw[32];
+  A v[P];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int g = 0; g < P; ++g) v[g] = g < NV ? in[g] : (A)0;
+  int off = 16;
+#pragma unroll
+  for (int half = P / 2; half > 0; half >>= 1, off >>= 1) {
+    const bool hi = lane & off;
+#pragma unroll
+    for (int k = 0; k < half; ++k) {
+      const A keep = hi ? v[k + half] : v[k], give = hi ? v[k] : v[k + half];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+    }
+  }
+#pragma unroll
+  for (int o = 16 >> B; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  __syncthreads();  // the previous call's sums have been read
+  if ((lane & ((32 >> B) - 1)) == 0) sw[wid][lane >> (5 - B)] = (double)v[0];
   __syncthreads();
-  if (lane == 0) sw[wid] = (double)v;
-  __syncthreads();
-  double d = (threadIdx.x < (blockDim.x >> 5)) ? sw[threadIdx.x] : 0.0;
-  if (wid == 0) d = warp_sum(d);
-  return d;
+  double sum = 0.0;
+  if (wid == 0) {
+    // lane 4 g + q adds warps q and q + 4 of value g, then the four lanes fold
+    const int g = lane >> 2, q = lane & 3;
+    static_assert(NW == 8, "two warps per lane");
+    double t = g < P ? sw[q][g] + sw[q + 4][g] : 0.0;
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    sum = __shfl_sync(0xffffffffu, t, (lane & 7) * 4);
+  }
+  return sum;
 }
 
 // Givens step j on column H[:, j] (ldh = restart + 1): the earlier rotations
@@ -107,10 +115,12 @@ __device__ void gs_norm_fix_one(double rho2, const double* __restrict__ hhat, do
   *sq = hs * hs;
 }
 
-// Whether this CTA is the last of the grid to finish; thread 0 wrote the
-// CTA's partials before the call. A fence orders them before the ticket.
+// Whether this CTA is the last of the grid to finish; threads of it wrote the
+// CTA's partials before the call (each with a fence of its own, and thread 0's
+// here, before the ticket).
 __device__ __forceinline__ bool last_cta(unsigned* ticket) {
   __shared__ bool last;
+  __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
@@ -120,59 +130,90 @@ __device__ __forceinline__ bool last_cta(unsigned* ticket) {
   return last;
 }
 
-// Sum of partial row g (kRedBlocks values) in the order of k_reduce_partials;
-// valid in thread 0. Read through L2: other CTAs wrote the row.
-__device__ __forceinline__ double partial_row_sum(const double* partial, int g) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) acc += __ldcg(partial + (size_t)g * kRedBlocks + i);
-  return block_sum(acc);
+// Sums over the grid's blocks of NV partial rows; thread g < NV returns row
+// g's. Read through L2: other CTAs wrote the rows.
+template <int NV>
+__device__ __forceinline__ double partial_sums(const double* partial) {
+  double acc[NV];
+#pragma unroll
+  for (int g = 0; g < NV; ++g) acc[g] = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+#pragma unroll
+    for (int g = 0; g < NV; ++g) acc[g] += __ldcg(partial + (size_t)g * kRedBlocks + i);
+  }
+  return block_sums<NV>(acc);
 }
 
 // Tail of a multi-dot launch (last CTA): the rows' sums into tail.out, then
 // the norm estimate.
-__device__ void dot_tail(const double* partial, int nv, const DotTail& tail) {
-  for (int g = 0; g < nv; ++g) {
-    const double v = partial_row_sum(partial, g);
-    if (threadIdx.x == 0) tail.out[g] = (g < tail.nscale) ? v * tail.scale[g] : v;
-  }
+template <int NV>
+__device__ void dot_tail(const double* partial, const DotTail& tail) {
+  const double v = partial_sums<NV>(partial);
+  const int g = threadIdx.x;
+  if (g < NV) tail.out[g] = (g < tail.nscale) ? v * tail.scale[g] : v;
   __syncthreads();
-  if (tail.nb > 0 && threadIdx.x < 32) gs_norm_estimate_warp(tail.out, tail.nb, tail.ww, tail.hhat, tail.hinv);
+  if (tail.nb > 0 && threadIdx.x < 32) gs_norm_estimate_warp(tail.h, tail.nb, tail.ww, tail.hhat, tail.hinv);
   if (threadIdx.x == 0) *tail.ticket = 0u;
 }
 
-// Tail of a multi-axpy launch (last CTA): the squares' sum, the norm fix and
-// the Givens step.
+// Tail of a multi-axpy launch (last CTA): the squares' sum, then what the
+// pass's place in the orthogonalisation asks for (AxpyTail).
 __device__ void axpy_tail(const double* partial_sq, const AxpyTail& tail) {
-  const double v = partial_row_sum(partial_sq, 0);
-  if (threadIdx.x == 0) {
+  const double v = partial_sums<1>(partial_sq);
+  if (tail.add)
+    for (int i = threadIdx.x; i < tail.nadd; i += blockDim.x) tail.hcol[i] += tail.add[i];
+  if (threadIdx.x != 0) return;
+  if (tail.hhat) {
     *tail.rho2 = v;
     gs_norm_fix_one(v, tail.hhat, tail.hsub, tail.vscale, tail.sq);
     givens_step(tail.H, tail.ldh, tail.j, tail.cs, tail.sn, tail.gvec, tail.res);
-    *tail.ticket = 0u;
+  } else {
+    *tail.sq = v;
+    if (tail.flag) {
+      const double f = (tail.eta >= 1.0 || v < tail.eta * tail.eta * *tail.before) ? 1.0 : 0.0;
+      *tail.ww = *tail.before;
+      *tail.flag = f;
+      *tail.count += f;
+    }
   }
+  *tail.ticket = 0u;
 }
 
-// FP64 vectors: one FMA per element and vector.// FP64 vectors: one FMA per element and vector.
+// FP64 vectors: one FMA per element and vector; pairs (vec: 16-byte aligned, ldv even).
 template <int NV>
 __global__ void __launch_bounds__(kRedThreads) k_multidot(const double* __restrict__ V, size_t ldv,
-                                                          const double* __restrict__ w, size_t n,
+                                                          const double* __restrict__ w, size_t n, int vec,
                                                           double* __restrict__ partial, const double* __restrict__ gate,
                                                           DotTail tail) {
   if (gate && *gate == 0.0) return;
   double acc[NV];
 #pragma unroll
   for (int g = 0; g < NV; ++g) acc[g] = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  size_t done = 0;
+  if (vec) {
+    const size_t n2 = n >> 1;
+    for (size_t i = t; i < n2; i += stride) {
+      const double2 wi = reinterpret_cast<const double2*>(w)[i];
+#pragma unroll
+      for (int g = 0; g < NV; ++g) {
+        const double2 v = reinterpret_cast<const double2*>(V + g * ldv)[i];
+        acc[g] = fma(v.x, wi.x, fma(v.y, wi.y, acc[g]));
+      }
+    }
+    done = 2 * n2;
+  }
+  for (size_t i = done + t; i < n; i += stride) {
     const double wi = w[i];
 #pragma unroll
     for (int g = 0; g < NV; ++g) acc[g] = fma(V[g * ldv + i], wi, acc[g]);
   }
-#pragma unroll
-  for (int g = 0; g < NV; ++g) {
-    const double s = block_sum(acc[g]);
-    if (threadIdx.x == 0) partial[g * kRedBlocks + blockIdx.x] = s;
+  const double s = block_sums<NV>(acc);
+  if (threadIdx.x < NV) {
+    partial[threadIdx.x * kRedBlocks + blockIdx.x] = s;
+    __threadfence();
   }
-  if (tail.ticket && last_cta(tail.ticket)) dot_tail(partial, NV, tail);
+  if (tail.ticket && last_cta(tail.ticket)) dot_tail<NV>(partial, tail);
 }
 
 // FP32 vectors (16-byte aligned, ldv % 4 == 0): 4-vectors, FP32 products
@@ -202,50 +243,60 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot_f32(const float* __res
 #pragma unroll
     for (int g = 0; g < NV; ++g) acc[g] = fmaf(V[g * ldv + i], wi, acc[g]);
   }
-#pragma unroll
-  for (int g = 0; g < NV; ++g) {
-    const double s = block_sum_f(acc[g]);
-    if (threadIdx.x == 0) partial[g * kRedBlocks + blockIdx.x] = s;
+  const double s = block_sums<NV>(acc);
+  if (threadIdx.x < NV) {
+    partial[threadIdx.x * kRedBlocks + blockIdx.x] = s;
+    __threadfence();
   }
-  if (tail.ticket && last_cta(tail.ticket)) dot_tail(partial, NV, tail);
-}
-
-__global__ void __launch_bounds__(kRedThreads) k_reduce_partials(const double* __restrict__ partial,
-                                                                 double* __restrict__ out,
-                                                                 const double* __restrict__ gate,
-                                                                 const double* __restrict__ scale, int nscale) {
-  if (gate && *gate == 0.0) return;
-  // blockIdx.x = vector g
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) acc += partial[blockIdx.x * kRedBlocks + i];
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) out[blockIdx.x] = ((int)blockIdx.x < nscale) ? acc * scale[blockIdx.x] : acc;
+  if (tail.ticket && last_cta(tail.ticket)) dot_tail<NV>(partial, tail);
 }
 
 template <int NV, bool SQ>
 __global__ void __launch_bounds__(kRedThreads) k_multi_axpy(double* __restrict__ w, const double* __restrict__ V,
                                                             size_t ldv, const double* __restrict__ coef,
-                                                            double sign, size_t n, double* __restrict__ partial_sq,
+                                                            double sign, size_t n, int vec,
+                                                            double* __restrict__ partial_sq,
                                                             const double* __restrict__ gate,
                                                             const double* __restrict__ cscale,
                                                             const double* __restrict__ post, AxpyTail tail) {
   if (gate && *gate == 0.0) return;
+  __shared__ double cs[NV];
+  if (threadIdx.x < NV) cs[threadIdx.x] = sign * coef[threadIdx.x] * (cscale ? cscale[threadIdx.x] : 1.0);
+  __syncthreads();
   double c[NV];
 #pragma unroll
-  for (int g = 0; g < NV; ++g) c[g] = sign * coef[g] * (cscale ? cscale[g] : 1.0);
+  for (int g = 0; g < NV; ++g) c[g] = cs[g];
   const double ps = post ? *post : 1.0;
-  double sq = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  double sq[1] = {0.0};
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  size_t done = 0;
+  if (vec) {
+    const size_t n2 = n >> 1;
+    for (size_t i = t; i < n2; i += stride) {
+      double2 wi = reinterpret_cast<const double2*>(w)[i];
+#pragma unroll
+      for (int g = 0; g < NV; ++g) {
+        const double2 v = reinterpret_cast<const double2*>(V + g * ldv)[i];
+        wi.x = fma(c[g], v.x, wi.x);
+        wi.y = fma(c[g], v.y, wi.y);
+      }
+      if (post) wi.x *= ps, wi.y *= ps;
+      reinterpret_cast<double2*>(w)[i] = wi;
+      if (SQ) sq[0] = fma(wi.x, wi.x, fma(wi.y, wi.y, sq[0]));
+    }
+    done = 2 * n2;
+  }
+  for (size_t i = done + t; i < n; i += stride) {
     double wi = w[i];
 #pragma unroll
     for (int g = 0; g < NV; ++g) wi = fma(c[g], V[g * ldv + i], wi);
     if (post) wi *= ps;
     w[i] = wi;
-    if (SQ) sq = fma(wi, wi, sq);
+    if (SQ) sq[0] = fma(wi, wi, sq[0]);
   }
   if (SQ) {
-    sq = block_sum(sq);
-    if (threadIdx.x == 0) partial_sq[blockIdx.x] = sq;
+    const double v = block_sums<1>(sq);
+    if (threadIdx.x == 0) partial_sq[blockIdx.x] = v;
     if (tail.ticket && last_cta(tail.ticket)) axpy_tail(partial_sq, tail);
   }
 }
@@ -261,11 +312,17 @@ __global__ void __launch_bounds__(kRedThreads) k_multi_axpy_f32(float* __restric
                                                                 const double* __restrict__ cscale,
                                                                 const double* __restrict__ post, AxpyTail tail) {
   if (gate && *gate == 0.0) return;
+  // the coefficients once per CTA: three FP64 instructions per vector in every
+  // thread would hold the FP64 pipe for several microseconds
+  __shared__ float cs[NV + 1];
+  if (threadIdx.x < NV) cs[threadIdx.x] = (float)(sign * coef[threadIdx.x] * (cscale ? cscale[threadIdx.x] : 1.0));
+  if (threadIdx.x == NV) cs[NV] = post ? (float)*post : 1.f;
+  __syncthreads();
   float c[NV];
 #pragma unroll
-  for (int g = 0; g < NV; ++g) c[g] = (float)(sign * coef[g] * (cscale ? cscale[g] : 1.0));
+  for (int g = 0; g < NV; ++g) c[g] = cs[g];
   const bool scaled = post != nullptr;
-  const float ps = scaled ? (float)*post : 1.f;
+  const float ps = cs[NV];
   float sq = 0.f;
   const size_t n4 = n >> 2, stride = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -293,16 +350,11 @@ __global__ void __launch_bounds__(kRedThreads) k_multi_axpy_f32(float* __restric
     if (SQ) sq = fmaf(wi, wi, sq);
   }
   if (SQ) {
-    const double b = block_sum_f(sq);
+    const float sqs[1] = {sq};
+    const double b = block_sums<1>(sqs);
     if (threadIdx.x == 0) partial_sq[blockIdx.x] = b;
     if (tail.ticket && last_cta(tail.ticket)) axpy_tail(partial_sq, tail);
   }
-}
-
-__global__ void k_givens(double* __restrict__ H, int ldh, int j, double* __restrict__ cs, double* __restrict__ sn,
-                         double* __restrict__ gvec, double* __restrict__ res) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  givens_step(H, ldh, j, cs, sn, gvec, res);
 }
 
 __global__ void k_backsolve(const double* __restrict__ H, int ldh, int k, const double* __restrict__ gvec,
@@ -316,53 +368,46 @@ __global__ void k_backsolve(const double* __restrict__ H, int ldh, int k, const 
   }
 }
 
-__global__ void k_vec_add_small(double* __restrict__ h, const double* __restrict__ h2, int n,
-                                const double* __restrict__ gate) {
-  if (gate && *gate == 0.0) return;
-  const int i = threadIdx.x;
-  if (i < n) h[i] += h2[i];
-}
-
-// flag = 1 when the Gram-Schmidt second pass is needed: ||w'||^2 < eta^2 ||w||^2
-// (or eta >= 1); counts the passes in *count.
-__global__ void k_reorth_flag(const double* __restrict__ ww, const double* __restrict__ sq, double eta,
-                              double* __restrict__ flag, double* __restrict__ count) {
-  if (threadIdx.x != 0) return;
-  const double f = (eta >= 1.0 || *sq < eta * eta * *ww) ? 1.0 : 0.0;
-  *flag = f;
-  *count += f;
-}
-
 __global__ void k_sqrt_scalar(const double* __restrict__ src, double* __restrict__ dst) {
   if (threadIdx.x == 0) *dst = sqrt(fmax(*src, 0.0));
 }
 
-// The norm of w after one classical Gram-Schmidt pass, estimated before the
-// pass from its projections h[0..nb) and h[nb] = ||w||^2: ||w||^2 - sum h_i^2,
-// floored at 1e-8 ||w||^2 (where cancellation leaves no digits the floor only
-// changes the stored vector's scale, which the exact norm taken in the same
-// pass then records). Writes ||w||^2, the estimate and its reciprocal (0 for
-// w = 0). One warp.
-__global__ void k_gs_norm_estimate(const double* __restrict__ h, int nb, double* __restrict__ ww,
-                                   double* __restrict__ hhat, double* __restrict__ hinv) {
-  gs_norm_estimate_warp(h, nb, ww, hhat, hinv);
-}
-
-// After the pass wrote the new basis vector scaled by 1 / hhat with squared
-// norm rho2: the Hessenberg entry h_{j+1,j} = hhat sqrt(rho2) (the norm of the
-// unscaled vector), the stored vector's inverse norm, and h_{j+1,j}^2 into sq.
-__global__ void k_gs_norm_fix(const double* __restrict__ rho2, const double* __restrict__ hhat,
-                              double* __restrict__ hsub, double* __restrict__ vscale, double* __restrict__ sq) {
-  if (threadIdx.x == 0) gs_norm_fix_one(*rho2, hhat, hsub, vscale, sq);
-}
-
-// h_{j+1,j} = sqrt(sq), for a basis vector that is then normalised exactly
-// (stored scale 1).
-__global__ void k_gs_norm_unit(const double* __restrict__ sq, double* __restrict__ hsub,
-                               double* __restrict__ vscale) {
-  if (threadIdx.x != 0) return;
-  *hsub = sqrt(fmax(*sq, 0.0));
-  *vscale = 1.0;
+// The end of an orthogonalisation with a possible second pass: w, of squared
+// norm *sq, normalised (scale 1 kept in *vscale), h_{j+1,j} = its norm, and the
+// Givens step of column j (block 0; no other block reads what it writes).
+template <typename E>
+__global__ void __launch_bounds__(256) k_gs_finish(E* __restrict__ w, size_t n, int vec, const double* __restrict__ sq,
+                                                   double* __restrict__ hsub, double* __restrict__ vscale,
+                                                   double* __restrict__ H, int ldh, int j, double* __restrict__ cs,
+                                                   double* __restrict__ sn, double* __restrict__ gvec,
+                                                   double* __restrict__ res) {
+  __shared__ double norm, inv;
+  if (threadIdx.x == 0) {  // once per CTA: an FP64 root and quotient in every thread would take longer than the pass
+    norm = sqrt(fmax(*sq, 0.0));
+    inv = 1.0 / norm;
+  }
+  __syncthreads();
+  const E f = (E)inv;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  size_t done = 0;
+  if (vec) {
+    constexpr int W = 16 / sizeof(E);
+    using V = typename std::conditional<sizeof(E) == 4, float4, double2>::type;
+    V* wv = reinterpret_cast<V*>(w);
+    for (size_t i = t; i < n / W; i += stride) {
+      V a = wv[i];
+      a.x *= f, a.y *= f;
+      if constexpr (W == 4) a.z *= f, a.w *= f;
+      wv[i] = a;
+    }
+    done = n / W * W;
+  }
+  for (size_t i = done + t; i < n; i += stride) w[i] *= f;
+  if (t == 0) {
+    *hsub = norm;
+    *vscale = 1.0;
+    givens_step(H, ldh, j, cs, sn, gvec, res);
+  }
 }
 
 // ---------------------------------------------------------------- small GMRES
@@ -734,10 +779,11 @@ void launch_multidot(const double* V, size_t ldv, int nvec, const double* w, siz
                      cudaStream_t s, const double* gate, const DotTail* tail) {
   const DotTail t = tail ? *tail : DotTail{};
   if (nvec < 1 || nvec > kDotGroup) return;
+  const int nb = red_blocks(n), vec = ldv % 2 == 0 && aligned16(V) && aligned16(w);
   prof_begin(P_DOT, s);
   switch (nvec) {
 #define IBRD_CASE(k) \
-  case k: k_multidot<k><<<kRedBlocks, kRedThreads, 0, s>>>(V, ldv, w, n, partial, gate, t); break;
+  case k: k_multidot<k><<<nb, kRedThreads, 0, s>>>(V, ldv, w, n, vec, partial, gate, t); break;
     IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
 #undef IBRD_CASE
     default: return;
@@ -750,10 +796,11 @@ void launch_multidot(const float* V, size_t ldv, int nvec, const float* w, size_
   const DotTail t = tail ? *tail : DotTail{};
   if (nvec < 1 || nvec > kDotGroup) return;
   if (ldv % 4 != 0 || !aligned16(V) || !aligned16(w)) throw CudaError{cudaErrorMisalignedAddress, "multidot_f32"};
+  const int nb = red_blocks(n);
   prof_begin(P_DOT, s);
   switch (nvec) {
 #define IBRD_CASE(k) \
-  case k: k_multidot_f32<k><<<kRedBlocks, kRedThreads, 0, s>>>(V, ldv, w, n, partial, gate, t); break;
+  case k: k_multidot_f32<k><<<nb, kRedThreads, 0, s>>>(V, ldv, w, n, partial, gate, t); break;
     IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
 #undef IBRD_CASE
     default: return;
@@ -761,45 +808,33 @@ void launch_multidot(const float* V, size_t ldv, int nvec, const float* w, size_
   prof_end(P_DOT, s, "multidot_f32", 4.0 * (nvec + 1) * n);
 }
 
-void launch_reduce_partials(const double* partial, int nvec, double* out, cudaStream_t s, const double* gate,
-                            const double* scale, int nscale) {
-  if (nvec <= 0) return;
-  prof_begin(P_REDUCE, s);
-  k_reduce_partials<<<nvec, kRedThreads, 0, s>>>(partial, out, gate, scale, scale ? nscale : 0);
-  prof_end(P_REDUCE, s, "reduce_partials");
+template <typename E>
+void launch_gs_finish(E* w, size_t n, const double* sq, double* hsub, double* vscale, double* H, int ldh, int j,
+                      double* cs, double* sn, double* gvec, double* res, cudaStream_t s) {
+  const int vec = aligned16(w);
+  const int blocks = red_blocks(n);
+  prof_begin(P_VEC, s);
+  k_gs_finish<E><<<blocks, 256, 0, s>>>(w, n, vec, sq, hsub, vscale, H, ldh, j, cs, sn, gvec, res);
+  prof_end(P_VEC, s, "gs_finish", 2.0 * sizeof(E) * n);
 }
-
-void launch_gs_norm_estimate(const double* h, int nb, double* ww, double* hhat, double* hinv, cudaStream_t s) {
-  prof_begin(P_SMALL, s);
-  k_gs_norm_estimate<<<1, 32, 0, s>>>(h, nb, ww, hhat, hinv);
-  prof_end(P_SMALL, s, "gs_norm_estimate");
-}
-
-void launch_gs_norm_fix(const double* rho2, const double* hhat, double* hsub, double* vscale, double* sq,
-                        cudaStream_t s) {
-  prof_begin(P_SMALL, s);
-  k_gs_norm_fix<<<1, 32, 0, s>>>(rho2, hhat, hsub, vscale, sq);
-  prof_end(P_SMALL, s, "gs_norm_fix");
-}
-
-void launch_gs_norm_unit(const double* sq, double* hsub, double* vscale, cudaStream_t s) {
-  prof_begin(P_SMALL, s);
-  k_gs_norm_unit<<<1, 32, 0, s>>>(sq, hsub, vscale);
-  prof_end(P_SMALL, s, "gs_norm_unit");
-}
+template void launch_gs_finish<double>(double*, size_t, const double*, double*, double*, double*, int, int, double*,
+                                       double*, double*, double*, cudaStream_t);
+template void launch_gs_finish<float>(float*, size_t, const double*, double*, double*, double*, int, int, double*,
+                                      double*, double*, double*, cudaStream_t);
 
 void launch_multi_axpy(double* w, const double* V, size_t ldv, int nvec, const double* coef, double sign, size_t n,
                        double* partial_sq, cudaStream_t s, const double* gate, const double* cscale,
                        const double* post, const AxpyTail* tail) {
   const AxpyTail t = (tail && partial_sq) ? *tail : AxpyTail{};
   if (nvec < 1 || nvec > kDotGroup) return;
+  const int nb = red_blocks(n), vec = ldv % 2 == 0 && aligned16(V) && aligned16(w);
   prof_begin(P_AXPY, s);
   if (partial_sq) {
     switch (nvec) {
 #define IBRD_CASE(k)                                                                                     \
   case k:                                                                                                \
-    k_multi_axpy<k, true><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, partial_sq, gate, \
-                                                             cscale, post, t);                           \
+    k_multi_axpy<k, true><<<nb, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, vec, partial_sq, gate,    \
+                                                     cscale, post, t);                                   \
     break;
       IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
 #undef IBRD_CASE
@@ -809,8 +844,8 @@ void launch_multi_axpy(double* w, const double* V, size_t ldv, int nvec, const d
     switch (nvec) {
 #define IBRD_CASE(k)                                                                                      \
   case k:                                                                                                 \
-    k_multi_axpy<k, false><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, nullptr, gate,   \
-                                                              cscale, post, t);                           \
+    k_multi_axpy<k, false><<<nb, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, vec, nullptr, gate,       \
+                                                      cscale, post, t);                                   \
     break;
       IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
 #undef IBRD_CASE
@@ -826,12 +861,13 @@ void launch_multi_axpy(float* w, const float* V, size_t ldv, int nvec, const dou
   const AxpyTail t = (tail && partial_sq) ? *tail : AxpyTail{};
   if (nvec < 1 || nvec > kDotGroup) return;
   if (ldv % 4 != 0 || !aligned16(V) || !aligned16(w)) throw CudaError{cudaErrorMisalignedAddress, "multi_axpy_f32"};
+  const int nb = red_blocks(n);
   prof_begin(P_AXPY, s);
   if (partial_sq) {
     switch (nvec) {
 #define IBRD_CASE(k)                                                                                           \
   case k:                                                                                                      \
-    k_multi_axpy_f32<k, true><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, partial_sq, gate, \
+    k_multi_axpy_f32<k, true><<<nb, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, partial_sq, gate, \
                                                                  cscale, post, t);                           \
     break;
       IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
@@ -842,7 +878,7 @@ void launch_multi_axpy(float* w, const float* V, size_t ldv, int nvec, const dou
     switch (nvec) {
 #define IBRD_CASE(k)                                                                                            \
   case k:                                                                                                       \
-    k_multi_axpy_f32<k, false><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, nullptr, gate, \
+    k_multi_axpy_f32<k, false><<<nb, kRedThreads, 0, s>>>(w, V, ldv, coef, sign, n, nullptr, gate, \
                                                                   cscale, post, t);                          \
     break;
       IBRD_CASE(1) IBRD_CASE(2) IBRD_CASE(3) IBRD_CASE(4) IBRD_CASE(5) IBRD_CASE(6) IBRD_CASE(7) IBRD_CASE(8)
@@ -853,28 +889,10 @@ void launch_multi_axpy(float* w, const float* V, size_t ldv, int nvec, const dou
   prof_end(P_AXPY, s, "multi_axpy_f32", 4.0 * (nvec + 2) * n);
 }
 
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* gvec, double* res, cudaStream_t s) {
-  prof_begin(P_SMALL, s);
-  k_givens<<<1, 32, 0, s>>>(H, ldh, j, cs, sn, gvec, res);
-  prof_end(P_SMALL, s, "givens");
-}
-
 void launch_backsolve(const double* H, int ldh, int k, const double* gvec, double* y, cudaStream_t s) {
   prof_begin(P_SMALL, s);
   k_backsolve<<<1, 32, 0, s>>>(H, ldh, k, gvec, y);
   prof_end(P_SMALL, s, "backsolve");
-}
-
-void launch_vec_add_small(double* h, const double* h2, int n, cudaStream_t s, const double* gate) {
-  prof_begin(P_SMALL, s);
-  k_vec_add_small<<<1, 64, 0, s>>>(h, h2, n, gate);
-  prof_end(P_SMALL, s, "vec_add_small");
-}
-
-void launch_reorth_flag(const double* ww, const double* sq, double eta, double* flag, double* count, cudaStream_t s) {
-  prof_begin(P_SMALL, s);
-  k_reorth_flag<<<1, 32, 0, s>>>(ww, sq, eta, flag, count);
-  prof_end(P_SMALL, s, "reorth_flag");
 }
 
 void launch_sqrt_scalar(const double* src, double* dst, cudaStream_t s) {
