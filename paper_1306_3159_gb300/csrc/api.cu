@@ -209,6 +209,7 @@ struct ibrd_grid_s {
   cudaStream_t s = nullptr;
   std::vector<Level> levels;
   int small_from = 0;           // first level handled by the single-CTA coarse V-cycle
+  int cluster_from = 1 << 30;   // first level of the FP64 V-cycle handled by the cluster kernel
   int exact32 = -1;             // FP32 V-cycles: level solved exactly by the Hartley transform (-1: none)
   Hier<double> h64;
   Hier<float> h32;
@@ -395,6 +396,7 @@ CoarseLevels small_levels(ibrd_grid g, int l, double shift) {
     cl.lgx[i] = lg(li.d.nx);
     cl.lgy[i] = lg(li.d.ny);
     cl.diag[i] = si.diag;
+    cl.inv[i] = 1.0 / si.diag;
     cl.offd[i] = si.off;
     tot += (int)li.d.n();
   }
@@ -424,8 +426,16 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
     launch_coarse_solve<T>(coarse_table<T>(g, shift), b, x, lv.d, g->s);
     return 0;
   }
-  // the coarse end of the hierarchy runs in one CTA out of shared memory
-  // (FP64 V-cycles, and FP32 ones on grids without an exact level)
+  // the coarse end of the hierarchy: FP64 by a thread block cluster, else
+  // (small hierarchies, and FP32 ones on grids without an exact level) in one
+  // CTA out of shared memory
+  if constexpr (sizeof(T) == 8) {
+    if (l >= g->cluster_from) {
+      launch_vcycle_cluster(small_levels(g, l, shift), b, x, bshift, coarse_table<double>(g, shift), zero, nu1, nu2,
+                            g->s);
+      return 0;
+    }
+  }
   if (l >= g->small_from && !(sizeof(T) == 4 && g->exact32 >= 0)) {
     const CoarseLevels cl = small_levels(g, l, shift);
     launch_vcycle_small<T>(cl, b, x, bshift, coarse_table<T>(g, shift), zero, nu1, nu2, g->s);
@@ -2804,6 +2814,11 @@ ibrd_status ibrd_grid_create(ibrd_grid* out, int nx, int ny, int nz, double h, d
       break;
     }
   ibrd_status st = guarded(g, "ibrd_grid_create", [&]() {
+    // FP64: the first level from which the cluster kernel takes the rest
+    const int L = (int)g->levels.size();
+    for (int l = std::max(0, L - kMaxSmallLevels); l < L && g->cluster_from > L; ++l)
+      if (vcycle_cluster_ok(small_levels(g, l, g->alpha))) g->cluster_from = l;
+    if (g->cluster_from > g->small_from) g->cluster_from = 1 << 30;
     g->scal = dalloc<double>(S_COUNT);
     g->partial = dalloc<double>((size_t)kRedBlocks * kDotGroup);
     g->dflag = dalloc<int>(4);

@@ -220,12 +220,18 @@ struct CoarseLevels {
   int off[kMaxSmallLevels];       // first cell of each level in the packed arrays
   int lgx[kMaxSmallLevels], lgy[kMaxSmallLevels];  // log2 of nx, ny, or -1 if not a power of 2
   double diag[kMaxSmallLevels], offd[kMaxSmallLevels];
+  double inv[kMaxSmallLevels];    // 1 / diag: an FP64 quotient in every thread of a CTA would hold its SM for microseconds
 };
 // Whole V-cycle over the levels in lv (the last one solved exactly with the
 // circulant table) in one CTA: x = V(b - bshift), from zero or from x.
 template <typename T>
 void launch_vcycle_small(const CoarseLevels& lv, const T* b, T* x, const double* bshift, const T* table, bool zero,
                          int nu1, int nu2, cudaStream_t s);
+// The same in FP64 by a thread block cluster that shares the larger levels
+// (coarse_cluster.cu); vcycle_cluster_ok: whether these levels fit it.
+bool vcycle_cluster_ok(const CoarseLevels& lv);
+void launch_vcycle_cluster(const CoarseLevels& lv, const double* b, double* x, const double* bshift,
+                           const double* table, bool zero, int nu1, int nu2, cudaStream_t s);
 // bc = mean over 8 children of (b - shift - A x) on the fine grid d.
 template <typename T>
 void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, Dims d, Stencil st,

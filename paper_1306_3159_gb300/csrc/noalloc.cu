@@ -133,7 +133,7 @@ void na_level(const NaPlan& P, double* S, int l, const double* b, const double* 
     launch_coarse_solve<double>(table, b, x, lv.d, s);
     return;
   }
-  if (l >= P.small_from) {
+  if (L - l <= kMaxSmallLevels) {
     CoarseLevels cl{};
     cl.n = L - l;
     int tot = 0;
@@ -148,12 +148,19 @@ void na_level(const NaPlan& P, double* S, int l, const double* b, const double* 
       cl.lgx[i] = lg(li.d.nx);
       cl.lgy[i] = lg(li.d.ny);
       cl.diag[i] = si.diag;
+      cl.inv[i] = 1.0 / si.diag;
       cl.offd[i] = si.off;
       tot += (int)li.d.n();
     }
     cl.total = tot;
-    launch_vcycle_small<double>(cl, b, x, bshift, table, zero, 2, 2, s);
-    return;
+    if (vcycle_cluster_ok(cl)) {
+      launch_vcycle_cluster(cl, b, x, bshift, table, zero, 2, 2, s);
+      return;
+    }
+    if (l >= P.small_from) {
+      launch_vcycle_small<double>(cl, b, x, bshift, table, zero, 2, 2, s);
+      return;
+    }
   }
   double* cur = x;
   double* oth = S + P.y[l];

@@ -18,6 +18,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "vcycle_small.h"
 
 namespace ibrd {
 namespace {
@@ -767,157 +768,23 @@ __global__ void __launch_bounds__(256) k_prolong8x2(const T* __restrict__ xc, T*
     }
 }
 
-// The coarse end of a V-cycle in ONE CTA: levels lv.first .. lv.n-1 (at most
-// a few thousand cells) live in shared memory (smem_raw, 2 lv.total values);
-// smoothing, residual restriction, the exact coarsest solve and prolongation
-// run with block-wide barriers between phases. Arithmetic matches the
-// multi-kernel levels.
-template <typename T>
-__device__ void vcycle_small_body(const CoarseLevels& lv, const T* __restrict__ bg, T* __restrict__ xg,
-                                  const double* __restrict__ bshift, const T* __restrict__ table, int zero, int nu1,
-                                  int nu2, unsigned char* smem_raw) {
-  T* X = reinterpret_cast<T*>(smem_raw);
-  T* B = X + lv.total;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const T sh = bshift ? (T)(*bshift) : (T)0;
-  {
-    const int n0 = lv.nx[0] * lv.ny[0] * lv.nz[0];
-    for (int c = tid; c < n0; c += nt) {
-      B[c] = bg[c] - sh;
-      X[c] = zero ? (T)0 : xg[c];
-    }
-    for (int c = n0 + tid; c < lv.total; c += nt) X[c] = (T)0;
-  }
-  __syncthreads();
-  // cell index -> (i, j, k); shifts when the level's nx, ny are powers of 2
-  auto decode = [&](int l, int c, int& i, int& j, int& k) {
-    const int lx = lv.lgx[l], ly = lv.lgy[l];
-    if (lx >= 0 && ly >= 0) {
-      i = c & (lv.nx[l] - 1);
-      j = (c >> lx) & (lv.ny[l] - 1);
-      k = c >> (lx + ly);
-    } else {
-      i = c % lv.nx[l];
-      j = (c / lv.nx[l]) % lv.ny[l];
-      k = c / (lv.nx[l] * lv.ny[l]);
-    }
-  };
-  // one red-black sweep on level l (all sides even): each half-sweep visits
-  // only the cells of its colour, enumerated as (i/2, j, k)
-  auto sweep = [&](int l) {
-    const int nx = lv.nx[l], ny = lv.ny[l], nz = lv.nz[l];
-    const int hx = nx >> 1, nh = hx * ny * nz, plane = nx * ny;
-    T* x = X + lv.off[l];
-    const T* b = B + lv.off[l];
-    const T inv = (T)(1.0 / lv.diag[l]), off = (T)lv.offd[l];
-    const int lx = lv.lgx[l], ly = lv.lgy[l];
-    const bool pow2 = lx >= 1 && ly >= 0;
-    for (int colour = 0; colour < 2; ++colour) {
-      for (int p = tid; p < nh; p += nt) {
-        int ih, j, k;
-        if (pow2) {
-          ih = p & (hx - 1);
-          j = (p >> (lx - 1)) & (ny - 1);
-          k = p >> (lx - 1 + ly);
-        } else {
-          ih = p % hx;
-          j = (p / hx) % ny;
-          k = p / (hx * ny);
-        }
-        const int i = 2 * ih + ((j + k + colour) & 1);
-        const int rowc = k * plane + j * nx;
-        const int c = rowc + i;
-        const int xw = rowc + (i == 0 ? nx - 1 : i - 1), xe = rowc + (i == nx - 1 ? 0 : i + 1);
-        const int ys = c + (j == 0 ? plane - nx : -nx), yn = c + (j == ny - 1 ? nx - plane : nx);
-        const int zd = c + (k == 0 ? plane * (nz - 1) : -plane), zu = c + (k == nz - 1 ? -plane * (nz - 1) : plane);
-        const T sum = ((x[xw] + x[xe]) + (x[ys] + x[yn])) + (x[zd] + x[zu]);
-        x[c] = (b[c] + off * sum) * inv;
-      }
-      __syncthreads();
-    }
-  };
-  const int last = lv.n - 1;
-  for (int l = 0; l < last; ++l) {
-    for (int sw = 0; sw < nu1; ++sw) sweep(l);
-    // residual restriction to level l+1
-    const int nx = lv.nx[l], ny = lv.ny[l], nz = lv.nz[l];
-    const int nxc = nx >> 1, nyc = ny >> 1, nc = nxc * nyc * (nz >> 1);
-    const T* x = X + lv.off[l];
-    const T* b = B + lv.off[l];
-    T* bc = B + lv.off[l + 1];
-    const T diag = (T)lv.diag[l], off = (T)lv.offd[l];
-    // one child per thread: entry e = 8 C + (dz, dy, dx) bits, so the 8
-    // children of a coarse cell sit in 8 neighbouring lanes and are summed
-    // by shuffles (the loop bound is a multiple of 32 so warps stay whole)
-    const int nf = 8 * nc, nround = (nf + 31) & ~31;
-    for (int e = tid; e < nround; e += nt) {
-      T r = 0;
-      if (e < nf) {
-        int I, J, K;
-        decode(l + 1, e >> 3, I, J, K);
-        const int i = 2 * I + (e & 1), j = 2 * J + ((e >> 1) & 1), k = 2 * K + (e >> 2 & 1);
-        const int c = (k * ny + j) * nx + i;
-        const T s = ((x[c - i + wrap(i - 1, nx)] + x[c - i + wrap(i + 1, nx)]) +
-                     (x[c + (wrap(j - 1, ny) - j) * nx] + x[c + (wrap(j + 1, ny) - j) * nx])) +
-                    (x[c + (wrap(k - 1, nz) - k) * nx * ny] + x[c + (wrap(k + 1, nz) - k) * nx * ny]);
-        r = b[c] - (diag * x[c] - off * s);
-      }
-      r += __shfl_xor_sync(0xffffffffu, r, 1);
-      r += __shfl_xor_sync(0xffffffffu, r, 2);
-      r += __shfl_xor_sync(0xffffffffu, r, 4);
-      if (e < nf && (e & 7) == 0) bc[e >> 3] = r * (T)0.125;
-    }
-    __syncthreads();
-  }
-  {
-    // exact coarsest solve with the circulant table
-    const int nx = lv.nx[last], ny = lv.ny[last], nz = lv.nz[last], n = nx * ny * nz;
-    T* x = X + lv.off[last];
-    const T* b = B + lv.off[last];
-    for (int t = tid; t < n; t += nt) {
-      const int ix = t % nx, iy = (t / nx) % ny, iz = t / (nx * ny);
-      T acc = 0;
-      for (int u = 0; u < n; ++u) {
-        const int jx = u % nx, jy = (u / nx) % ny, jz = u / (nx * ny);
-        const int dx = ix - jx + (ix < jx ? nx : 0), dy = iy - jy + (iy < jy ? ny : 0), dz = iz - jz + (iz < jz ? nz : 0);
-        acc += table[(dz * ny + dy) * nx + dx] * b[u];
-      }
-      x[t] = acc;
-    }
-    __syncthreads();
-  }
-  for (int l = last - 1; l >= 0; --l) {
-    const int nx = lv.nx[l], ny = lv.ny[l], nz = lv.nz[l], n = nx * ny * nz;
-    const int nxc = nx >> 1, nyc = ny >> 1, nzc = nz >> 1;
-    T* x = X + lv.off[l];
-    const T* xc = X + lv.off[l + 1];
-    for (int c = tid; c < n; c += nt) {
-      int i, j, k;
-      decode(l, c, i, j, k);
-      const int I = i >> 1, J = j >> 1, K = k >> 1;
-      const int I2 = (i & 1) ? wrap(I + 1, nxc) : wrap(I - 1, nxc);
-      const int J2 = (j & 1) ? wrap(J + 1, nyc) : wrap(J - 1, nyc);
-      const int K2 = (k & 1) ? wrap(K + 1, nzc) : wrap(K - 1, nzc);
-      auto e = [&](int kk, int jj, int ii) { return xc[(kk * nyc + jj) * nxc + ii]; };
-      // z, then y, then x (each axis scaled by 4)
-      auto zy = [&](int ii) {
-        return prolong_axis(prolong_axis(e(K, J, ii), e(K2, J, ii)), prolong_axis(e(K, J2, ii), e(K2, J2, ii)));
-      };
-      x[c] = prolong_add(x[c], prolong_axis(zy(I), zy(I2)));
-    }
-    __syncthreads();
-    for (int sw = 0; sw < nu2; ++sw) sweep(l);
-  }
-  const int n0 = lv.nx[0] * lv.ny[0] * lv.nz[0];
-  for (int c = tid; c < n0; c += nt) xg[c] = X[c];
-}
-
 template <typename T>
 __global__ void __launch_bounds__(1024) k_vcycle_small(CoarseLevels lv, const T* __restrict__ bg, T* __restrict__ xg,
                                                        const double* __restrict__ bshift, const T* __restrict__ table,
                                                        int zero, int nu1, int nu2) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  vcycle_small_body<T>(lv, bg, xg, bshift, table, zero, nu1, nu2, smem_raw);
+  T* X = reinterpret_cast<T*>(smem_raw);
+  T* B = X + lv.total;
+  const int tid = threadIdx.x, nt = blockDim.x, n0 = lv.nx[0] * lv.ny[0] * lv.nz[0];
+  const T sh = bshift ? (T)(*bshift) : (T)0;
+  for (int c = tid; c < n0; c += nt) {
+    B[c] = bg[c] - sh;
+    X[c] = zero ? (T)0 : xg[c];
+  }
+  for (int c = n0 + tid; c < lv.total; c += nt) X[c] = (T)0;
+  __syncthreads();
+  vcycle_small_levels<T>(lv, 0, X, B, table, nu1, nu2);
+  for (int c = tid; c < n0; c += nt) xg[c] = X[c];
 }
 
 }  // namespace
