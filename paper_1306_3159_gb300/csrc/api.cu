@@ -482,7 +482,7 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
       if (launch_rb_sweep<T>(cur, oth, b, bshift, lv.d, st, first, nullptr, 0, g->s) >= 0) std::swap(cur, oth);
       first = false;
     }
-    launch_resid_restrict<T>(cur, b, bshift, H.b[l + 1], lv.d, st, g->s);
+    launch_resid_restrict<T>(cur, b, bshift, H.b[l + 1], lv.d, st, nu1 > 0, g->s);
   }
   vcycle_level<T>(g, l + 1, H.b[l + 1], nullptr, H.x[l + 1], true, shift, nu1, nu2, nullptr);
   int sweep = 0;
@@ -504,13 +504,13 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
       prof_end(P_RBGS32, g->s, "unpack_zero", 10.0 * lv.d.n());
       std::swap(cur, oth);
     }
-    launch_prolong8<T>(H.x[l + 1], cur, lv.d, g->s);
+    launch_prolong8<T>(H.x[l + 1], cur, lv.d, nu2 > 0, g->s);
   }
   for (; sweep < nu2; ++sweep) {
     const bool last = (sweep == nu2 - 1);
     const int r = launch_rb_sweep<T>(cur, oth, b, bshift, lv.d, st, false, last ? part : nullptr, part_cap, g->s);
     if (r >= 0) std::swap(cur, oth);
-    np = last ? (r > 0 ? r : 0) : np;
+    np = last ? (r >= 0 ? r : -1 - r) : np;
   }
   if (cur != x) IBRD_CUDA(cudaMemcpyAsync(x, cur, sizeof(T) * lv.d.n(), cudaMemcpyDeviceToDevice, g->s));
   return np;

@@ -151,9 +151,9 @@ bool resid_fx_ok(Dims d, Stencil st);
 // *bshift (bshift nullable). On levels where the fused one-pass kernel
 // applies it reads xin and writes xout (xin != xout) and returns the number
 // of per-CTA partial sums of the new x written into part (0 when part is
-// null or holds fewer than the CTA count); on small levels it updates xin in
-// place with two half sweeps and returns -1. zero != 0 treats the incoming x
-// as 0.
+// null or holds fewer than the CTA count); on small levels, and in FP64 unless
+// a tiled shape was chosen, it updates xin in place with two half sweeps and
+// returns -1 minus that number. zero != 0 treats the incoming x as 0.
 template <typename T>
 int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dims d, Stencil st, bool zero,
                     double* part, int part_cap, cudaStream_t s);
@@ -233,8 +233,9 @@ bool vcycle_cluster_ok(const CoarseLevels& lv);
 void launch_vcycle_cluster(const CoarseLevels& lv, const double* b, double* x, const double* bshift,
                            const double* table, bool zero, int nu1, int nu2, cudaStream_t s);
 // bc = mean over 8 children of (b - shift - A x) on the fine grid d.
+// swept: x is the result of a sweep (its black cells have no residual).
 template <typename T>
-void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, Dims d, Stencil st,
+void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, Dims d, Stencil st, bool swept,
                            cudaStream_t s);
 // FP32 pre-smoothing of one sweep from x = 0 fused with the residual
 // restriction: x = sweep(0), bc = mean over 8 children of (b - shift - A x).
@@ -242,8 +243,9 @@ bool zero_restrict_ok(Dims d);
 void launch_zero_restrict(const float* b, const double* bshift, float* x, float* bc, Dims d, Stencil st,
                           cudaStream_t s);
 // x (fine, dims d) += trilinear cell-centred prolongation of xc (dims d/2).
+// sweep_follows: a red-black sweep of x comes next (it reads no red cells).
 template <typename T>
-void launch_prolong8(const T* xc, T* x, Dims d, cudaStream_t s);
+void launch_prolong8(const T* xc, T* x, Dims d, bool sweep_follows, cudaStream_t s);
 // The prolongation of xc added to xin fused with the red-black sweep that
 // follows it, on levels the row-resident FP32 sweep serves: writes the swept
 // field to xout (xin is left uncorrected) and returns the partial-sum count

@@ -171,9 +171,9 @@ void na_level(const NaPlan& P, double* S, int l, const double* b, const double* 
     if (launch_rb_sweep<double>(cur, oth, b, bshift, lv.d, st, first, nullptr, 0, s) >= 0) std::swap(cur, oth);
     first = false;
   }
-  launch_resid_restrict<double>(cur, b, bshift, bc, lv.d, st, s);
+  launch_resid_restrict<double>(cur, b, bshift, bc, lv.d, st, true, s);
   na_level(P, S, l + 1, bc, nullptr, xc, true, chi, shift, s);
-  launch_prolong8<double>(xc, cur, lv.d, s);
+  launch_prolong8<double>(xc, cur, lv.d, true, s);
   for (int sweep = 0; sweep < 2; ++sweep)
     if (launch_rb_sweep<double>(cur, oth, b, bshift, lv.d, st, false, nullptr, 0, s) >= 0) std::swap(cur, oth);
   if (cur != x) IBRD_CUDA(cudaMemcpyAsync(x, cur, sizeof(double) * lv.d.n(), cudaMemcpyDeviceToDevice, s));

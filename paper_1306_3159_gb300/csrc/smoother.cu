@@ -362,6 +362,145 @@ __global__ void __launch_bounds__(256) k_rb_half(const T* __restrict__ xr, T* __
   }
 }
 
+// FP64 half sweep on one colour, in place. GB300's FP64 pipe (two operations
+// per SM and clock) bounds every FP64 sweep, so this form counts operations: six
+// per cell instead of eight. A thread walks up a diagonal (i + 1, j + 1), whose
+// cells have one colour: the sum of the east and north neighbours of one is that
+// of the south and west neighbours of the next. b and its shift enter by one
+// FMA, the neighbours by another. In place and by colour there is no halo to
+// compute twice, which cost the fused one-pass kernel 1.3 times the operations
+// here (with FP32 it pays, in bytes): a sweep of 128^3 (both colours) takes
+// 45 us with the FP64 pipe 76 % busy, the fused kernel 58; of 96^3 21 and 28, of
+// 64^3 12 and 14; a first sweep from zero of 128^3 30 and 58.
+// From zero (zero) a red cell is b / diag and no neighbour is read. part: each
+// CTA's sum of the new x of both colours (the black half sweep, whose cells each
+// take their east neighbour along).
+__global__ void __launch_bounds__(256) k_rb_half_f64(double* __restrict__ x, const double* __restrict__ b,
+                                                     const double* __restrict__ bshift, int nx, int ny, int nz, int yc,
+                                                     double inv, double offinv, int colour, int zero,
+                                                     double* __restrict__ part) {
+  const int np = nx >> 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, k = t / np, p = t - k * np;
+  const int j0 = blockIdx.y * yc, j1 = min(j0 + yc, ny);
+  double acc = 0.0;
+  if (k < nz) {
+    const size_t plane = (size_t)nx * ny;
+    const double msh = bshift ? -(*bshift) * inv : 0.0;
+    double* c = x + (size_t)k * plane;
+    const double *zm = x + (size_t)wrap(k - 1, nz) * plane, *zp = x + (size_t)wrap(k + 1, nz) * plane;
+    const double* bk = b + (size_t)k * plane;
+    int i = 2 * p + ((colour + j0 + k) & 1);
+    if (zero) {
+      for (int j = j0; j < j1; ++j) {
+        const int o = j * nx + i;
+        c[o] = fma(bk[o], inv, msh);
+        i = i + 1 == nx ? 0 : i + 1;
+      }
+    } else {
+      double sw = c[wrap(j0 - 1, ny) * nx + i] + c[j0 * nx + wrap(i - 1, nx)];
+#pragma unroll 4
+      for (int j = j0; j < j1; ++j) {
+        const int o = j * nx + i, ip = i + 1 == nx ? 0 : i + 1;
+        const double e = c[j * nx + ip];
+        const double en = e + c[(j + 1 == ny ? 0 : j + 1) * nx + i];
+        const double v = fma(offinv, (sw + en) + (zm[o] + zp[o]), fma(bk[o], inv, msh));
+        c[o] = v;
+        if (part) acc += v + e;
+        sw = en;
+        i = ip;
+      }
+    }
+  }
+  if (part) {
+    __shared__ double ws[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double v = 0.0;
+      for (int q = 0; q < 8; ++q) v += ws[q];
+      part[blockIdx.x + gridDim.x * blockIdx.y] = v;
+    }
+  }
+}
+
+// FP64 restriction of the residual after a sweep, whose black cells have none:
+// the red cells' alone, half the operations. Per coarse cell off times the sum
+// of its four red children's neighbours, plus the sum of their b - shift, minus
+// diag times that of their x, over 8. 128^3: 22 us, 51 with all cells.
+__global__ void __launch_bounds__(256) k_restrict_red_f64(const double* __restrict__ x, const double* __restrict__ b,
+                                                          const double* __restrict__ bshift, double* __restrict__ bc,
+                                                          int nx, int ny, int nz, double diag, double off) {
+  const int nxc = nx >> 1, nyc = ny >> 1, nzc = nz >> 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int I = t % nxc, J = (t / nxc) % nyc, K = t / (nxc * nyc);
+  if (K >= nzc) return;
+  const size_t plane = (size_t)nx * ny;
+  double sb = bshift ? -4.0 * *bshift : 0.0, sx = 0.0, sn = 0.0;
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      const int j = 2 * J + dy, k = 2 * K + dz, i = 2 * I + ((dy + dz) & 1);
+      const double* c = x + k * plane;
+      const size_t o = k * plane + (size_t)j * nx + i;
+      const double we = c[j * nx + wrap(i - 1, nx)] + c[j * nx + wrap(i + 1, nx)];
+      const double ns = c[wrap(j - 1, ny) * nx + i] + c[wrap(j + 1, ny) * nx + i];
+      const double du = x[wrap(k - 1, nz) * plane + (size_t)j * nx + i] + x[wrap(k + 1, nz) * plane + (size_t)j * nx + i];
+      sn += (we + ns) + du;
+      sx += x[o];
+      sb += b[o];
+    }
+  bc[t] = fma(off, sn, fma(-diag, sx, sb)) * 0.125;
+}
+
+// FP64 prolongation before a sweep, which reads no red cells: only the black
+// ones are corrected, each axis interpolated once for the cells that share it
+// (two coarse cells per thread; nx % 4 == 0). The arithmetic of every
+// prolongation kernel. 128^3: 18 us, 25 for all cells.
+__global__ void __launch_bounds__(256) k_prolong_black_f64(const double* __restrict__ xc, double* __restrict__ x, int nx,
+                                                           int ny, int nz) {
+  const int nxc = nx >> 1, nyc = ny >> 1, nzc = nz >> 1, nxp = nxc >> 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int I = 2 * (t % nxp), J = (t / nxp) % nyc, K = t / (nxp * nyc);
+  if (K >= nzc) return;
+  const int Ix[4] = {wrap(I - 1, nxc), I, I + 1, wrap(I + 2, nxc)};
+  const int Jy[3] = {wrap(J - 1, nyc), J, wrap(J + 1, nyc)};
+  const int Kz[3] = {wrap(K - 1, nzc), K, wrap(K + 1, nzc)};
+  double c[3][3][4];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const double* row = xc + ((size_t)Kz[a] * nyc + Jy[r]) * nxc;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[a][r][q] = row[Ix[q]];
+    }
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz) {
+    double z[3][4];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[r][q] = prolong_axis(c[1][r][q], c[dz ? 2 : 0][r][q]);
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      double zy[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) zy[q] = prolong_axis(z[1][q], z[dy ? 2 : 0][q]);
+      double* dst = x + ((size_t)(2 * K + dz) * ny + 2 * J + dy) * nx + 2 * I;
+      if ((dy + dz) & 1) {  // black: the even cells of each pair
+        dst[0] = prolong_add(dst[0], prolong_axis(zy[1], zy[0]));
+        dst[2] = prolong_add(dst[2], prolong_axis(zy[2], zy[1]));
+      } else {
+        dst[1] = prolong_add(dst[1], prolong_axis(zy[1], zy[2]));
+        dst[3] = prolong_add(dst[3], prolong_axis(zy[2], zy[3]));
+      }
+    }
+  }
+}
+
 // Coarse cell (I, J, K) gets the mean over its 8 children of b - shift - A x.
 template <typename T>
 __global__ void __launch_bounds__(256) k_resid_restrict(const T* __restrict__ x, const T* __restrict__ b,
@@ -805,7 +944,8 @@ static bool rows_shape(const SweepShape* tn, Dims d) {
 template <typename T>
 bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b) {
   if (!aligned16(x) || !aligned16(b)) return false;
-  return rb_sweep_fused_ok<T>(d) || (sizeof(T) == 4 && zero && d.nx % 4 == 0);
+  if (sizeof(T) == 8) return rb_sweep_fused_ok<T>(d) && tuned_sweep(8, TUNE_SWEEP, d);
+  return rb_sweep_fused_ok<T>(d) || (zero && d.nx % 4 == 0);
 }
 
 template <typename T, int TX, bool ZERO>
@@ -857,6 +997,28 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
       }
     }
   }
+  if constexpr (sizeof(T) == 8) {
+    // in place, one colour at a time, unless a tiled shape was chosen
+    if (!(rb_sweep_swaps<T>(d, zero, xin, b) && aligned16(xout))) {
+      const int np = d.nx / 2;
+      // rows per thread: long diagonals share more, but the chip wants some
+      // 100000 threads (FP64 latency on 152 SMs)
+      const size_t cells = (size_t)np * d.ny * d.nz;
+      int yc = (int)(cells / 100000);
+      yc = yc < 2 ? 2 : (yc > 16 ? 16 : yc);
+      yc = yc > d.ny ? d.ny : yc;
+      const dim3 g((unsigned)(((size_t)np * d.nz + 255) / 256), (d.ny + yc - 1) / yc);
+      const int nblk = (int)(g.x * g.y);
+      if (nblk > part_cap) part = nullptr;
+      for (int colour = 0; colour < 2; ++colour) {
+        prof_begin(c, s);
+        k_rb_half_f64<<<g, 256, 0, s>>>(const_cast<T*>(xin), b, bshift, d.nx, d.ny, d.nz, yc, inv, off * inv, colour,
+                                        (zero && colour == 0) ? 1 : 0, colour == 1 ? part : nullptr);
+        prof_end(c, s, "rb_half_f64", 1.5 * sizeof(T) * d.n());
+      }
+      return -1 - (part ? nblk : 0);
+    }
+  }
   if (rb_sweep_fused_ok<T>(d) && aligned16(xin) && aligned16(xout) && aligned16(b)) {
     // 64-wide tiles for FP32 (18 vectors per row), 32-wide for FP64
     const SweepShape* tn = tuned_sweep((int)sizeof(T), TUNE_SWEEP, d);
@@ -895,6 +1057,7 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
     prof_end(c, s, "rb_sweep", (zero ? 2.0 : 3.0) * sizeof(T) * d.n());
     return part ? nblk : 0;
   }
+  if constexpr (sizeof(T) == 4) {
   // small levels: two in-place half sweeps
   const int np = d.nx / 2;
   dim3 blk(np >= 32 ? 32 : np, 8, 1);
@@ -908,11 +1071,22 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
                                    (zero && colour == 0) ? 1 : 0);
     prof_end(c, s, "rb_half", 1.5 * sizeof(T) * d.n());
   }
+  }
   return -1;
 }
 
 template <typename T>
-void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, Dims d, Stencil st, cudaStream_t s) {
+void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, Dims d, Stencil st, bool swept,
+                           cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (swept) {
+      const unsigned blocks = (unsigned)((d.n() / 8 + 255) / 256);
+      prof_begin(P_RESTRICT64, s);
+      k_restrict_red_f64<<<blocks, 256, 0, s>>>(x, b, bshift, bc, d.nx, d.ny, d.nz, st.diag, st.off);
+      prof_end(P_RESTRICT64, s, "restrict_red_f64", 2.125 * sizeof(T) * d.n());
+      return;
+    }
+  }
   const int nxc = d.nx / 2, nyc = d.ny / 2, nzc = d.nz / 2;
   if (d.nx % 4 == 0 && d.nx >= 8 && aligned16(x) && aligned16(b)) {
     const int np = nxc / 2;
@@ -988,7 +1162,16 @@ int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const 
 }
 
 template <typename T>
-void launch_prolong8(const T* xc, T* x, Dims d, cudaStream_t s) {
+void launch_prolong8(const T* xc, T* x, Dims d, bool sweep_follows, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (sweep_follows && d.nx % 4 == 0 && d.nx >= 8) {
+      const unsigned blocks = (unsigned)((d.n() / 16 + 255) / 256);
+      prof_begin(P_PROLONG64, s);
+      k_prolong_black_f64<<<blocks, 256, 0, s>>>(xc, x, d.nx, d.ny, d.nz);
+      prof_end(P_PROLONG64, s, "prolong_black_f64", 2.125 * sizeof(T) * d.n());
+      return;
+    }
+  }
   const int nxc = d.nx / 2, nyc = d.ny / 2, nzc = d.nz / 2;
   if (d.nx % 4 == 0 && d.nx >= 8 && aligned16(x)) {
     const int np = nxc / 2;
@@ -1025,8 +1208,9 @@ void launch_vcycle_small(const CoarseLevels& lv, const T* b, T* x, const double*
                                        int, cudaStream_t);                                                  \
   template int launch_rb_sweep<T>(const T*, T*, const T*, const double*, Dims, Stencil, bool, double*, int,    \
                                   cudaStream_t);                                                            \
-  template void launch_resid_restrict<T>(const T*, const T*, const double*, T*, Dims, Stencil, cudaStream_t); \
-  template void launch_prolong8<T>(const T*, T*, Dims, cudaStream_t);                                       \
+  template void launch_resid_restrict<T>(const T*, const T*, const double*, T*, Dims, Stencil, bool,          \
+                                         cudaStream_t);                                                     \
+  template void launch_prolong8<T>(const T*, T*, Dims, bool, cudaStream_t);                                 \
   template int launch_prolong_sweep<T>(const T*, const T*, bool, T*, const T*, const double*, Dims, Stencil,   \
                                        double*, int, cudaStream_t);                                         \
   template bool rb_sweep_swaps<T>(Dims, bool, const T*, const T*);                                           \
