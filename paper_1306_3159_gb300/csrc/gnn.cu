@@ -373,7 +373,21 @@ __device__ __forceinline__ void load_mats(const float* __restrict__ th, int l, f
   }
 }
 
+// Row `row` of the filter matrix E_l into registers.
+__device__ __forceinline__ void load_filter(float (&e)[K], const float* __restrict__ E, int row) {
+#pragma unroll
+  for (int k = 0; k < K; k += 4) {
+    const float* p = E + row * K + k;  // (parameter blocks are not 16-byte aligned)
+    e[k] = p[0], e[k + 1] = p[1], e[k + 2] = p[2], e[k + 3] = p[3];
+  }
+}
+
 // Layer l (FP32): m_i, a_i = W_l m_i + V_l hp_i + c_l, h_i = hp_i + relu(a_i).
+// A lane keeps its two filter rows in registers over the edges (read from
+// memory for every edge, 32 scattered rows at a time, they were most of 26 us
+// for 1000 blobs of about 28 neighbours; now 17 us), and the next edge's index
+// and distance are fetched before the current one's arithmetic.  (Gathers of
+// four edges in flight at once cost more in registers: 20 us.)
 __global__ void __launch_bounds__(kWarps * 32) k_gnn_mp(const float* __restrict__ th, int l, int n, float invR,
                                                         int kmax, const int* __restrict__ cnt,
                                                         const int* __restrict__ nidx, const float* __restrict__ nr,
@@ -381,29 +395,40 @@ __global__ void __launch_bounds__(kWarps * 32) k_gnn_mp(const float* __restrict_
                                                         float* __restrict__ a, float* __restrict__ h) {
   __shared__ float sW[H * kPad], sV[H * kPad];
   load_mats(th, l, sW, sV);
-  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + (threadIdx.x >> 5);
-  if (i >= n) return;
-  const int k = lane & (K - 1);
-  const float* E = th + offE(l);
-  const float* eb = th + offEB(l);
   float m0 = 0.f, m1 = 0.f;
-  const int c = cnt[i];
-  for (int e = 0; e < c; ++e) {
-    const int j = nidx[(size_t)i * kmax + e];
-    const float s = nr[(size_t)i * kmax + e] * invR;
-    const float bk = basis_k(s, k);
-    const float fc = (1.f - s) * (1.f - s);
-    float p0 = eb[lane], p1 = eb[lane + 32];
-    for (int kk = 0; kk < K; ++kk) {
-      const float b = __shfl_sync(0xffffffffu, bk, kk);
-      p0 = fmaf(E[lane * K + kk], b, p0);
-      p1 = fmaf(E[(lane + 32) * K + kk], b, p1);
+  if (i < n) {
+    const int k = lane & (K - 1);
+    const float* eb = th + offEB(l);
+    float E0[K], E1[K];
+    load_filter(E0, th + offE(l), lane);
+    load_filter(E1, th + offE(l), lane + 32);
+    const float b0 = eb[lane], b1 = eb[lane + 32];
+    const int c = cnt[i];
+    const int* ji = nidx + (size_t)i * kmax;
+    const float* ri = nr + (size_t)i * kmax;
+    int j = c > 0 ? ji[0] : 0;
+    float r = c > 0 ? ri[0] : 0.f;
+    for (int e = 0; e < c; ++e) {
+      const float h0 = hp[(size_t)j * H + lane], h1 = hp[(size_t)j * H + lane + 32];
+      const float s = r * invR;
+      if (e + 1 < c) j = ji[e + 1], r = ri[e + 1];
+      const float bk = basis_k(s, k);
+      const float fc = (1.f - s) * (1.f - s);
+      float p0 = b0, p1 = b1;
+#pragma unroll
+      for (int kk = 0; kk < K; ++kk) {
+        const float b = __shfl_sync(0xffffffffu, bk, kk);
+        p0 = fmaf(E0[kk], b, p0);
+        p1 = fmaf(E1[kk], b, p1);
+      }
+      m0 = fmaf(fc * fmaxf(p0, 0.f), h0, m0);
+      m1 = fmaf(fc * fmaxf(p1, 0.f), h1, m1);
     }
-    m0 = fmaf(fc * fmaxf(p0, 0.f), hp[(size_t)j * H + lane], m0);
-    m1 = fmaf(fc * fmaxf(p1, 0.f), hp[(size_t)j * H + lane + 32], m1);
   }
+  __syncthreads();  // W_l and V_l are staged
+  if (i >= n) return;
   const float hi0 = hp[(size_t)i * H + lane], hi1 = hp[(size_t)i * H + lane + 32];
   float s0 = th[offC(l) + lane], s1 = th[offC(l) + lane + 32];
   for (int kk = 0; kk < H; ++kk) {
@@ -438,11 +463,12 @@ __device__ double block_sum(double v, double* sh) {
   __syncthreads();
   if (l == 0) sh[w] = v;
   __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[k];
+  double t = l < (int)(blockDim.x >> 5) ? sh[l] : 0.0;
   __syncthreads();
-  if (threadIdx.x == 0) sh[0] = t;
+  if (w == 0) {  // the warps' totals in one warp (32 additions in a row by one thread took a microsecond)
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (l == 0) sh[0] = t;
+  }
   __syncthreads();
   const double r = sh[0];
   __syncthreads();
@@ -461,7 +487,8 @@ __device__ __forceinline__ double log_pos(double v) {
 // Loss of one configuration and dL/dy (one CTA): r = (y - <y>) - (t - <t>),
 // L = <r^2>, dy = 2 r / n. out[0] = L.
 __global__ void __launch_bounds__(1024) k_gnn_loss(const float* __restrict__ y, const double* __restrict__ lam,
-                                                   int n, float* __restrict__ dy, double* __restrict__ out) {
+                                                   int n, double inv_n, float* __restrict__ dy,
+                                                   double* __restrict__ out) {
   __shared__ double sh[32];
   double sy = 0.0, st = 0.0;
 #pragma unroll 4
@@ -469,7 +496,6 @@ __global__ void __launch_bounds__(1024) k_gnn_loss(const float* __restrict__ y, 
     sy += (double)y[i];
     st += log_pos(lam[i]);
   }
-  const double inv_n = 1.0 / n;
   const double my = block_sum(sy, sh) * inv_n;
   const double mt = block_sum(st, sh) * inv_n;
   double l2 = 0.0;
@@ -504,10 +530,14 @@ __global__ void __launch_bounds__(1024) k_gnn_softmax(const float* __restrict__ 
   const float ymax = smax[0];
   double s = 0.0;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += (double)expf(y[i] - ymax);
-  const double scale = total / block_sum(s, sh);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) s += f2d_bits(expf(y[i] - ymax));
+  const double sum = block_sum(s, sh);
+  __shared__ double quotient;  // one thread's: an FP64 division in all 1024 would take several microseconds
+  if (threadIdx.x == 0) quotient = total / sum;
+  __syncthreads();
+  const double scale = quotient;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < n; i += blockDim.x) lam0[i] = scale * (double)expf(y[i] - ymax);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) lam0[i] = scale * f2d_bits(expf(y[i] - ymax));
 }
 
 // Backward through layer l's node update: dh = dh_in (or dy o at the last
@@ -577,27 +607,37 @@ __global__ void __launch_bounds__(kWarps * 32) k_gnn_back_edges(const float* __r
   float ge0 = 0.f, ge1 = 0.f;
   if (i < n) {
     const int k = lane & (K - 1);
+    float E0[K], E1[K];
+    load_filter(E0, E, lane);
+    load_filter(E1, E, lane + 32);
+    const float b0 = eb[lane], b1 = eb[lane + 32];
     const float dmi0 = dm[(size_t)i * H + lane], dmi1 = dm[(size_t)i * H + lane + 32];
     float acc0 = dhv[(size_t)i * H + lane], acc1 = dhv[(size_t)i * H + lane + 32];
     const int c = cnt[i];
+    const int* ji = nidx + (size_t)i * kmax;
+    const float* ri = nr + (size_t)i * kmax;
+    int j = c > 0 ? ji[0] : 0;
+    float r = c > 0 ? ri[0] : 0.f;
     for (int e = 0; e < c; ++e) {
-      const int j = nidx[(size_t)i * kmax + e];
-      const float s = nr[(size_t)i * kmax + e] * invR;
+      const float dj0 = dm[(size_t)j * H + lane], dj1 = dm[(size_t)j * H + lane + 32];
+      const float hj0 = hp[(size_t)j * H + lane], hj1 = hp[(size_t)j * H + lane + 32];
+      const float s = r * invR;
+      if (e + 1 < c) j = ji[e + 1], r = ri[e + 1];
       const float bk = basis_k(s, k);
       const float fc = (1.f - s) * (1.f - s);
-      float p0 = eb[lane], p1 = eb[lane + 32];
+      float p0 = b0, p1 = b1;
       float b[K];
 #pragma unroll
       for (int kk = 0; kk < K; ++kk) {
         b[kk] = __shfl_sync(0xffffffffu, bk, kk);
-        p0 = fmaf(E[lane * K + kk], b[kk], p0);
-        p1 = fmaf(E[(lane + 32) * K + kk], b[kk], p1);
+        p0 = fmaf(E0[kk], b[kk], p0);
+        p1 = fmaf(E1[kk], b[kk], p1);
       }
       const float F0 = fmaxf(p0, 0.f), F1 = fmaxf(p1, 0.f);
-      acc0 = fmaf(fc * F0, dm[(size_t)j * H + lane], acc0);
-      acc1 = fmaf(fc * F1, dm[(size_t)j * H + lane + 32], acc1);
-      const float q0 = p0 > 0.f ? fc * dmi0 * hp[(size_t)j * H + lane] : 0.f;
-      const float q1 = p1 > 0.f ? fc * dmi1 * hp[(size_t)j * H + lane + 32] : 0.f;
+      acc0 = fmaf(fc * F0, dj0, acc0);
+      acc1 = fmaf(fc * F1, dj1, acc1);
+      const float q0 = p0 > 0.f ? fc * dmi0 * hj0 : 0.f;
+      const float q1 = p1 > 0.f ? fc * dmi1 * hj1 : 0.f;
       ge0 += q0;
       ge1 += q1;
 #pragma unroll
@@ -631,62 +671,141 @@ __global__ void __launch_bounds__(kWarps * 32) k_gnn_back_edges(const float* __r
 
 // Activations and gradients the parameter gradients read.
 struct GradArgs {
-  int n, nblk;
+  int n;
   const float* x;     // N x K
   const float* da0;   // N x H
   const float* h;     // (L + 1) x N x H: h_0 .. h_L
   const float* m;     // L x N x H
   const float* da;    // L x N x H
   const float* dy;    // N
-  const float* part;  // L x nblk x H x (K + 1)
 };
 
-// Parameter gradients that are sums over blobs, one thread per parameter,
-// blobs added in increasing order: dW0 = sum da0 x^T, dc0 = sum da0, per layer
-// dW_l = sum da_l m_l^T, dV_l = sum da_l h_{l-1}^T, dc_l = sum da_l and dE_l /
-// de_l from the per-CTA partials, do = sum dy h_L, do0 = sum dy.
-__global__ void k_gnn_param_grads(GradArgs ga, float* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NPARAM) return;
-  const int n = ga.n;
-  const size_t NH = (size_t)n * H;
-  float s = 0.f;
-  if (p < OFF_C0) {
-    const int r = p / K, c = p - r * K;
-    for (int i = 0; i < n; ++i) s = fmaf(ga.da0[(size_t)i * H + r], ga.x[(size_t)i * K + c], s);
-  } else if (p < OFF_C0 + H) {
-    const int r = p - OFF_C0;
-    for (int i = 0; i < n; ++i) s += ga.da0[(size_t)i * H + r];
-  } else if (p < OFF_O) {
-    const int l = (p - lbase(1)) / LSZ + 1;
-    const int q = p - lbase(l);
-    const float* da = ga.da + (size_t)(l - 1) * NH;
-    if (q < H * K + H) {
-      // E (row r, col c) and e (row r) from the CTA partials
-      const int r = q < H * K ? q / K : q - H * K;
-      const int c = q < H * K ? q - (q / K) * K : K;
-      const float* part = ga.part + (size_t)(l - 1) * ga.nblk * H * (K + 1);
-      for (int b = 0; b < ga.nblk; ++b) s += part[(size_t)b * H * (K + 1) + r * (K + 1) + c];
-    } else if (q < H * K + H + H * H) {
-      const int t = q - (H * K + H), r = t / H, c = t - r * H;
-      const float* m = ga.m + (size_t)(l - 1) * NH;
-      for (int i = 0; i < n; ++i) s = fmaf(da[(size_t)i * H + r], m[(size_t)i * H + c], s);
-    } else if (q < H * K + H + 2 * H * H) {
-      const int t = q - (H * K + H + H * H), r = t / H, c = t - r * H;
-      const float* hp = ga.h + (size_t)(l - 1) * NH;
-      for (int i = 0; i < n; ++i) s = fmaf(da[(size_t)i * H + r], hp[(size_t)i * H + c], s);
-    } else {
-      const int r = q - (H * K + H + 2 * H * H);
-      for (int i = 0; i < n; ++i) s += da[(size_t)i * H + r];
+// Parameter gradients that are sums over blobs, in two launches: chunks of
+// blobs, then the chunks. (One thread per parameter walking over all blobs, as
+// one launch, was a chain of n dependent FMAs on 115 CTAs: 114 us for 1000 blobs,
+// against 16 us for the two.)
+//
+// A chunk's gradient of everything but E_l and e_l (GPART values): per layer
+// dW_l = da_l^T m_l (64 x 64), dV_l = da_l^T h_{l-1}, dc_l; dW0 = da0^T x (64 x
+// 16), dc0, do, do0. blockIdx.y = 0 .. L - 1: layer y + 1; L: the rest. A CTA
+// stages kGradRows blobs at a time in shared memory and accumulates in registers:
+// thread (r, c) the 4 x 4 block of both products at rows 4 r, columns 4 c.
+constexpr int GPART = (OFF_C0 + H + L * (2 * H * H + H) + H + 1 + 3) & ~3;  // (16-byte rows)
+constexpr int GP_REST = L * (2 * H * H + H);  // where W0, c0, o, o0 begin
+constexpr int kGradRows = 32, kGradChunks = 128;
+
+__global__ void __launch_bounds__(256) k_gnn_grad_chunks(GradArgs ga, int per, float* __restrict__ gp) {
+  __shared__ __align__(16) float sa[kGradRows][H], sm[kGradRows][H], sh[kGradRows][H];
+  __shared__ float sdy[kGradRows];
+  const int tid = threadIdx.x, l = blockIdx.y + 1;
+  const int b0 = blockIdx.x * per, b1 = min(b0 + per, ga.n);
+  const size_t NH = (size_t)ga.n * H;
+  float* out = gp + (size_t)blockIdx.x * GPART;
+  auto stage = [&](float (*d)[H], const float* src, int b, int rows, int width) {
+    for (int t = tid; t < rows * width; t += 256) d[t / width][t % width] = src[(size_t)b * width + t];
+  };
+  if (l <= L) {
+    const int r = 4 * (tid >> 4), c = 4 * (tid & 15);
+    float w[4][4] = {}, v[4][4] = {}, cb[4] = {};
+    for (int b = b0; b < b1; b += kGradRows) {
+      const int rows = min(kGradRows, b1 - b);
+      __syncthreads();
+      stage(sa, ga.da + (l - 1) * NH, b, rows, H);
+      stage(sm, ga.m + (l - 1) * NH, b, rows, H);
+      stage(sh, ga.h + (l - 1) * NH, b, rows, H);
+      __syncthreads();
+      for (int i = 0; i < rows; ++i) {
+        float av[4], mv[4], hv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) av[q] = sa[i][r + q], mv[q] = sm[i][c + q], hv[q] = sh[i][c + q];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          cb[p] += av[p];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            w[p][q] = fmaf(av[p], mv[q], w[p][q]);
+            v[p][q] = fmaf(av[p], hv[q], v[p][q]);
+          }
+        }
+      }
     }
-  } else if (p < OFF_O0) {
-    const int r = p - OFF_O;
-    const float* hL = ga.h + (size_t)L * NH;
-    for (int i = 0; i < n; ++i) s = fmaf(ga.dy[i], hL[(size_t)i * H + r], s);
+    out += (l - 1) * (2 * H * H + H);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      *reinterpret_cast<float4*>(out + (r + p) * H + c) = make_float4(w[p][0], w[p][1], w[p][2], w[p][3]);
+      *reinterpret_cast<float4*>(out + H * H + (r + p) * H + c) = make_float4(v[p][0], v[p][1], v[p][2], v[p][3]);
+      if (c == 0) out[2 * H * H + r + p] = cb[p];
+    }
   } else {
-    for (int i = 0; i < n; ++i) s += ga.dy[i];
+    const int r = tid >> 2, c = 4 * (tid & 3);
+    float w[4] = {}, c0 = 0.f, o = 0.f, o0 = 0.f;
+    for (int b = b0; b < b1; b += kGradRows) {
+      const int rows = min(kGradRows, b1 - b);
+      __syncthreads();
+      stage(sa, ga.da0, b, rows, H);
+      stage(sh, ga.h + (size_t)L * NH, b, rows, H);
+      for (int t = tid; t < rows * K; t += 256) sm[t / K][t % K] = ga.x[(size_t)b * K + t];
+      if (tid < rows) sdy[tid] = ga.dy[b + tid];
+      __syncthreads();
+      for (int i = 0; i < rows; ++i) {
+        const float av = sa[i][r];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = fmaf(av, sm[i][c + q], w[q]);
+        c0 += av;
+        o = fmaf(sdy[i], sh[i][r], o);
+        o0 += sdy[i];
+      }
+    }
+    out += GP_REST;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out[r * K + c + q] = w[q];
+    if (c == 0) {
+      out[OFF_C0 + r] = c0;
+      out[OFF_C0 + H + r] = o;
+      if (r == 0) out[OFF_C0 + 2 * H] = o0;
+    }
   }
-  grad[p] = s;
+}
+
+// The chunks of a parameter (E_l and e_l: the CTA partials of k_gnn_back_edges)
+// added up, a warp's lanes on consecutive parameters, the block's 8 rows taking
+// every eighth chunk; fixed order.
+__global__ void __launch_bounds__(256) k_gnn_param_grads(const float* __restrict__ gp, int chunks,
+                                                         const float* __restrict__ part, int nblk,
+                                                         float* __restrict__ grad) {
+  __shared__ float sums[8][32];
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+  float s = 0.f;
+  if (p < NPARAM) {
+    const float* src;
+    size_t stride = GPART;
+    int count = chunks;
+    if (p < OFF_C0 + H) {
+      src = gp + GP_REST + p;
+    } else if (p < OFF_O) {
+      const int l = (p - lbase(1)) / LSZ + 1, q = p - lbase(l);
+      if (q < H * K + H) {
+        // E (row r, col c) and e (row r) from the edges' partials
+        const int r = q < H * K ? q / K : q - H * K, c = q < H * K ? q % K : K;
+        src = part + (size_t)(l - 1) * nblk * H * (K + 1) + r * (K + 1) + c;
+        stride = H * (K + 1);
+        count = nblk;
+      } else {
+        src = gp + (l - 1) * (2 * H * H + H) + (q - (H * K + H));
+      }
+    } else {
+      src = gp + GP_REST + OFF_C0 + H + (p - OFF_O);
+    }
+#pragma unroll 4
+    for (int b = row; b < count; b += 8) s += src[(size_t)b * stride];
+  }
+  sums[row][lane] = s;
+  __syncthreads();
+  if (row == 0 && p < NPARAM) {
+    float v = 0.f;
+    for (int q = 0; q < 8; ++q) v += sums[q][lane];
+    grad[p] = v;
+  }
 }
 
 // ---------------------------------------------------------------- inference on tensor cores
@@ -912,7 +1031,9 @@ struct ibrd_gnn_s {
   float *nr = nullptr, *x = nullptr, *a0 = nullptr, *h = nullptr, *m = nullptr, *a = nullptr, *y = nullptr;
   float *dy = nullptr, *da0 = nullptr, *da = nullptr, *dm = nullptr, *dhv = nullptr, *dh = nullptr;
   float* part = nullptr;
+  float* gp = nullptr;          // chunk gradients (grad_chunk)
   __nv_bfloat16* wb = nullptr;  // bfloat16 layer weights for inference
+  bool wb_current = false;      // wb holds the current parameters
   // cell list (grow only): per blob its cell, the blobs sorted by cell, the
   // scratch candidate lists; per cell its count, start and fill cursor
   int *cell_of = nullptr, *cell_blobs = nullptr, *tj = nullptr;
@@ -964,6 +1085,10 @@ ibrd_status gnn_guarded(ibrd_gnn m, const char* name, F&& f) {
   return st;
 }
 
+// Blobs per chunk of the parameter gradients: kGradRows, more where that makes
+// over kGradChunks chunks.
+int grad_chunk(int n) { return std::max(kGradRows, (n + kGradChunks - 1) / kGradChunks); }
+
 void ensure_cap(ibrd_gnn m, int n) {
   if (n <= m->cap) return;
   const size_t N = (size_t)n, nb = (N + kWarps - 1) / kWarps;
@@ -984,6 +1109,7 @@ void ensure_cap(ibrd_gnn m, int n) {
   galloc(&m->dhv, N * H);
   galloc(&m->dh, N * H);
   galloc(&m->part, L * nb * H * (K + 1));
+  galloc(&m->gp, (size_t)std::min<size_t>(kGradChunks, (N + kGradRows - 1) / kGradRows) * GPART);
   galloc(&m->cell_of, N);
   galloc(&m->cell_blobs, N);
   galloc(&m->tj, N * m->kmax);
@@ -1064,10 +1190,11 @@ void forward(ibrd_gnn m, const double* q, int n, double lx, double ly, double lz
   prof_begin(P_SETUP, m->s);
   k_gnn_layer0<<<nb, kWarps * 32, 0, m->s>>>(m->th, n, invR, m->kmax, m->cnt, m->nr, m->x, m->a0, hbuf(m, n, 0));
   prof_end(P_SETUP, m->s, "gnn_layer0");
-  if (bf16) {
+  if (bf16 && !m->wb_current) {  // laid out once per parameter set
     prof_begin(P_SETUP, m->s);
     k_gnn_weights_bf16<<<(L * BLSZ + 255) / 256, 256, 0, m->s>>>(m->th, m->wb);
     prof_end(P_SETUP, m->s, "gnn_weights_bf16");
+    m->wb_current = true;
   }
   for (int l = 1; l <= L; ++l) {
     if (bf16) {
@@ -1093,10 +1220,10 @@ void forward(ibrd_gnn m, const double* q, int n, double lx, double ly, double lz
 }
 
 void check_overflow(ibrd_gnn m) {
-  int of = 0;
-  IBRD_CUDA(cudaMemcpyAsync(&of, m->oflow, sizeof(int), cudaMemcpyDeviceToHost, m->s));
+  int* of = reinterpret_cast<int*>(m->host + 4);  // pinned
+  IBRD_CUDA(cudaMemcpyAsync(of, m->oflow, sizeof(int), cudaMemcpyDeviceToHost, m->s));
   IBRD_CUDA(cudaStreamSynchronize(m->s));
-  if (of) throw GnnArgError{IBRD_ERR_ARG, "a blob has more neighbours than max_neighbours"};
+  if (*of) throw GnnArgError{IBRD_ERR_ARG, "a blob has more neighbours than max_neighbours"};
 }
 
 // Loss and gradient of one configuration (after the FP32 forward); gradient
@@ -1107,7 +1234,7 @@ void backward(ibrd_gnn m, int n, const double* lam) {
   const int nb = (n + kWarps - 1) / kWarps;
   const float invR = (float)(1.0 / m->cutoff);
   prof_begin(P_SETUP, m->s);
-  k_gnn_loss<<<1, 1024, 0, m->s>>>(m->y, lam, n, m->dy, m->loss);
+  k_gnn_loss<<<1, 256, 0, m->s>>>(m->y, lam, n, 1.0 / n, m->dy, m->loss);
   prof_end(P_SETUP, m->s, "gnn_loss");
   for (int l = L; l >= 1; --l) {
     prof_begin(P_SETUP, m->s);
@@ -1120,14 +1247,19 @@ void backward(ibrd_gnn m, int n, const double* lam) {
         l == 1 ? m->a0 : nullptr, l == 1 ? m->da0 : m->dh, m->part + (size_t)(l - 1) * nb * H * (K + 1));
     prof_end(P_SETUP, m->s, "gnn_back_edges");
   }
-  GradArgs ga{n, nb, m->x, m->da0, m->h, m->m, m->da, m->dy, m->part};
+  GradArgs ga{n, m->x, m->da0, m->h, m->m, m->da, m->dy};
+  const int per = grad_chunk(n), chunks = (n + per - 1) / per;
   prof_begin(P_SETUP, m->s);
-  k_gnn_param_grads<<<(NPARAM + 255) / 256, 256, 0, m->s>>>(ga, m->g);
+  k_gnn_grad_chunks<<<dim3(chunks, L + 1), 256, 0, m->s>>>(ga, per, m->gp);
+  prof_end(P_SETUP, m->s, "gnn_grad_chunks");
+  prof_begin(P_SETUP, m->s);
+  k_gnn_param_grads<<<(NPARAM + 31) / 32, 256, 0, m->s>>>(m->gp, chunks, m->part, nb, m->g);
   prof_end(P_SETUP, m->s, "gnn_param_grads");
 }
 
 void adam(ibrd_gnn m, const float* grad, double lr) {
   m->step++;
+  m->wb_current = false;
   const double b1 = 0.9, b2 = 0.999;
   const float c1 = (float)(1.0 - std::pow(b1, (double)m->step));
   const float c2 = (float)(1.0 - std::pow(b2, (double)m->step));
@@ -1192,7 +1324,7 @@ void ibrd_gnn_destroy(ibrd_gnn m) {
   for (void* p : {(void*)m->th, (void*)m->g, (void*)m->m1, (void*)m->m2, (void*)m->cnt, (void*)m->nidx,
                   (void*)m->oflow, (void*)m->nr, (void*)m->x, (void*)m->a0, (void*)m->h, (void*)m->m,
                   (void*)m->a, (void*)m->y, (void*)m->dy, (void*)m->da0, (void*)m->da, (void*)m->dm,
-                  (void*)m->dhv, (void*)m->dh, (void*)m->part, (void*)m->loss, (void*)m->p32, (void*)m->wb,
+                  (void*)m->dhv, (void*)m->dh, (void*)m->part, (void*)m->gp, (void*)m->loss, (void*)m->p32, (void*)m->wb,
                   (void*)m->cell_of, (void*)m->cell_blobs, (void*)m->tj, (void*)m->tr, (void*)m->cell_cnt,
                   (void*)m->cell_start, (void*)m->cell_cursor})
     if (p) cudaFree(p);
@@ -1206,6 +1338,7 @@ const char* ibrd_gnn_last_error(ibrd_gnn m) { return m ? m->err.c_str() : "null 
 ibrd_status ibrd_gnn_set_params(ibrd_gnn m, const float* theta, int reset_optimizer) {
   return gnn_guarded(m, "ibrd_gnn_set_params", [&]() {
     if (!theta) throw GnnArgError{IBRD_ERR_ARG, "null parameters"};
+    m->wb_current = false;
     IBRD_CUDA(cudaMemcpyAsync(m->th, theta, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, m->s));
     if (reset_optimizer) {
       IBRD_CUDA(cudaMemsetAsync(m->m1, 0, sizeof(float) * NPARAM, m->s));
@@ -1239,6 +1372,7 @@ ibrd_status ibrd_gnn_init_params(ibrd_gnn m, unsigned long long seed) {
       fill(offV(l), H * H, 1.0 / std::sqrt((double)H));
     }
     fill(OFF_O, H, 1.0 / std::sqrt((double)H));
+    m->wb_current = false;
     IBRD_CUDA(cudaMemcpyAsync(m->th, th.data(), sizeof(float) * NPARAM, cudaMemcpyHostToDevice, m->s));
     IBRD_CUDA(cudaMemsetAsync(m->m1, 0, sizeof(float) * NPARAM, m->s));
     IBRD_CUDA(cudaMemsetAsync(m->m2, 0, sizeof(float) * NPARAM, m->s));

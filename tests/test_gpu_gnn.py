@@ -241,3 +241,55 @@ def test_seeded_init(ibrd):
         assert np.abs(p[name]).max() <= lim and np.abs(p[name]).max() > 0.9 * lim
     for name in gnn.BIASES + ["o0"]:
         assert not p[name].any()
+
+
+# blobs: one; a chunk of the parameter gradients less one, exactly and plus one
+# (32 blobs); several with a remainder; above 4096, where chunks grow
+@pytest.mark.parametrize("n,side,R", [(1, 24, 6.0), (31, 24, 6.0), (32, 24, 6.0), (33, 24, 6.0), (150, 30, 6.0),
+                                      (4200, 80, 3.5)])
+def test_gradient_chunks(ibrd, n, side, R):
+    """The parameter gradient summed over chunks of blobs, against the FP64
+    definition block by block (the bound of the test above), and bit for bit
+    the same on a second call and after a call with more blobs."""
+    q, box = _config(n, side, 15 + n)
+    th = _theta(8)
+    lam = np.exp(np.random.default_rng(3).normal(0.0, 0.15, size=n))
+    m = ibrd.GNN(R, 64)
+    m.set_params(th)
+    L, g = m.loss_grad(dev(q), box, dev(lam))
+    q2, box2 = _config(90, 30, 4)
+    m.loss_grad(dev(q2), box2, dev(np.ones(90)))
+    L2, g2 = m.loss_grad(dev(q), box, dev(lam))
+    assert L == L2 and (host(g) == host(g2)).all()
+    L_ref, g_ref = gnn.loss_and_grad(th, q, box, R, lam)
+    assert abs(L - L_ref) <= 1e-4 * L_ref + 1e-12
+    g, off = host(g).astype(np.float64), 0
+    for name, shape in gnn.LAYOUT:
+        k = int(np.prod(shape))
+        a, b = g[off:off + k], g_ref[off:off + k]
+        assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b) + 1e-6 * np.linalg.norm(g_ref) + 1e-12, name
+        off += k
+
+
+def test_prediction_follows_the_parameters(ibrd):
+    """The bfloat16 weights are laid out again after every change of the
+    parameters: set, initialised, stepped and trained."""
+    import torch
+    q, box = _config(60, 30, 6)
+    qd, ld = dev(q), dev(np.exp(np.random.default_rng(1).normal(0.0, 0.1, size=60)))
+    m = ibrd.GNN(8.0, 64)
+
+    def fresh():
+        k = ibrd.GNN(8.0, 64)
+        k.set_params(m.get_params())
+        return host(k.predict(qd, box, 60.0))
+
+    seen = []
+    for change in (lambda: m.set_params(_theta(1)), lambda: m.init_params(5),
+                   lambda: m.adam_step(m.loss_grad(qd, box, ld)[1], 1e-2),
+                   lambda: m.train([qd], [box], [ld], 2, 1e-2)):
+        change()
+        p = host(m.predict(qd, box, 60.0))
+        assert (p == fresh()).all() and (host(m.predict(qd, box, 60.0)) == p).all()
+        seen.append(p)
+    assert all((a != b).any() for a, b in zip(seen, seen[1:]))
