@@ -2740,8 +2740,8 @@ void ibrd_grid_destroy(ibrd_grid g) {
   for (auto& e : g->h32.tables) F(e.second);
   for (auto& e : g->h32.hartley) F(e.second);
   BlobSet& b = g->blobs;
-  F(b.q); F(b.idx); F(b.w64); F(b.w32); F(b.tile_count); F(b.tile_offset); F(b.tile_cursor); F(b.tile_blobs);
-  F(b.active); F(b.d_meta); F(b.cell_count); F(b.cell_offset); F(b.cells); F(b.cell_tile);
+  F(b.q); F(b.idx); F(b.w64); F(b.w32); F(b.tile_count); F(b.tile_offset); F(b.tile_raw); F(b.tile_blobs);
+  F(b.active); F(b.d_meta); F(b.cells); F(b.cell_tile);
   F(g->scal); F(g->partial); F(g->dflag); F(g->ticket); F(g->gst); F(g->ghist);
   if (g->host) cudaFreeHost(g->host);
   F(g->V); F(g->Z); F(g->H); F(g->cs); F(g->sn); F(g->gvec); F(g->yv); F(g->hb2); F(g->vsc); F(g->xs); F(g->bs);
@@ -2828,7 +2828,7 @@ ibrd_status ibrd_grid_create(ibrd_grid* out, int nx, int ny, int nz, double h, d
     g->tune.wait_err = reinterpret_cast<int*>(g->scal + S_WAIT);
     IBRD_CUDA(cudaMallocHost(&g->host, sizeof(double) * 64));
     IBRD_CUDA(cudaMemsetAsync(g->scal, 0, sizeof(double) * S_COUNT, g->s));
-    blobs_setup(g->blobs, g->d, g->h, nullptr, 0, g->s);
+    blobs_setup(g->blobs, g->d, g->h, nullptr, 0, nullptr, g->s);
     return IBRD_OK;
   });
   if (st != IBRD_OK) {
@@ -2844,11 +2844,11 @@ ibrd_status ibrd_set_blobs(ibrd_grid g, const double* q, int n) {
     if (n < 0 || (n > 0 && !q)) throw ArgError{IBRD_ERR_ARG, "bad blob array"};
     IBRD_CUDA(cudaMemsetAsync(g->dflag, 0, sizeof(int), g->s));
     if (n > 0) launch_nonfinite<double>(q, (size_t)3 * n, g->dflag, g->s);
-    int flag = 0;
-    IBRD_CUDA(cudaMemcpyAsync(&flag, g->dflag, sizeof(int), cudaMemcpyDeviceToHost, g->s));
+    int* host = reinterpret_cast<int*>(g->host + 60);
+    IBRD_CUDA(cudaMemcpyAsync(host, g->dflag, sizeof(int), cudaMemcpyDeviceToHost, g->s));
     IBRD_CUDA(cudaStreamSynchronize(g->s));
-    if (flag) throw ArgError{IBRD_ERR_NONFINITE, "non-finite blob position"};
-    blobs_setup(g->blobs, g->d, g->h, q, n, g->s);
+    if (*host) throw ArgError{IBRD_ERR_NONFINITE, "non-finite blob position"};
+    blobs_setup(g->blobs, g->d, g->h, q, n, host, g->s);
     g->blob_version++;
     return IBRD_OK;
   });

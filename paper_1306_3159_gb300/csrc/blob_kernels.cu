@@ -8,6 +8,7 @@
 // cells, the contributions of the tile's blobs in increasing blob index, so
 // the result is deterministic and each field cell is written once.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "internal.h"
@@ -39,160 +40,258 @@ __device__ __forceinline__ int pmod(int a, int n) {
   return r < 0 ? r + n : r;
 }
 
-// Per blob and axis: wrapped position, 4 wrapped cell indices, 4 weights.
-__global__ void k_blob_prep(const double* __restrict__ qin, int n, int nx, int ny, int nz, double h, int width,
-                            double* __restrict__ q, int* __restrict__ idx, double* __restrict__ w64,
-                            float* __restrict__ w32) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n) return;
-  const int dims[3] = {nx, ny, nz};
+// The distinct tiles under a blob's 4 cells of one axis, in order of appearance;
+// -1 where there are fewer. Three only where the last tile of the axis has one
+// or two cells and the support crosses all of it.
+__device__ __forceinline__ void axis_tiles(int4 ix, int* t) {
+  const int a = ix.x / kTile, b = ix.y / kTile, c = ix.z / kTile, d = ix.w / kTile;
+  t[0] = a;
+  t[1] = b != a ? b : c != a ? c : d != a ? d : -1;
+  t[2] = (c != a && c != t[1]) ? c : (d != a && d != t[1]) ? d : -1;
+}
+int max_axis_tiles(int n, int tiles) { return std::min(tiles, n % kTile == 1 || n % kTile == 2 ? 3 : 2); }
+
+// visit(tile) for the tiles of a blob, shared out over 8 threads: thread c takes
+// the ones whose place along (x, y, z) has the parities of c's bits.
+template <typename F>
+__device__ __forceinline__ void blob_tiles(int4 ix, int4 iy, int4 iz, int c, int ntx, int nty, F&& visit) {
+  int tx[3], ty[3], tz[3];
+  axis_tiles(ix, tx);
+  axis_tiles(iy, ty);
+  axis_tiles(iz, tz);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const double L = dims[a] * h;
-    double p = qin[3 * b + a];
+  for (int u = 0; u < 8; ++u) {  // first or second place of each axis that the thread has
+    const int px = c & 1, py = (c >> 1) & 1, pz = c >> 2;
+    const int x = (u & 1) ? (px ? -1 : tx[2]) : (px ? tx[1] : tx[0]);
+    const int y = (u & 2) ? (py ? -1 : ty[2]) : (py ? ty[1] : ty[0]);
+    const int z = (u & 4) ? (pz ? -1 : tz[2]) : (pz ? tz[1] : tz[0]);
+    if (x >= 0 && y >= 0 && z >= 0) visit(x + ntx * (y + nty * z));
+  }
+}
+
+// Per blob and axis: wrapped position, 4 wrapped cell indices, 4 weights; and the
+// number of blobs that touch each tile (count zeroed before). One CTA per 32
+// blobs: a thread per blob and axis for the weights, whose divisions and square
+// roots are a long FP64 chain, then 8 threads per blob for its tiles. (A thread
+// per blob in CTAs of 128 left 4096 blobs on 32 of the SMs: 14.5 us, and 3.4 us
+// for the counts in a launch of their own; 7.0 us for both.)
+constexpr int kPrepBlobs = 32;
+__global__ void __launch_bounds__(8 * kPrepBlobs)
+    k_blob_prep(const double* __restrict__ qin, int n, int nx, int ny, int nz, double h, int width,
+                double* __restrict__ q, int* __restrict__ idx, double* __restrict__ w64, float* __restrict__ w32,
+                int ntx, int nty, int* __restrict__ count) {
+  __shared__ int4 cells[3 * kPrepBlobs];
+  const int b0 = blockIdx.x * kPrepBlobs, t = threadIdx.x;
+  const int g = 3 * b0 + t;  // 3 blob + axis
+  if (t < 3 * kPrepBlobs && g < 3 * n) {
+    const int a = t % 3;
+    const int dim = a == 0 ? nx : a == 1 ? ny : nz;
+    const double L = dim * h;
+    double p = qin[g];
     p -= floor(p / L) * L;
     if (p >= L) p -= L;
     if (p < 0.0) p = 0.0;
-    q[3 * b + a] = p;
+    q[g] = p;
     const double u = p / h - 0.5;  // position in cell-index units (centres at integers)
     int base;
     if (width == 4)
       base = (int)floor(u) - 1;
     else
       base = (int)floor(u + 0.5) - 1;
+    double w[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       const double r = u - (double)(base + s);
-      double wt;
       if (width == 4)
-        wt = phi4(r);
+        w[s] = phi4(r);
       else
-        wt = (s < 3) ? phi3(r) : 0.0;
-      const int o = (b * 3 + a) * 4 + s;
-      idx[o] = pmod(base + s, dims[a]);
-      w64[o] = wt;
-      w32[o] = (float)wt;
+        w[s] = (s < 3) ? phi3(r) : 0.0;
     }
+    const int4 c = make_int4(pmod(base, dim), pmod(base + 1, dim), pmod(base + 2, dim), pmod(base + 3, dim));
+    cells[t] = c;
+    reinterpret_cast<int4*>(idx)[g] = c;
+    reinterpret_cast<double2*>(w64)[2 * (size_t)g] = make_double2(w[0], w[1]);
+    reinterpret_cast<double2*>(w64)[2 * (size_t)g + 1] = make_double2(w[2], w[3]);
+    reinterpret_cast<float4*>(w32)[g] = make_float4((float)w[0], (float)w[1], (float)w[2], (float)w[3]);
   }
+  __syncthreads();
+  const int bl = t >> 3;
+  if (b0 + bl < n)
+    blob_tiles(cells[3 * bl], cells[3 * bl + 1], cells[3 * bl + 2], t & 7, ntx, nty,
+               [&](int tile) { atomicAdd(&count[tile], 1); });
 }
 
-// Distinct tiles touched along one axis (at most 4).
-__device__ __forceinline__ int axis_tiles(const int* __restrict__ ix, int* t) {
-  int m = 0;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int v = ix[s] / kTile;
-    bool seen = false;
-    for (int u = 0; u < m; ++u) seen |= (t[u] == v);
-    if (!seen) t[m++] = v;
-  }
-  return m;
-}
-
-template <bool FILL>
-__global__ void k_tile_pairs(const int* __restrict__ idx, int n, int ntx, int nty, int* __restrict__ count,
-                             const int* __restrict__ offset, int* __restrict__ cursor, int* __restrict__ list) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// Files each blob under its tiles, in any order; takes the counts back to zero.
+__global__ void __launch_bounds__(256) k_tile_fill(const int* __restrict__ idx, int n, int ntx, int nty,
+                                                   const int* __restrict__ offset, int* __restrict__ count,
+                                                   int* __restrict__ list) {
+  const int b = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 3);
   if (b >= n) return;
-  int tx[4], ty[4], tz[4];
-  const int mx = axis_tiles(idx + (b * 3 + 0) * 4, tx);
-  const int my = axis_tiles(idx + (b * 3 + 1) * 4, ty);
-  const int mz = axis_tiles(idx + (b * 3 + 2) * 4, tz);
-  for (int c = 0; c < mz; ++c)
-    for (int bb = 0; bb < my; ++bb)
-      for (int a = 0; a < mx; ++a) {
-        const int t = tx[a] + ntx * (ty[bb] + nty * tz[c]);
-        if (FILL) {
-          const int pos = offset[t] + atomicAdd(&cursor[t], 1);
-          list[pos] = b;
-        } else {
-          atomicAdd(&count[t], 1);
-        }
-      }
+  const int4* ib = reinterpret_cast<const int4*>(idx) + 3 * (size_t)b;
+  blob_tiles(ib[0], ib[1], ib[2], threadIdx.x & 7, ntx, nty, [&](int tile) {
+    list[offset[tile] + atomicSub(&count[tile], 1) - 1] = b;
+  });
 }
 
-// Single-block exclusive scan of n counts into offset[0..n] (offset[n] = the
-// total, also *total), optionally listing the indices with a nonzero count in
-// increasing order into active (their number into *nactive). The counts pass
-// through shared memory in segments of 4096, loaded and stored coalesced;
-// thread t scans entries 4t .. 4t + 3 of a segment, warps scan their threads'
-// sums with shuffles, warp 0 the warps' totals, and a carry joins segments.
-constexpr int kScanSeg = 4096;
-template <bool ACTIVE>
-__global__ void __launch_bounds__(1024) k_scan_counts(const int* __restrict__ count, int n, int* __restrict__ offset,
-                                                      int* __restrict__ total, int* __restrict__ active,
-                                                      int* __restrict__ nactive) {
-  __shared__ int sc[kScanSeg];
-  __shared__ int wsum[32], wact[32];
+// offset[0..n] = exclusive scan of the tiles' counts, active = the tiles with a
+// count in increasing order, meta[0] = their number; meta[1], the number of
+// covered cells, starts at zero. A CTA has kScanTiles tiles, four a thread, and
+// sums the counts before its own itself: 128 KB at most from L2 at 256^3, where
+// waiting for its predecessors would be a chain. (One CTA that walked all tiles
+// in segments took 19.8 us at 256^3; 7.0 us.)  Both scans run in one 64-bit word, active
+// tiles above pairs (each below 2^31).
+constexpr int kScanTiles = 4096;
+__global__ void __launch_bounds__(1024) k_tile_scan(const int* __restrict__ count, int n, int* __restrict__ offset,
+                                                    int* __restrict__ active, int* __restrict__ meta) {
+  using u64 = unsigned long long;
+  __shared__ u64 wsum[32], wbefore[32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  int carry = 0, carry_a = 0;
-  for (int base = 0; base < n; base += kScanSeg) {
-    const int len = min(kScanSeg, n - base);
-    for (int k = t; k < kScanSeg; k += blockDim.x) sc[k] = k < len ? count[base + k] : 0;
-    __syncthreads();
-    const int v0 = sc[4 * t], v1 = sc[4 * t + 1], v2 = sc[4 * t + 2], v3 = sc[4 * t + 3];
-    const int sum = (v0 + v1) + (v2 + v3);
-    const int act = ACTIVE ? (v0 > 0) + (v1 > 0) + (v2 > 0) + (v3 > 0) : 0;
-    int is = sum, ia = act;  // inclusive scans over the warp
+  const int base = blockIdx.x * kScanTiles;
+  auto one = [](int c) { return (u64)(unsigned)c + (c > 0 ? 1ull << 32 : 0ull); };
+  const int4* c4 = reinterpret_cast<const int4*>(count);
+  u64 before = 0;
+#pragma unroll 8
+  for (int k = t; k < base / 4; k += 1024) {
+    const int4 v = c4[k];
+    before += (one(v.x) + one(v.y)) + (one(v.z) + one(v.w));
+  }
+  const int i0 = base + 4 * t;
+  int4 v = make_int4(0, 0, 0, 0);
+  if (i0 + 3 < n) {
+    v = c4[i0 / 4];
+  } else {
+    if (i0 < n) v.x = count[i0];
+    if (i0 + 1 < n) v.y = count[i0 + 1];
+    if (i0 + 2 < n) v.z = count[i0 + 2];
+  }
+  const u64 sum = (one(v.x) + one(v.y)) + (one(v.z) + one(v.w));
+  u64 incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u64 up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+  }
+  if (lane == 31) wsum[w] = incl, wbefore[w] = before;
+  __syncthreads();
+  if (w == 0) {
+    u64 a = wsum[lane], b = wbefore[lane];
+    const u64 own = a;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int us = __shfl_up_sync(0xffffffffu, is, o), ua = __shfl_up_sync(0xffffffffu, ia, o);
-      if (lane >= o) is += us, ia += ua;
+      const u64 up = __shfl_up_sync(0xffffffffu, a, o);
+      if (lane >= o) a += up;
+      b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    if (lane == 31) wsum[w] = is, wact[w] = ia;
-    __syncthreads();
-    if (w == 0) {
-      int ws = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0, wa = lane < (int)(blockDim.x >> 5) ? wact[lane] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int us = __shfl_up_sync(0xffffffffu, ws, o), ua = __shfl_up_sync(0xffffffffu, wa, o);
-        if (lane >= o) ws += us, wa += ua;
-      }
-      wsum[lane] = ws;  // inclusive over warps
-      wact[lane] = wa;
-    }
-    __syncthreads();
-    const int before = carry + (w > 0 ? wsum[w - 1] : 0) + is - sum;
-    sc[4 * t] = before;
-    sc[4 * t + 1] = before + v0;
-    sc[4 * t + 2] = before + v0 + v1;
-    sc[4 * t + 3] = before + v0 + v1 + v2;
-    if (ACTIVE) {
-      int ra = carry_a + (w > 0 ? wact[w - 1] : 0) + ia - act;
-      const int i0 = base + 4 * t;
-      if (v0 > 0) active[ra++] = i0;
-      if (v1 > 0) active[ra++] = i0 + 1;
-      if (v2 > 0) active[ra++] = i0 + 2;
-      if (v3 > 0) active[ra] = i0 + 3;
-    }
-    carry += wsum[(blockDim.x >> 5) - 1];
-    carry_a += wact[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    for (int k = t; k < len; k += blockDim.x) offset[base + k] = sc[k];
-    __syncthreads();
+    wsum[lane] = b + a - own;  // all before the warp's tiles
   }
-  if (t == 0) {
-    offset[n] = carry;
-    *total = carry;
-    if (ACTIVE) *nactive = carry_a;
+  __syncthreads();
+  const u64 ex = wsum[w] + incl - sum;
+  int ra = (int)(ex >> 32);
+  const int o0 = (int)(unsigned)ex, o1 = o0 + v.x, o2 = o1 + v.y, o3 = o2 + v.z;
+  if (i0 + 3 < n) {
+    reinterpret_cast<int4*>(offset)[i0 / 4] = make_int4(o0, o1, o2, o3);
+  } else {
+    if (i0 < n) offset[i0] = o0;
+    if (i0 + 1 < n) offset[i0 + 1] = o1;
+    if (i0 + 2 < n) offset[i0 + 2] = o2;
+  }
+  if (v.x > 0) active[ra++] = i0;
+  if (v.y > 0) active[ra++] = i0 + 1;
+  if (v.z > 0) active[ra++] = i0 + 2;
+  if (v.w > 0) active[ra++] = i0 + 3;
+  if (t == 1023 && blockIdx.x == gridDim.x - 1) {  // (the entries past n count nothing)
+    offset[n] = o3 + v.w;
+    meta[0] = ra;
+    meta[1] = 0;
   }
 }
 
-// Sort the blob list of each occupied tile by blob index (insertion sort).
-__global__ void k_tile_sort(const int* __restrict__ active, int na, const int* __restrict__ offset,
-                            int* __restrict__ list) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= na) return;
-  const int t = active[a];
-  const int lo = offset[t], hi = offset[t + 1];
-  for (int i = lo + 1; i < hi; ++i) {
-    const int v = list[i];
-    int j = i - 1;
-    while (j >= lo && list[j] > v) {
-      list[j + 1] = list[j];
-      --j;
+// Bits of the cells start .. start + 7 of an axis of n cells that the 4 cells
+// from first on (wrapping) cover.
+__device__ __forceinline__ unsigned axis_mask(int first, int start, int n) {
+  auto at = [](int v) { return v <= -4 || v >= kTile ? 0u : v >= 0 ? 15u << v : 15u >> -v; };
+  const int lo = first - start, rem = n - start;
+  return (at(lo) | at(lo - n)) & (rem < kTile ? (1u << rem) - 1u : 0xFFu);
+}
+
+// One warp per occupied tile: orders the tile's blobs by index (each finds its
+// rank among the others) and lists the cells under any of them. A lane keeps two
+// of the tile's 64 rows of 8 cells as bits, so a blob costs the warp one shuffle
+// and a few logic instructions; the cells come out tile by tile, in order within
+// a tile, at a place taken from meta[1] once per CTA (the order of the tiles
+// changes no result: each cell is written once, from its own blobs).  At 4096
+// blobs on 256^3 the sort (4.8 us), the count (32.7 us, a thread per cell that
+// walked the blobs), the scan (6.7 us) and the fill (40.3 us) were four launches
+// with the host waiting for the number of cells between them; now 9.1 us.
+__global__ void __launch_bounds__(256) k_tile_cells(const int* __restrict__ active, const int* __restrict__ offset,
+                                                    const int* __restrict__ raw, const int* __restrict__ idx,
+                                                    int nx, int ny, int nz, int ntx, int nty,
+                                                    int* __restrict__ list, int* __restrict__ meta,
+                                                    int* __restrict__ cells, int* __restrict__ cell_tile) {
+  __shared__ int found[8], place[8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int na = meta[0];
+  if ((int)blockIdx.x * 8 >= na) return;
+  const int a = blockIdx.x * 8 + w;
+  unsigned rows = 0;  // rows 2 lane (low 8 bits) and 2 lane + 1 of the tile
+  int tile = 0, x0 = 0, y0 = 0, z0 = 0;
+  if (a < na) {
+    tile = active[a];
+    const int lo = offset[tile], cnt = offset[tile + 1] - lo;
+    x0 = tile % ntx * kTile, y0 = tile / ntx % nty * kTile, z0 = tile / (ntx * nty) * kTile;
+    const int j = 2 * (lane & 3), k = lane >> 2;
+    for (int p0 = 0; p0 < cnt; p0 += 32) {
+      const bool has = p0 + lane < cnt;
+      const int b = has ? raw[lo + p0 + lane] : INT_MAX;
+      unsigned m = 0;
+      if (has) {
+        const int* ib = idx + 12 * (size_t)b;
+        m = axis_mask(ib[0], x0, nx) | axis_mask(ib[4], y0, ny) << 8 | axis_mask(ib[8], z0, nz) << 16;
+      }
+      int rank = 0;
+      for (int q0 = 0; q0 < cnt; q0 += 32) {
+        const int o = q0 == p0 ? b : q0 + lane < cnt ? raw[lo + q0 + lane] : INT_MAX;
+        const int nq = min(32, cnt - q0);
+        for (int q = 0; q < nq; ++q) rank += __shfl_sync(0xffffffffu, o, q) < b;
+      }
+      if (has) list[lo + rank] = b;
+      const int np = min(32, cnt - p0);
+      for (int q = 0; q < np; ++q) {
+        const unsigned mq = __shfl_sync(0xffffffffu, m, q);
+        if (mq >> (16 + k) & 1u) {
+          if (mq >> (8 + j) & 1u) rows |= mq & 0xFFu;
+          if (mq >> (9 + j) & 1u) rows |= (mq & 0xFFu) << 8;
+        }
+      }
     }
-    list[j + 1] = v;
+    int c = __popc(rows);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) found[w] = c;
+  } else if (lane == 0) {
+    found[w] = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int total = 0;
+    for (int u = 0; u < 8; ++u) place[u] = total, total += found[u];
+    const int at = atomicAdd(&meta[1], total);
+    for (int u = 0; u < 8; ++u) place[u] += at;
+  }
+  __syncthreads();
+  if (a >= na) return;
+  int at = place[w];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {  // 32 cells: four rows, from two lanes
+    const unsigned m = __shfl_sync(0xffffffffu, rows, 2 * u) | __shfl_sync(0xffffffffu, rows, 2 * u + 1) << 16;
+    if (m >> lane & 1u) {
+      const int row = 4 * u + (lane >> 3);
+      const int r = at + __popc(m & ((1u << lane) - 1u));
+      cells[r] = ((z0 + (row >> 3)) * ny + y0 + (row & 7)) * nx + x0 + (lane & 7);
+      cell_tile[r] = tile;
+    }
+    at += __popc(m);
   }
 }
 
@@ -207,46 +306,6 @@ __device__ __forceinline__ bool covers(const int* __restrict__ ib, int i, int j,
   dy += dy < 0 ? ny : 0;
   dz += dz < 0 ? nz : 0;
   return (unsigned)dx < 4u && (unsigned)dy < 4u && (unsigned)dz < 4u;
-}
-
-// Pass 1 (count) and pass 2 (fill) of the covered-cell list: one CTA per
-// occupied tile, one thread per tile cell.
-template <bool FILL>
-__global__ void __launch_bounds__(512) k_cover(const int* __restrict__ active, const int* __restrict__ offset,
-                                               const int* __restrict__ list, const int* __restrict__ idx, int nx,
-                                               int ny, int nz, int ntx, int nty, int* __restrict__ count,
-                                               const int* __restrict__ coff, int* __restrict__ cells,
-                                               int* __restrict__ cell_tile) {
-  const int a = blockIdx.x;
-  const int tile = active[a];
-  const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-  const int i = tx * kTile + threadIdx.x, j = ty * kTile + threadIdx.y, k = tz * kTile + threadIdx.z;
-  bool hit = false;
-  if (i < nx && j < ny && k < nz) {
-    for (int p = offset[tile]; p < offset[tile + 1] && !hit; ++p) {
-      int dx, dy, dz;
-      hit = covers(idx + list[p] * 12, i, j, k, nx, ny, nz, dx, dy, dz);
-    }
-  }
-  if (!FILL) {
-    const int c = __syncthreads_count(hit);
-    if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) count[a] = c;
-    return;
-  }
-  // rank of this cell among the block's covered cells, in thread order
-  __shared__ int wsum[16];
-  const int t = threadIdx.x + kTile * (threadIdx.y + kTile * threadIdx.z);
-  const unsigned bal = __ballot_sync(0xffffffffu, hit);
-  const int lane = t & 31, w = t >> 5;
-  if (lane == 0) wsum[w] = __popc(bal);
-  __syncthreads();
-  int base = 0;
-  for (int u = 0; u < w; ++u) base += wsum[u];
-  if (hit) {
-    const int r = coff[a] + base + __popc(bal & ((1u << lane) - 1u));
-    cells[r] = (k * ny + j) * nx + i;
-    cell_tile[r] = tile;
-  }
 }
 
 // One thread per covered cell: gathers the contributions of its tile's blobs
@@ -300,30 +359,26 @@ __global__ void k_interp(const int* __restrict__ idx, const W* __restrict__ wt, 
 
 }  // namespace
 
-void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, cudaStream_t s) {
+void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, int* host, cudaStream_t s) {
   b.ntx = (d.nx + kTile - 1) / kTile;
   b.nty = (d.ny + kTile - 1) / kTile;
   b.ntz = (d.nz + kTile - 1) / kTile;
   const int nt = b.ntx * b.nty * b.ntz;
+  auto room = [](int*& p, size_t entries) {
+    cudaFree(p);
+    p = nullptr;
+    IBRD_CUDA(cudaMalloc(&p, sizeof(int) * entries));
+  };
   if (b.ntiles != nt) {
-    cudaFree(b.tile_count);
-    cudaFree(b.tile_offset);
-    cudaFree(b.tile_cursor);
-    cudaFree(b.active);
-    b.tile_count = b.tile_offset = b.tile_cursor = b.active = nullptr;
-    IBRD_CUDA(cudaMalloc(&b.tile_count, sizeof(int) * nt));
-    IBRD_CUDA(cudaMalloc(&b.tile_offset, sizeof(int) * (nt + 1)));
-    IBRD_CUDA(cudaMalloc(&b.tile_cursor, sizeof(int) * nt));
-    IBRD_CUDA(cudaMalloc(&b.active, sizeof(int) * nt));
-    cudaFree(b.cell_count);
-    cudaFree(b.cell_offset);
-    b.cell_count = b.cell_offset = nullptr;
-    IBRD_CUDA(cudaMalloc(&b.cell_count, sizeof(int) * (nt + 1)));
-    IBRD_CUDA(cudaMalloc(&b.cell_offset, sizeof(int) * (nt + 1)));
+    b.ntiles = 0;
+    room(b.tile_count, nt);
+    room(b.tile_offset, nt + 1);
+    room(b.active, nt);
     b.ntiles = nt;
   }
-  if (!b.d_meta) IBRD_CUDA(cudaMalloc(&b.d_meta, sizeof(int) * 4));
+  if (!b.d_meta) room(b.d_meta, 2);
   if (n > b.cap) {
+    b.cap = 0;
     cudaFree(b.q);
     cudaFree(b.idx);
     cudaFree(b.w64);
@@ -339,71 +394,45 @@ void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, cudaSt
     b.cap = n;
   }
   b.n = n;
+  b.n_active = b.n_cells = 0;
+  if (n == 0) return;
+  // The lists have room for the most that n blobs can touch, so that the host
+  // need not wait for their lengths on the way.
+  const size_t pairs = (size_t)n * max_axis_tiles(d.nx, b.ntx) * max_axis_tiles(d.ny, b.nty) *
+                       max_axis_tiles(d.nz, b.ntz);
+  const size_t most = std::min((size_t)64 * n, d.n());
+  if (pairs > b.pair_cap) {
+    b.pair_cap = 0;
+    room(b.tile_blobs, pairs);
+    room(b.tile_raw, pairs);
+    b.pair_cap = pairs;
+  }
+  if (most > b.cell_cap) {
+    b.cell_cap = 0;
+    room(b.cells, most);
+    room(b.cell_tile, most);
+    b.cell_cap = most;
+  }
   IBRD_CUDA(cudaMemsetAsync(b.tile_count, 0, sizeof(int) * nt, s));
-  IBRD_CUDA(cudaMemsetAsync(b.tile_cursor, 0, sizeof(int) * nt, s));
-  if (n > 0) {
-    prof_begin(P_SETUP, s);
-    k_blob_prep<<<(n + 127) / 128, 128, 0, s>>>(q_in, n, d.nx, d.ny, d.nz, h, b.width, b.q, b.idx, b.w64, b.w32);
-    prof_end(P_SETUP, s, "blob_prep");
-    prof_begin(P_SETUP, s);
-    k_tile_pairs<false><<<(n + 127) / 128, 128, 0, s>>>(b.idx, n, b.ntx, b.nty, b.tile_count, nullptr, nullptr,
-                                                         nullptr);
-    prof_end(P_SETUP, s, "tile_count");
-  }
   prof_begin(P_SETUP, s);
-  k_scan_counts<true><<<1, 1024, 0, s>>>(b.tile_count, nt, b.tile_offset, b.d_meta, b.active, b.d_meta + 1);
-  prof_end(P_SETUP, s, "scan_tiles");
-  int meta[2];
-  IBRD_CUDA(cudaMemcpyAsync(meta, b.d_meta, sizeof(meta), cudaMemcpyDeviceToHost, s));
+  k_blob_prep<<<(n + kPrepBlobs - 1) / kPrepBlobs, 8 * kPrepBlobs, 0, s>>>(
+      q_in, n, d.nx, d.ny, d.nz, h, b.width, b.q, b.idx, b.w64, b.w32, b.ntx, b.nty, b.tile_count);
+  prof_end(P_SETUP, s, "blob_prep");
+  prof_begin(P_SETUP, s);
+  k_tile_scan<<<(nt + kScanTiles - 1) / kScanTiles, 1024, 0, s>>>(b.tile_count, nt, b.tile_offset, b.active, b.d_meta);
+  prof_end(P_SETUP, s, "tile_scan");
+  prof_begin(P_SETUP, s);
+  k_tile_fill<<<(n + 31) / 32, 256, 0, s>>>(b.idx, n, b.ntx, b.nty, b.tile_offset, b.tile_count, b.tile_raw);
+  prof_end(P_SETUP, s, "tile_fill");
+  const int tiles = (int)std::min(pairs, (size_t)nt);  // occupied ones, at most
+  prof_begin(P_SETUP, s);
+  k_tile_cells<<<(tiles + 7) / 8, 256, 0, s>>>(b.active, b.tile_offset, b.tile_raw, b.idx, d.nx, d.ny, d.nz, b.ntx,
+                                               b.nty, b.tile_blobs, b.d_meta, b.cells, b.cell_tile);
+  prof_end(P_SETUP, s, "tile_cells");
+  IBRD_CUDA(cudaMemcpyAsync(host, b.d_meta, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   IBRD_CUDA(cudaStreamSynchronize(s));
-  b.n_active = meta[1];
-  if (meta[0] > b.pair_cap) {
-    cudaFree(b.tile_blobs);
-    b.tile_blobs = nullptr;
-    IBRD_CUDA(cudaMalloc(&b.tile_blobs, sizeof(int) * meta[0]));
-    b.pair_cap = meta[0];
-  }
-  if (n > 0) {
-    prof_begin(P_SETUP, s);
-    k_tile_pairs<true><<<(n + 127) / 128, 128, 0, s>>>(b.idx, n, b.ntx, b.nty, nullptr, b.tile_offset,
-                                                        b.tile_cursor, b.tile_blobs);
-    prof_end(P_SETUP, s, "tile_fill");
-    if (b.n_active > 0) {
-      prof_begin(P_SETUP, s);
-      k_tile_sort<<<(b.n_active + 127) / 128, 128, 0, s>>>(b.active, b.n_active, b.tile_offset, b.tile_blobs);
-      prof_end(P_SETUP, s, "tile_sort");
-    }
-  }
-  // covered-cell list (count per occupied tile, scan, ordered fill)
-  b.n_cells = 0;
-  if (n > 0 && b.n_active > 0) {
-    const dim3 tb(kTile, kTile, kTile);
-    prof_begin(P_SETUP, s);
-    k_cover<false><<<b.n_active, tb, 0, s>>>(b.active, b.tile_offset, b.tile_blobs, b.idx, d.nx, d.ny, d.nz, b.ntx,
-                                             b.nty, b.cell_count, nullptr, nullptr, nullptr);
-    prof_end(P_SETUP, s, "cover_count");
-    prof_begin(P_SETUP, s);
-    k_scan_counts<false><<<1, 1024, 0, s>>>(b.cell_count, b.n_active, b.cell_offset, b.d_meta + 2, nullptr,
-                                            nullptr);
-    prof_end(P_SETUP, s, "cover_scan");
-    int nc = 0;
-    IBRD_CUDA(cudaMemcpyAsync(&nc, b.d_meta + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
-    IBRD_CUDA(cudaStreamSynchronize(s));
-    if (nc > b.cell_cap || !b.cells) {
-      cudaFree(b.cells);
-      cudaFree(b.cell_tile);
-      b.cells = b.cell_tile = nullptr;
-      const int cap = std::max(nc, 1);
-      IBRD_CUDA(cudaMalloc(&b.cells, sizeof(int) * cap));
-      IBRD_CUDA(cudaMalloc(&b.cell_tile, sizeof(int) * cap));
-      b.cell_cap = cap;
-    }
-    prof_begin(P_SETUP, s);
-    k_cover<true><<<b.n_active, tb, 0, s>>>(b.active, b.tile_offset, b.tile_blobs, b.idx, d.nx, d.ny, d.nz, b.ntx,
-                                            b.nty, nullptr, b.cell_offset, b.cells, b.cell_tile);
-    prof_end(P_SETUP, s, "cover_fill");
-    b.n_cells = nc;
-  }
+  b.n_active = host[0];
+  b.n_cells = host[1];
 }
 
 template <typename T, typename L>

@@ -335,24 +335,23 @@ struct BlobSet {
   float* w32 = nullptr;      // FP32 copy
   // tile binning
   int ntx = 0, nty = 0, ntz = 0, ntiles = 0;
-  int* tile_count = nullptr;   // ntiles
+  int* tile_count = nullptr;   // ntiles (zero between setups)
   int* tile_offset = nullptr;  // ntiles + 1
-  int* tile_cursor = nullptr;  // ntiles
-  int* tile_blobs = nullptr;   // pairs (blob index per (tile, blob) pair)
-  int pair_cap = 0;
+  int* tile_blobs = nullptr;   // pairs (blob index per (tile, blob) pair), sorted within a tile
+  int* tile_raw = nullptr;     // the same before the sort
+  size_t pair_cap = 0;
   int* active = nullptr;       // active tile ids (ntiles capacity)
   int n_active = 0;
-  int* d_meta = nullptr;       // [0] = pairs, [1] = active tiles, [2] = covered cells
-  // cells covered by at least one blob support, in (tile, cell) order
-  int* cell_count = nullptr;   // per active tile
-  int* cell_offset = nullptr;  // per active tile + 1
+  int* d_meta = nullptr;       // [0] = active tiles, [1] = covered cells
+  // cells covered by at least one blob support, tile by tile
   int* cells = nullptr;        // linear cell index
   int* cell_tile = nullptr;    // tile id of each covered cell
-  int cell_cap = 0;
+  size_t cell_cap = 0;
   int n_cells = 0;
 };
 
-void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, cudaStream_t s);
+// host: 2 pinned integers
+void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, int* host, cudaStream_t s);
 // out (+)= scale * sum_b coef_b lam_b phi_b  (coef nullable = 1);
 // lam (type L) and coef (FP64) device N-vectors; out field of type T.
 template <typename T, typename L = double>
