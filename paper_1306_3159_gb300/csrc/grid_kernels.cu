@@ -16,21 +16,25 @@
 namespace ibrd {
 namespace {
 
-constexpr int BX = 32, BY = 8, ZCH = 16;
+constexpr int BX = 32, BY = 8;
 
 __device__ __forceinline__ int wrap_dec(int i, int n) { return i == 0 ? n - 1 : i - 1; }
 __device__ __forceinline__ int wrap_inc(int i, int n) { return i == n - 1 ? 0 : i + 1; }
 
 // y = A x (RESID = false) or y = b - A x (RESID = true); 2.5D z-march with the
-// z-neighbours kept in registers and x/y neighbours served by L1.
+// z-neighbours kept in registers and x/y neighbours served by L1. Seven FP64
+// instructions per cell bound it (two lanes per SM and clock): 229 us at 256^3,
+// 83 % of that rate. (Sharing the sums of x- and y-neighbours along diagonals
+// makes it six, but four cells per thread leave too few warps: 251 us.)
 template <typename T, bool RESID>
 __global__ void __launch_bounds__(BX* BY) k_apply(const T* __restrict__ x, const T* __restrict__ b,
-                                                  T* __restrict__ y, int nx, int ny, int nz, T diag, T off) {
+                                                  T* __restrict__ y, int nx, int ny, int nz, int zc, T diag,
+                                                  T off) {
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   if (i >= nx || j >= ny) return;
-  const int k0 = blockIdx.z * ZCH;
-  const int k1 = min(k0 + ZCH, nz);
+  const int k0 = blockIdx.z * zc;
+  const int k1 = min(k0 + zc, nz);
   const int im = wrap_dec(i, nx), ip = wrap_inc(i, nx);
   const size_t plane = (size_t)nx * ny;
   const size_t rj = (size_t)j * nx, rjm = (size_t)wrap_dec(j, ny) * nx, rjp = (size_t)wrap_inc(j, ny) * nx;
@@ -1041,6 +1045,19 @@ inline int stream_blocks(size_t n, int threads) {
   return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
+// Blocks of k_apply and planes per block. What counts is the most planes that one
+// SM gets, a block's march costing about one more for its start: 16 planes a block
+// left 32^3 on 8 SMs (14.5 us; 3.5 with one plane each) and gave 96^3 two blocks
+// on some SMs and one on others (20.6 us; 16.1 with 12 planes). 16 stays where it is as good.
+dim3 apply_grid(Dims d, int& zc) {
+  const int bx = (d.nx + BX - 1) / BX, by = (d.ny + BY - 1) / BY;
+  auto cost = [&](int z) { return ((long long)bx * by * ((d.nz + z - 1) / z) + 151) / 152 * (z + 1); };
+  zc = 16;
+  for (int z = 15; z >= 1; --z)
+    if (cost(z) < cost(zc)) zc = z;
+  return dim3(bx, by, (d.nz + zc - 1) / zc);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
@@ -1064,9 +1081,10 @@ void launch_apply_A(const T* x, T* y, Dims d, Stencil st, cudaStream_t s) {
       return;
     }
   }
-  dim3 g((d.nx + BX - 1) / BX, (d.ny + BY - 1) / BY, (d.nz + ZCH - 1) / ZCH);
+  int zc;
+  const dim3 g = apply_grid(d, zc);
   prof_begin(c, s);
-  k_apply<T, false><<<g, dim3(BX, BY), 0, s>>>(x, nullptr, y, d.nx, d.ny, d.nz, (T)st.diag, (T)st.off);
+  k_apply<T, false><<<g, dim3(BX, BY), 0, s>>>(x, nullptr, y, d.nx, d.ny, d.nz, zc, (T)st.diag, (T)st.off);
   prof_end(c, s, "apply_A", 2.0 * sizeof(T) * d.n());
 }
 
@@ -1113,9 +1131,10 @@ void launch_residual(const T* x, const T* b, T* y, Dims d, Stencil st, double* s
       return;
     }
   }
-  dim3 g((d.nx + BX - 1) / BX, (d.ny + BY - 1) / BY, (d.nz + ZCH - 1) / ZCH);
+  int zc;
+  const dim3 g = apply_grid(d, zc);
   prof_begin(c, s);
-  k_apply<T, true><<<g, dim3(BX, BY), 0, s>>>(x, b, y, d.nx, d.ny, d.nz, (T)st.diag, (T)st.off);
+  k_apply<T, true><<<g, dim3(BX, BY), 0, s>>>(x, b, y, d.nx, d.ny, d.nz, zc, (T)st.diag, (T)st.off);
   prof_end(c, s, "residual", 3.0 * sizeof(T) * d.n());
 }
 
