@@ -1051,10 +1051,14 @@ inline int stream_blocks(size_t n, int threads) {
 // on some SMs and one on others (20.6 us; 16.1 with 12 planes). 16 stays where it is as good.
 dim3 apply_grid(Dims d, int& zc) {
   const int bx = (d.nx + BX - 1) / BX, by = (d.ny + BY - 1) / BY;
-  auto cost = [&](int z) { return ((long long)bx * by * ((d.nz + z - 1) / z) + 151) / 152 * (z + 1); };
+  const unsigned columns = (unsigned)bx * by, nz = d.nz;
+  auto cost = [&](unsigned z) { return (columns * ((nz + z - 1) / z) + 151) / 152 * (z + 1); };
   zc = 16;
-  for (int z = 15; z >= 1; --z)
-    if (cost(z) < cost(zc)) zc = z;
+  unsigned best = cost(16);
+  for (unsigned z = 15; z >= 1; --z) {
+    const unsigned c = cost(z);
+    if (c < best) best = c, zc = (int)z;
+  }
   return dim3(bx, by, (d.nz + zc - 1) / zc);
 }
 
