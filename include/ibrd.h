@@ -204,7 +204,9 @@ void ibrd_grid_destroy(ibrd_grid g);
    of N x 3 FP64 values (x, y, z per blob, AoS). Positions are wrapped into the
    periodic box. Computes each blob's 1-D kernel weights and bins blobs by
    8 x 8 x 8 cell tile for spreading. N >= 0; N = 0 clears the blobs.
-   Synchronizes the stream (it reads back the number of occupied tiles). */
+   Synchronizes the stream (it reads back the number of covered cells).
+   A refused argument (IBRD_ERR_ARG, IBRD_ERR_NONFINITE) leaves the blobs as
+   they were; after IBRD_ERR_OOM or IBRD_ERR_CUDA the handle has none. */
 ibrd_status ibrd_set_blobs(ibrd_grid g, const double* q, int n_blobs);
 
 /* y = A c = alpha c - chi L c (Sec. III.A, Eq. Helmholtz). c and y must not

@@ -486,8 +486,13 @@ class Grid:
         return torch.full((nz, ny, nx), float(fill), dtype=torch.float64, device="cuda")
 
     def set_blobs(self, q):
+        try:
+            ibrd_set_blobs(self.handle, q)
+        except IbrdError as e:
+            if STATUS.get(e.status) in ("IBRD_ERR_OOM", "IBRD_ERR_CUDA"):
+                self.n_blobs = 0  # a refused argument keeps the old blobs, a failed set-up has none
+            raise
         self.n_blobs = int(q.shape[0])
-        ibrd_set_blobs(self.handle, q)
 
     def apply_L(self, c, y=None):
         y = self.field() if y is None else y

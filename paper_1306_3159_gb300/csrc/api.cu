@@ -2848,8 +2848,8 @@ ibrd_status ibrd_set_blobs(ibrd_grid g, const double* q, int n) {
     IBRD_CUDA(cudaMemcpyAsync(host, g->dflag, sizeof(int), cudaMemcpyDeviceToHost, g->s));
     IBRD_CUDA(cudaStreamSynchronize(g->s));
     if (*host) throw ArgError{IBRD_ERR_NONFINITE, "non-finite blob position"};
+    g->blob_version++;  // also when the set-up fails: the old blobs are gone then
     blobs_setup(g->blobs, g->d, g->h, q, n, host, g->s);
-    g->blob_version++;
     return IBRD_OK;
   });
 }

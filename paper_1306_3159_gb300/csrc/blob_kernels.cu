@@ -360,6 +360,9 @@ __global__ void k_interp(const int* __restrict__ idx, const W* __restrict__ wt, 
 }  // namespace
 
 void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, int* host, cudaStream_t s) {
+  // no blobs until everything of the new set is there: an allocation that fails
+  // on the way leaves a handle without blobs, whose calls read none of the arrays
+  b.n = b.n_cells = 0;
   b.ntx = (d.nx + kTile - 1) / kTile;
   b.nty = (d.ny + kTile - 1) / kTile;
   b.ntz = (d.nz + kTile - 1) / kTile;
@@ -393,8 +396,6 @@ void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, int* h
     IBRD_CUDA(cudaMalloc(&b.w32, sizeof(float) * 12 * n));
     b.cap = n;
   }
-  b.n = n;
-  b.n_active = b.n_cells = 0;
   if (n == 0) return;
   // The lists have room for the most that n blobs can touch, so that the host
   // need not wait for their lengths on the way.
@@ -431,8 +432,8 @@ void blobs_setup(BlobSet& b, Dims d, double h, const double* q_in, int n, int* h
   prof_end(P_SETUP, s, "tile_cells");
   IBRD_CUDA(cudaMemcpyAsync(host, b.d_meta, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   IBRD_CUDA(cudaStreamSynchronize(s));
-  b.n_active = host[0];
   b.n_cells = host[1];
+  b.n = n;
 }
 
 template <typename T, typename L>

@@ -335,13 +335,12 @@ struct BlobSet {
   float* w32 = nullptr;      // FP32 copy
   // tile binning
   int ntx = 0, nty = 0, ntz = 0, ntiles = 0;
-  int* tile_count = nullptr;   // ntiles (zero between setups)
+  int* tile_count = nullptr;   // ntiles
   int* tile_offset = nullptr;  // ntiles + 1
   int* tile_blobs = nullptr;   // pairs (blob index per (tile, blob) pair), sorted within a tile
   int* tile_raw = nullptr;     // the same before the sort
   size_t pair_cap = 0;
   int* active = nullptr;       // active tile ids (ntiles capacity)
-  int n_active = 0;
   int* d_meta = nullptr;       // [0] = active tiles, [1] = covered cells
   // cells covered by at least one blob support, tile by tile
   int* cells = nullptr;        // linear cell index
