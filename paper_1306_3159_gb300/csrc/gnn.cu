@@ -1092,6 +1092,7 @@ int grad_chunk(int n) { return std::max(kGradRows, (n + kGradChunks - 1) / kGrad
 void ensure_cap(ibrd_gnn m, int n) {
   if (n <= m->cap) return;
   const size_t N = (size_t)n, nb = (N + kWarps - 1) / kWarps;
+  m->cap = 0;  // a call after a failed allocation below allocates everything again
   galloc(&m->cnt, N);
   galloc(&m->p32, N);
   galloc(&m->nidx, N * m->kmax);
@@ -1150,6 +1151,7 @@ void neighbour_lists(ibrd_gnn m, const double* q, int n, double lx, double ly, d
   if (cl.nx && cl.ny && cl.nz) {
     const int ncell = cl.nx * cl.ny * cl.nz;
     if (ncell > m->cell_cap) {
+      m->cell_cap = 0;
       galloc(&m->cell_cnt, ncell);
       galloc(&m->cell_start, ncell + 1);
       galloc(&m->cell_cursor, ncell);

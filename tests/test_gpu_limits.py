@@ -80,3 +80,22 @@ def test_refused_blobs_keep_the_old_ones(ibrd):
         g.set_blobs(dev(bad))
     assert g.n_blobs == 9
     assert torch.equal(g.interp(c).cpu(), torch.from_numpy(want))
+
+
+def test_model_that_does_not_fit(ibrd):
+    """A blob takes about 8 KB here: 200 000 blobs do not fit 500
+    MB. A smaller call on the same model then allocates what it needs."""
+    import torch
+    q = torch.rand(200_000, 3, dtype=torch.float64, device="cuda") * 400.0
+    few = torch.rand(40, 3, dtype=torch.float64, device="cuda") * 40.0
+    lam = torch.rand(40, dtype=torch.float64, device="cuda") + 0.5
+    m = ibrd.GNN(6.0, 64)
+    m.init_params(3)
+    want, grad = m.predict(few, (40.0,) * 3, 40.0), m.loss_grad(few, (40.0,) * 3, lam)[1]
+    out = torch.empty(200_000, dtype=torch.float64, device="cuda")
+    with only(500):
+        with pytest.raises(ibrd.IbrdError) as e:
+            m.predict(q, (400.0,) * 3, 1.0, out)
+        assert "OOM" in str(e.value)
+    assert torch.equal(m.predict(few, (40.0,) * 3, 40.0), want)
+    assert torch.equal(m.loss_grad(few, (40.0,) * 3, lam)[1], grad)
