@@ -58,9 +58,8 @@ def test_blobs_that_do_not_fit(ibrd):
         assert "OOM" in str(e.value) and g.n_blobs == 0
         back.fill_(7.0)
         g.interp(cd, back)
-        assert bool((back == 7.0).all())
         g.spread(ld, out)
-        assert not bool(out.any())
+    assert bool((back == 7.0).all()) and not bool(out.any())
     g.set_blobs(dev(q))
     assert rel_max(host(g.spread(ld)), op.spread(lam, q, dims, 1.0, 4)) < 1e-13
 
