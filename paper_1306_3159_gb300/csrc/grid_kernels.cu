@@ -683,14 +683,18 @@ __device__ void fin_tail(const double* partial, const FinTail& t) {
 }
 
 // Sum of x. 16-byte vectors, four in flight per thread (vec; the last n % V
-// entries one by one): FP32 values are summed in FP32 over runs of 8 and the
-// runs in FP64 (two FP64 instructions per run, hidden behind the loads). 19 us
-// for a 256^3 FP32 field (67 MB) and 84 us at 512^3 (0.94 of the copy bandwidth);
-// 28 and 156 us with scalar loads and runs of 4.
+// entries one by one). FP32 values are summed in FP32 over runs of 4, a vector
+// each, and the runs in FP64; fields of less than kRunsFrom entries in FP64 alone.
+// (This sum is the mean taken off a singular right-hand side: longer runs in FP32
+// would cost it digits, and the loads hide one FP64 addition per run.)
+// 19 us for a 256^3 FP32 field (67 MB) and 85 us at 512^3 (0.93 of the copy bandwidth);
+// 28 and 156 us with scalar loads.
+constexpr size_t kRunsFrom = (size_t)4 * kRedBlocks * kRedThreads;  // 4 entries a thread
+
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict__ x, size_t n, int vec,
                                                              double* __restrict__ partial, FinTail tail) {
-  double acc = 0.0;
+  double acc = 0.0, acc1 = 0.0;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   size_t done = 0;
@@ -699,18 +703,21 @@ __global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict
       const size_t n4 = n >> 2;
       auto at = [&](size_t i) { return reinterpret_cast<const float4*>(x)[i]; };
       auto run = [](float4 v) { return (v.x + v.y) + (v.z + v.w); };
+      const bool runs = n >= kRunsFrom;
       size_t i = t;
-      for (; i + 3 * stride < n4; i += 4 * stride) {
+      for (; runs && i + 3 * stride < n4; i += 4 * stride) {
         const float4 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
-        acc += (double)(run(a) + run(b));
-        acc += (double)(run(c) + run(d));
+        acc += f2d_bits(run(a)) + f2d_bits(run(b));
+        acc1 += f2d_bits(run(c)) + f2d_bits(run(d));
       }
-      for (; i < n4; i += stride) acc += (double)run(at(i));
+      for (; i < n4; i += stride) {
+        const float4 v = at(i);
+        acc += runs ? f2d_bits(run(v)) : (f2d_bits(v.x) + f2d_bits(v.y)) + (f2d_bits(v.z) + f2d_bits(v.w));
+      }
       done = 4 * n4;
     } else {
       const size_t n2 = n >> 1;
       auto at = [&](size_t i) { return reinterpret_cast<const double2*>(x)[i]; };
-      double acc1 = 0.0;
       size_t i = t;
       for (; i + 3 * stride < n2; i += 4 * stride) {
         const double2 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
@@ -721,12 +728,11 @@ __global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict
         const double2 a = at(i);
         acc += a.x + a.y;
       }
-      acc += acc1;
       done = 2 * n2;
     }
   }
   for (size_t i = done + t; i < n; i += stride) acc += (double)x[i];
-  acc = block_sum(acc);
+  acc = block_sum(acc + acc1);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
   if (tail.ticket) fin_tail(partial, tail);
 }

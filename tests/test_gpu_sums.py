@@ -1,0 +1,48 @@
+"""What the streaming sums keep of their terms, through the launchers (-m gpu)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+P, Z, D = ctypes.c_void_p, ctypes.c_size_t, ctypes.c_double
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import paper_1306_3159_gb300 as p
+    return p.load_library()
+
+
+def launcher(lib, name, *args):
+    """A launcher of the library (C++ linkage; the last two arguments are its
+    stream and its ticket, none here)."""
+    import torch
+    f = getattr(lib, name)
+    f.argtypes, f.restype = list(args) + [P, P], None
+
+    def call(*values):
+        f(*[v.data_ptr() if isinstance(v, torch.Tensor) else v for v in values],
+          torch.cuda.current_stream().cuda_stream, None)
+    return call
+
+
+def scratch():
+    import torch
+    return torch.zeros(2 * 608, dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
+
+
+# a few entries; fields summed in FP64 alone, up to the last such size; the first
+# with runs, one and several vectors a thread, remainders
+@pytest.mark.parametrize("n", [1, 7, 1000, 262144, 622591, 622592, 1000003, 4000002])
+def test_runs_of_the_fp32_sum(lib, n):
+    """FP32 entries are added in FP32 over four of them at most (none in fields
+    below 622592): sums of four whole numbers below 2^22 (of one below 2^24) are
+    exact, longer ones are not, so the total is exact."""
+    import torch
+    x = np.random.default_rng(n).integers(1, 1 << (24 if n < 622592 else 22), n)
+    partial, out = scratch()
+    launcher(lib, "_ZN4ibrd10launch_sumIfEEvPKT_mPdS4_dP11CUstream_stPj", P, Z, P, P, D)(
+        torch.from_numpy(x.astype(np.float32)).cuda(), n, partial, out, 1.0)
+    assert out.item() == float(x.sum())
