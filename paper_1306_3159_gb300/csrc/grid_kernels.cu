@@ -682,54 +682,49 @@ __device__ void fin_tail(const double* partial, const FinTail& t) {
   if (threadIdx.x == 0) *t.ticket = 0u;
 }
 
-// Sum of x. 16-byte vectors, four in flight per thread (vec; the last n % V
-// entries one by one). FP32 values are summed in FP32 over runs of 4, a vector
-// each, and the runs in FP64; fields of less than kRunsFrom entries in FP64 alone.
-// (This sum is the mean taken off a singular right-hand side: longer runs in FP32
-// would cost it digits, and the loads hide one FP64 addition per run.)
-// 19 us for a 256^3 FP32 field (67 MB) and 85 us at 512^3 (0.93 of the copy bandwidth);
-// 28 and 156 us with scalar loads.
+// Sum of x. FP32: 16-byte vectors, four in flight per thread; the `head` entries
+// before the first 16-byte boundary and the last few one by one. The values are
+// summed in FP32 over runs of 4, a vector each, and the runs in FP64; fields of
+// less than kRunsFrom entries in FP64 alone. (This sum is the mean taken off a
+// singular right-hand side: longer runs in FP32 would cost it digits, and the
+// loads hide one FP64 addition per run.) 19 us for a 256^3 field (67 MB) and 85 us at
+// 512^3 (0.93 of the copy bandwidth), wherever the field starts; 28 and 156 us with
+// scalar loads in runs of 4, 72 and 508 us with one scalar load in flight and an FP64
+// addition for each. FP64: single entries, four in flight: 43 us at 256^3 and 268
+// at 512^3, where pairs took 44 and 282.
 constexpr size_t kRunsFrom = (size_t)4 * kRedBlocks * kRedThreads;  // 4 entries a thread
 
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict__ x, size_t n, int vec,
+__global__ void __launch_bounds__(kRedThreads) k_sum_partial(const T* __restrict__ x0, size_t n0, int head,
                                                              double* __restrict__ partial, FinTail tail) {
   double acc = 0.0, acc1 = 0.0;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  size_t done = 0;
-  if (vec) {
-    if constexpr (sizeof(T) == 4) {
-      const size_t n4 = n >> 2;
-      auto at = [&](size_t i) { return reinterpret_cast<const float4*>(x)[i]; };
-      auto run = [](float4 v) { return (v.x + v.y) + (v.z + v.w); };
-      const bool runs = n >= kRunsFrom;
-      size_t i = t;
-      for (; runs && i + 3 * stride < n4; i += 4 * stride) {
-        const float4 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
-        acc += f2d_bits(run(a)) + f2d_bits(run(b));
-        acc1 += f2d_bits(run(c)) + f2d_bits(run(d));
-      }
-      for (; i < n4; i += stride) {
-        const float4 v = at(i);
-        acc += runs ? f2d_bits(run(v)) : (f2d_bits(v.x) + f2d_bits(v.y)) + (f2d_bits(v.z) + f2d_bits(v.w));
-      }
-      done = 4 * n4;
-    } else {
-      const size_t n2 = n >> 1;
-      auto at = [&](size_t i) { return reinterpret_cast<const double2*>(x)[i]; };
-      size_t i = t;
-      for (; i + 3 * stride < n2; i += 4 * stride) {
-        const double2 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
-        acc += (a.x + a.y) + (b.x + b.y);
-        acc1 += (c.x + c.y) + (d.x + d.y);
-      }
-      for (; i < n2; i += stride) {
-        const double2 a = at(i);
-        acc += a.x + a.y;
-      }
-      done = 2 * n2;
+  const T* x = x0 + head;
+  const size_t n = n0 - head;
+  if (t < head) acc = (double)x0[t];
+  size_t done;
+  if constexpr (sizeof(T) == 4) {
+    const size_t n4 = n >> 2;
+    auto at = [&](size_t i) { return reinterpret_cast<const float4*>(x)[i]; };
+    auto run = [](float4 v) { return (v.x + v.y) + (v.z + v.w); };
+    const bool runs = n >= kRunsFrom;
+    size_t i = t;
+    for (; runs && i + 3 * stride < n4; i += 4 * stride) {
+      const float4 a = at(i), b = at(i + stride), c = at(i + 2 * stride), d = at(i + 3 * stride);
+      acc += f2d_bits(run(a)) + f2d_bits(run(b));
+      acc1 += f2d_bits(run(c)) + f2d_bits(run(d));
     }
+    for (; i < n4; i += stride) {
+      const float4 v = at(i);
+      acc += runs ? f2d_bits(run(v)) : (f2d_bits(v.x) + f2d_bits(v.y)) + (f2d_bits(v.z) + f2d_bits(v.w));
+    }
+    done = 4 * n4;
+  } else {
+    size_t i = t;
+    for (; i + 3 * stride < n; i += 4 * stride)
+      acc += (x[i] + x[i + stride]) + (x[i + 2 * stride] + x[i + 3 * stride]);
+    done = i - t;
   }
   for (size_t i = done + t; i < n; i += stride) acc += (double)x[i];
   acc = block_sum(acc + acc1);
@@ -1218,9 +1213,10 @@ template <typename T>
 void launch_sum(const T* x, size_t n, double* partial, double* out, double scale, cudaStream_t s, unsigned* ticket) {
   FinTail t;
   if (ticket) t = FinTail{ticket, out, scale, nullptr, 1.0};
-  const int nb = red_blocks(n);
+  const int nb = red_blocks(n), off = (int)((uintptr_t)x & 15u) / (int)sizeof(T);
+  const int head = sizeof(T) == 4 && off ? (int)std::min<size_t>(n, 4 - off) : 0;
   prof_begin(P_DOT, s);
-  k_sum_partial<T><<<nb, kRedThreads, 0, s>>>(x, n, aligned16(x), partial, t);
+  k_sum_partial<T><<<nb, kRedThreads, 0, s>>>(x, n, head, partial, t);
   prof_end(P_DOT, s, "sum_partial", 1.0 * sizeof(T) * n);
   if (ticket) return;
   prof_begin(P_REDUCE, s);

@@ -46,3 +46,35 @@ def test_runs_of_the_fp32_sum(lib, n):
     launcher(lib, "_ZN4ibrd10launch_sumIfEEvPKT_mPdS4_dP11CUstream_stPj", P, Z, P, P, D)(
         torch.from_numpy(x.astype(np.float32)).cuda(), n, partial, out, 1.0)
     assert out.item() == float(x.sum())
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("n,start", [(1, 1), (2, 3), (3, 2), (1000, 1), (1000003, 2), (1000001, 3), (1 << 25, 1)])
+def test_sum_off_a_boundary(lib, n, start, bits):
+    """Fields that start anywhere are summed whole (below 2^22: as above) and, being
+    bound by their one read, in the time of an aligned one, within a third."""
+    import torch
+    x = torch.randint(1, 1 << 22, (n + 4,), device="cuda")
+    total = float(x[start:start + n].sum())
+    x = x.to(torch.float32 if bits == 32 else torch.float64)
+    partial, out = scratch()
+    kind = "f" if bits == 32 else "d"
+    add = launcher(lib, f"_ZN4ibrd10launch_sumI{kind}EEvPKT_mPdS4_dP11CUstream_stPj", P, Z, P, P, D)
+    add(x[start:], n, partial, out, 1.0)
+    assert out.item() == total
+    if n < 1 << 25:
+        return
+
+    def time(field):
+        best = 1e9
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(4):
+                add(field, n, partial, out, 1.0)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    assert time(x[start:]) < 4 / 3 * time(x)
