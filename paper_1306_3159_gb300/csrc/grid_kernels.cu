@@ -648,6 +648,28 @@ __device__ __forceinline__ double block_sum_f(float v) {
   return d;
 }
 
+// The same for four values per thread, each folded over the warp by itself: every
+// fold passes on half of what a lane holds until one value is left, whose sum
+// over the warp is then in eight lanes; the 32 totals are a value per lane of warp 0.
+__device__ __forceinline__ double block_sum_f(float4 v) {
+  static_assert(kRedThreads == 256, "8 warps of 4 values");
+  __shared__ float sw[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool h = lane & 16, q = lane & 8;
+  float a = h ? v.z : v.x, b = h ? v.w : v.y;
+  a += __shfl_xor_sync(0xffffffffu, h ? v.x : v.z, 16);
+  b += __shfl_xor_sync(0xffffffffu, h ? v.y : v.w, 16);
+  float c = (q ? b : a) + __shfl_xor_sync(0xffffffffu, q ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if ((lane & 7) == 0) sw[4 * wid + (lane >> 3)] = c;
+  __syncthreads();
+  double d = 0.0;
+  if (wid == 0) d = warp_sum(f2d_bits(sw[lane]));
+  __syncthreads();
+  return d;
+}
+
 // Optional tail of a partial-sum kernel: the last CTA of the grid to finish
 // (a ticket taken after a fence; no CTA waits) adds the CTAs' partials in the
 // order of k_finalize into *out0 (times scale0) and, with out1, the second
@@ -984,40 +1006,52 @@ __global__ void k_scale_by_inv(const E* __restrict__ x, E* __restrict__ y, size_
 
 // y = (float) x * sigma, with the sum of squares of y: per thread and across
 // a warp in FP32 (terms of one sign; a thread holds about a hundred of a
-// 256^3 field), across warps and blocks in FP64. vec: 16-byte aligned, four
-// values per thread and step, two steps in flight; 34 us at 256^3 (201 MB, 0.87 of
+// 256^3 field), across warps and blocks in FP64. Four sums per thread, one per
+// component of its vectors, each folded over the warp by itself: one of them has
+// no more terms than a thread with one entry at a time would give it. vec:
+// 16-byte aligned, four values per thread and step, two steps in flight; 34 us at 256^3 (201 MB, 0.87 of
 // the copy bandwidth), 70 us with scalar loads.
 __global__ void __launch_bounds__(kRedThreads) k_convert_sq(const double* __restrict__ x, float* __restrict__ y,
                                                             size_t n, int vec, float sigma,
                                                             const double* __restrict__ sigma_dev,
                                                             double* __restrict__ partial, FinTail tail) {
   if (sigma_dev) sigma = (float)*sigma_dev;
-  float acc = 0.f;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   const size_t stride = (size_t)gridDim.x * blockDim.x, t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  size_t done = 0;
+  size_t i = t;
   if (vec) {
     const size_t n4 = n >> 2;
     auto put = [&](size_t i, double2 a, double2 b) {
       const float4 v = make_float4(d2f_bits(a.x) * sigma, d2f_bits(a.y) * sigma, d2f_bits(b.x) * sigma,
                                    d2f_bits(b.y) * sigma);
       reinterpret_cast<float4*>(y)[i] = v;
-      acc = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, acc))));
+      acc = make_float4(fmaf(v.x, v.x, acc.x), fmaf(v.y, v.y, acc.y), fmaf(v.z, v.z, acc.z), fmaf(v.w, v.w, acc.w));
     };
     const double2* x2 = reinterpret_cast<const double2*>(x);
-    size_t i = t;
     for (; i + stride < n4; i += 2 * stride) {
       const double2 a = x2[2 * i], b = x2[2 * i + 1], c = x2[2 * (i + stride)], d = x2[2 * (i + stride) + 1];
       put(i, a, b);
       put(i + stride, c, d);
     }
     if (i < n4) put(i, x2[2 * i], x2[2 * i + 1]);
-    done = 4 * n4;
+    i = 4 * n4 + (stride - 1 - t);  // the last threads, which hold the fewest vectors
   }
-  for (size_t i = done + t; i < n; i += stride) {
+  auto one = [&](size_t i) {
     const float v = d2f_bits(x[i]) * sigma;
     y[i] = v;
-    acc = fmaf(v, v, acc);
+    return v;
+  };
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    const float a = one(i), b = one(i + stride), c = one(i + 2 * stride), d = one(i + 3 * stride);
+    acc = make_float4(fmaf(a, a, acc.x), fmaf(b, b, acc.y), fmaf(c, c, acc.z), fmaf(d, d, acc.w));
   }
+  float* const part = &acc.x;
+#pragma unroll
+  for (int r = 0; r < 3; ++r, i += stride)
+    if (i < n) {
+      const float a = one(i);
+      part[r] = fmaf(a, a, part[r]);
+    }
   const double s = block_sum_f(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
   if (tail.ticket) fin_tail(partial, tail);
@@ -1235,7 +1269,7 @@ void launch_convert_sum(const X* x, T* y, size_t n, double* partial, double* out
                         cudaStream_t s, unsigned* ticket) {
   FinTail t;
   if (ticket) t = FinTail{ticket, out_in, 1.0, out_out, 1.0};
-  const int nb = red_blocks(n);
+  const int nb = red_blocks(n, 256);
   prof_begin(P_VEC, s);
   if constexpr (sizeof(X) == 4 && sizeof(T) == 4) {
     if (aligned16(x) && aligned16(y))
@@ -1266,8 +1300,8 @@ void launch_dot(const E* x, const E* y, size_t n, double* partial, double* out, 
   FinTail t;
   if (ticket) t = FinTail{ticket, out, scale, nullptr, 1.0};
   prof_begin(P_DOT, s);
-  const int nb = red_blocks(n);
-  k_dot_partial<E><<<nb, kRedThreads, 0, s>>>(x, y, n, partial, aligned16(x) && aligned16(y), t);
+  const int vec = aligned16(x) && aligned16(y), nb = red_blocks(n, sizeof(E) == 4 && !vec ? 256 : 512);
+  k_dot_partial<E><<<nb, kRedThreads, 0, s>>>(x, y, n, partial, vec, t);
   prof_end(P_DOT, s, "dot_partial", 2.0 * sizeof(E) * n);
   if (ticket) return;
   prof_begin(P_REDUCE, s);

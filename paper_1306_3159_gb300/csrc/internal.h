@@ -131,8 +131,10 @@ __device__ __forceinline__ double f2d_bits(float f) {
 // not; entries a thread takes one after the other cost a memory latency each.
 constexpr int kRedBlocks = 608;   // 4 x 152 SMs
 constexpr int kRedThreads = 256;
-inline int red_blocks(size_t n) {
-  const size_t b = (n + 511) / 512;
+// Kernels that add single FP32 entries per thread take one entry a thread
+// (entries = 256): a second one would double the terms of a warp's FP32 sum.
+inline int red_blocks(size_t n, int entries = 512) {
+  const size_t b = (n + entries - 1) / entries;
   return b < 1 ? 1 : (b > (size_t)kRedBlocks ? kRedBlocks : (int)b);
 }
 

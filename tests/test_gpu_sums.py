@@ -78,3 +78,31 @@ def test_sum_off_a_boundary(lib, n, start, bits):
         return best
 
     assert time(x[start:]) < 4 / 3 * time(x)
+
+
+# start 1: no 16-byte alignment
+@pytest.mark.parametrize("n", [1, 7, 1000, 100003, 262145])
+@pytest.mark.parametrize("start", [0, 1])
+def test_terms_of_the_fp32_partial_sums(lib, n, start):
+    """Squares, products and converted entries are added in FP32 over a warp of a
+    small field's threads, one term each: 32 whole numbers of at most 700 x 700
+    (of one below 2^24) are exact, 64 and more are not, so the totals are exact."""
+    import torch
+    rng = np.random.default_rng(n + start)
+    a, b = (rng.integers(1, 701, n + start).astype(np.float64) for _ in (0, 1))
+    x, y = torch.from_numpy(a).cuda()[start:], torch.empty(n + start, dtype=torch.float32, device="cuda")[start:]
+    partial, out = scratch()
+    launcher(lib, "_ZN4ibrd17launch_convert_sqEPKdPfmdPdS3_P11CUstream_stPj", P, P, Z, D, P, P)(
+        x, y, n, 1.0, partial, out)
+    assert out.item() == (a[start:] ** 2).sum() and torch.equal(y.double(), x)
+    if n <= 155648:
+        if start:  # (aligned, a thread's sum takes the four products of its vector)
+            f, g = (torch.from_numpy(v).cuda().float()[start:] for v in (a, b))
+            launcher(lib, "_ZN4ibrd10launch_dotIfEEvPKT_S3_mPdS4_dP11CUstream_stPj", P, P, Z, P, P, D)(
+                f, g, n, partial, out, 1.0)
+            assert out.item() == (a[start:] * b[start:]).sum()
+        c = rng.integers(1, 1 << 24, n + start).astype(np.float64)
+        both = torch.zeros(2, dtype=torch.float64, device="cuda")
+        launcher(lib, "_ZN4ibrd18launch_convert_sumIdfEEvPKT_PT0_mPdS6_S6_P11CUstream_stPj", P, P, Z, P, P, P)(
+            torch.from_numpy(c).cuda()[start:], y, n, partial, both, both[1:])
+        assert both[0].item() == both[1].item() == c[start:].sum()
