@@ -16,9 +16,13 @@
 //   halo plane on each side, and its planes of b, in shared memory; the cells a
 //   half-sweep updates in its outer planes are also stored in the neighbours'
 //   halos (distributed shared memory), and a cluster barrier ends the half-sweep.
-// * b is kept divided by the diagonal: an update is five additions and one FMA.
+// * An update is (b + off * neighbours) * inv, with the one rounding of inv = 1 / diag
+//   in both terms. (b kept divided by the diagonal and a rounded off / diag save
+//   one of its seven instructions, but the sweeps then scale smooth fields: the error of a
+//   V-cycle at 64^3 went from 6e-16 to 1e-15 for alpha = 0.01.)
 // * After a sweep the residual of the black cells is zero: the restriction forms
-//   it in the red cells only (all of them when there was no sweep), and the
+//   it in the red cells only (all of them when there was no sweep), together with
+//   what the rounding of inv leaves in the black ones (slack x), and the
 //   prolongation corrects only the black cells when a sweep follows, which reads
 //   no others. Its z-part is formed once per fine plane and coarse cell, also
 //   for the halo planes, so that it needs no exchange.
@@ -96,14 +100,10 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
   const int tid = threadIdx.x, nt = blockDim.x, rank = blockIdx.x;  // the grid is one cluster
   double* own_x = sm + L.own;
   double* own_b = own_x + (lv.total - lv.off[shared]);
-  __shared__ double offinv[kMaxSmallLevels];
-  if (tid < lv.n) offinv[tid] = lv.offd[tid] * lv.inv[tid];
-  __syncthreads();
-
   // this CTA's part of shared level l
   struct Part {
     int nx, ny, nz, plane, k0, np, below, above, below_np;  // planes [k0, k0 + np); the ranks next to them in z
-    double inv, offinv, diag, off;
+    double inv, diag, off;
   };
   auto part = [&](int l) {
     Part p;
@@ -118,7 +118,6 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
     p.below_np = 2 * (s.start(p.below + 1) - s.start(p.below));
     p.diag = lv.diag[l], p.off = lv.offd[l];
     p.inv = lv.inv[l];
-    p.offinv = offinv[l];
     return p;
   };
   // the neighbours' values around cell (i, j) of local plane kk (x planes are shifted by the lower halo)
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
     for (int colour = 0; colour < 2; ++colour) {
       for_colour(p, colour, [&](int i, int j, int kk) {
         const int o = j * p.nx + i;
-        const double v = fma(p.offinv, nbr_sum(X, p, i, j, kk), B[kk * p.plane + o]);
+        const double v = fma(p.off, nbr_sum(X, p, i, j, kk), B[kk * p.plane + o]) * p.inv;
         X[(kk + 1) * p.plane + o] = v;
         if (kk == 0) put_peer(peer(X + (p.below_np + 1) * p.plane + o, p.below), v);
         if (kk == p.np - 1) put_peer(peer(X + o, p.above), v);
@@ -152,12 +151,12 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
     }
   };
 
-  // set-up: x (the guess or zero) and b / diag of the top level, zero x below
+  // set-up: x (the guess or zero) and b of the top level, zero x below
   {
     const double sh = bshift ? *bshift : 0.0;
     const Part p = part(0);
     double* X = sm + L.x[0];
-    for (int c = tid; c < p.np * p.plane; c += nt) sm[L.b[0] + c] = (bg[(size_t)p.k0 * p.plane + c] - sh) * p.inv;
+    for (int c = tid; c < p.np * p.plane; c += nt) sm[L.b[0] + c] = bg[(size_t)p.k0 * p.plane + c] - sh;
     for (int c = tid; c < (p.np + 2) * p.plane; c += nt) {
       const int kk = c / p.plane, k = p.k0 - 1 + kk;
       X[c] = zero || p.np == 0 ? 0.0
@@ -182,7 +181,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
     const int nxc = p.nx >> 1, nyc = p.ny >> 1, cplane = nxc * nyc, nc = cplane * (p.np >> 1);
     const bool next_shared = l + 1 < shared;
     const Split sn(p.nz >> 1, C);  // of the next level, when it is shared
-    const double inv_next = lv.inv[l + 1];
+    const double slack = nu1 > 0 ? fma(-p.diag, p.inv, 1.0) * p.diag : 0.0;
     for (int e = tid; e < ((4 * nc + 31) & ~31); e += nt) {
       const int cell = e >> 2, dy = e & 1, dz = (e >> 1) & 1;
       double r = 0.0;
@@ -193,8 +192,8 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
         const int J = o / nxc, I = o - J * nxc, j = 2 * J + dy, kk = 2 * K + dz;
         for (int colour = 0; colour < (nu1 > 0 ? 1 : 2); ++colour) {
           const int i = 2 * I + ((j + p.k0 + kk + colour) & 1), at = j * p.nx + i;
-          const double d = B[kk * p.plane + at] - X[(kk + 1) * p.plane + at];
-          r += fma(p.diag, d, p.off * nbr_sum(X, p, i, j, kk));
+          const double x = X[(kk + 1) * p.plane + at];
+          r += fma(slack, x, fma(p.off, nbr_sum(X, p, i, j, kk), fma(-p.diag, x, B[kk * p.plane + at])));
         }
       }
       r += __shfl_xor_sync(0xffffffffu, r, 1);
@@ -204,7 +203,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_vcycle_cluster(const __grid
         r *= 0.125;
         if (next_shared) {
           const int to = sn.owner(Kg >> 1);
-          put_peer(peer(sm + L.b[l + 1] + (Kg - 2 * sn.start(to)) * cplane + o, to), r * inv_next);
+          put_peer(peer(sm + L.b[l + 1] + (Kg - 2 * sn.start(to)) * cplane + o, to), r);
         } else {
           put_peer(peer(own_b + Kg * cplane + o, 0), r);
         }

@@ -366,8 +366,11 @@ __global__ void __launch_bounds__(256) k_rb_half(const T* __restrict__ xr, T* __
 // per SM and clock) bounds every FP64 sweep, so this form counts operations: six
 // per cell instead of eight. A thread walks up a diagonal (i + 1, j + 1), whose
 // cells have one colour: the sum of the east and north neighbours of one is that
-// of the south and west neighbours of the next. b and its shift enter by one
-// FMA, the neighbours by another. In place and by colour there is no halo to
+// of the south and west neighbours of the next. The neighbours enter b by one
+// FMA, and the product with 1 / diag takes the shift in by another: both terms
+// carry the rounding of 1 / diag alone (with a rounded off / diag beside it the
+// sweeps scaled smooth fields, 1e-15 of error in a V-cycle instead of 6e-16, at
+// 64^3 with alpha = 0.01). In place and by colour there is no halo to
 // compute twice, which cost the fused one-pass kernel 1.3 times the operations
 // here (with FP32 it pays, in bytes): a sweep of 128^3 (both colours) takes
 // 45 us with the FP64 pipe 76 % busy, the fused kernel 58; of 96^3 21 and 28, of
@@ -377,7 +380,7 @@ __global__ void __launch_bounds__(256) k_rb_half(const T* __restrict__ xr, T* __
 // take their east neighbour along).
 __global__ void __launch_bounds__(256) k_rb_half_f64(double* __restrict__ x, const double* __restrict__ b,
                                                      const double* __restrict__ bshift, int nx, int ny, int nz, int yc,
-                                                     double inv, double offinv, int colour, int zero,
+                                                     double inv, double off, int colour, int zero,
                                                      double* __restrict__ part) {
   const int np = nx >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, k = t / np, p = t - k * np;
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(256) k_rb_half_f64(double* __restrict__ x, con
         const int o = j * nx + i, ip = i + 1 == nx ? 0 : i + 1;
         const double e = c[j * nx + ip];
         const double en = e + c[(j + 1 == ny ? 0 : j + 1) * nx + i];
-        const double v = fma(offinv, (sw + en) + (zm[o] + zp[o]), fma(bk[o], inv, msh));
+        const double v = fma(fma(off, (sw + en) + (zm[o] + zp[o]), bk[o]), inv, msh);
         c[o] = v;
         if (part) acc += v + e;
         sw = en;
@@ -428,10 +431,14 @@ __global__ void __launch_bounds__(256) k_rb_half_f64(double* __restrict__ x, con
 // FP64 restriction of the residual after a sweep, whose black cells have none:
 // the red cells' alone, half the operations. Per coarse cell off times the sum
 // of its four red children's neighbours, plus the sum of their b - shift, minus
-// diag times that of their x, over 8. 128^3: 22 us, 51 with all cells.
+// diag times that of their x, over 8. What the rounding of 1 / diag leaves in a
+// black cell, slack x with slack = (1 - diag inv) diag, is not averaged out by the
+// coarse levels: it is added, the black cells' x being a sixth of what the red
+// cells' neighbours sum to (one FMA). 128^3: 22 us, 51 with all cells.
 __global__ void __launch_bounds__(256) k_restrict_red_f64(const double* __restrict__ x, const double* __restrict__ b,
                                                           const double* __restrict__ bshift, double* __restrict__ bc,
-                                                          int nx, int ny, int nz, double diag, double off) {
+                                                          int nx, int ny, int nz, double diag, double off,
+                                                          double slack6) {
   const int nxc = nx >> 1, nyc = ny >> 1, nzc = nz >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int I = t % nxc, J = (t / nxc) % nyc, K = t / (nxc * nyc);
@@ -452,7 +459,7 @@ __global__ void __launch_bounds__(256) k_restrict_red_f64(const double* __restri
       sx += x[o];
       sb += b[o];
     }
-  bc[t] = fma(off, sn, fma(-diag, sx, sb)) * 0.125;
+  bc[t] = fma(slack6, sn, fma(off, sn, fma(-diag, sx, sb))) * 0.125;
 }
 
 // FP64 prolongation before a sweep, which reads no red cells: only the black
@@ -1012,7 +1019,7 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
       if (nblk > part_cap) part = nullptr;
       for (int colour = 0; colour < 2; ++colour) {
         prof_begin(c, s);
-        k_rb_half_f64<<<g, 256, 0, s>>>(const_cast<T*>(xin), b, bshift, d.nx, d.ny, d.nz, yc, inv, off * inv, colour,
+        k_rb_half_f64<<<g, 256, 0, s>>>(const_cast<T*>(xin), b, bshift, d.nx, d.ny, d.nz, yc, inv, off, colour,
                                         (zero && colour == 0) ? 1 : 0, colour == 1 ? part : nullptr);
         prof_end(c, s, "rb_half_f64", 1.5 * sizeof(T) * d.n());
       }
@@ -1081,8 +1088,9 @@ void launch_resid_restrict(const T* x, const T* b, const double* bshift, T* bc, 
   if constexpr (sizeof(T) == 8) {
     if (swept) {
       const unsigned blocks = (unsigned)((d.n() / 8 + 255) / 256);
+      const double slack = std::fma(-st.diag, 1.0 / st.diag, 1.0) * st.diag;
       prof_begin(P_RESTRICT64, s);
-      k_restrict_red_f64<<<blocks, 256, 0, s>>>(x, b, bshift, bc, d.nx, d.ny, d.nz, st.diag, st.off);
+      k_restrict_red_f64<<<blocks, 256, 0, s>>>(x, b, bshift, bc, d.nx, d.ny, d.nz, st.diag, st.off, slack / 6.0);
       prof_end(P_RESTRICT64, s, "restrict_red_f64", 2.125 * sizeof(T) * d.n());
       return;
     }
