@@ -449,27 +449,24 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
   const bool one_pass = sizeof(T) == 4 && nu1 == 1 && zero && aligned16(b) && aligned16(x);
   const bool rows = one_pass && zero_restrict_rows_ok(lv.d) && wait_error_flag();
   const bool tile = one_pass && zero_restrict_ok(lv.d) && lv.d.n() <= (size_t(1) << 21);
-  bool packed = false;  // cur holds the black cells only
+  // whether the sweep from zero leaves the black cells only, for the post-smoothing sweep with the prolongation
+  const bool packed = rows && nu2 > 0 && prolong_sweep_on(lv.d);
   if (zero) {
     // the cycle starts in whichever of the two fields its out-of-place passes
     // lead from to x (a copy at the end would move the level once more)
     const bool sw = rb_sweep_swaps<T>(lv.d, false, x, b);
     int swaps = sw ? nu2 : 0;
-    if (rows)
-      swaps = nu2 > 0 ? nu2 : 1;  // without a post-smoothing sweep: the unpacking
-    else if (!tile && nu1 > 0)
-      swaps += (rb_sweep_swaps<T>(lv.d, true, x, b) ? 1 : 0) + (sw ? nu1 - 1 : 0);
+    if (!rows && !tile && nu1 > 0) swaps += (rb_sweep_swaps<T>(lv.d, true, x, b) ? 1 : 0) + (sw ? nu1 - 1 : 0);
     if (swaps & 1) std::swap(cur, oth);
   }
   if (rows) {
     // the single pre-smoothing sweep from zero and the restriction in one
-    // pass, row-resident and fed by TMA; only the black cells are stored
+    // pass, row-resident and fed by TMA
     prof_begin(P_RBGS32, g->s);
-    launch_zero_restrict_rows(reinterpret_cast<const float*>(b), bshift, reinterpret_cast<float*>(cur),
+    launch_zero_restrict_rows(reinterpret_cast<const float*>(b), bshift, reinterpret_cast<float*>(cur), !packed,
                               reinterpret_cast<float*>(H.b[l + 1]), lv.d, st, zero_restrict_rows_default_zc(lv.d),
                               g->s);
-    prof_end(P_RBGS32, g->s, "zero_restrict_rows", 6.5 * lv.d.n());
-    packed = true;
+    prof_end(P_RBGS32, g->s, "zero_restrict_rows", (packed ? 6.5 : 8.5) * lv.d.n());
   } else if (tile) {
     // the single pre-smoothing sweep from zero and the restriction in one pass
     // (levels up to 128^3 cells; on larger ones the kernel is bound by its
@@ -497,13 +494,7 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
     }
   }
   if (sweep == 0) {
-    if (packed) {
-      prof_begin(P_RBGS32, g->s);
-      launch_unpack_zero(reinterpret_cast<const float*>(cur), reinterpret_cast<const float*>(b), bshift,
-                         reinterpret_cast<float*>(oth), lv.d, st, g->s);
-      prof_end(P_RBGS32, g->s, "unpack_zero", 10.0 * lv.d.n());
-      std::swap(cur, oth);
-    }
+    if (packed) throw CudaError{cudaErrorInvalidValue, "packed cells without the sweep that reads them"};
     launch_prolong8<T>(H.x[l + 1], cur, lv.d, nu2 > 0, g->s);
   }
   for (; sweep < nu2; ++sweep) {

@@ -203,16 +203,14 @@ int launch_rows_prolong_sweep(const float* xc, const float* xin, bool packed, fl
                               const double* bshift, Dims d, Stencil st, int zc, double* part, int part_cap,
                               cudaStream_t s);
 // The first sweep from zero fused with the residual restriction on the same
-// levels as the row-resident sweep: xb = the black cells of x = sweep(0) (nx /
-// 2 per row; the red cells are (b - shift) / diag), bc = mean over 8 children
-// of b - shift - A x (bc 8-byte aligned). zc = planes per CTA (made even).
+// levels as the row-resident sweep: x = sweep(0), bc = mean over 8 children of
+// b - shift - A x (bc 8-byte aligned). Without full only the black cells of x are
+// written, nx / 2 per row (the red cells are (b - shift) / diag), as
+// launch_rows_prolong_sweep reads them. zc = planes per CTA (made even).
 bool zero_restrict_rows_ok(Dims d);
 int zero_restrict_rows_default_zc(Dims d);
-void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, float* bc, Dims d, Stencil st,
-                               int zc, cudaStream_t s);
-// x from the packed black cells xb and b: the whole field after that sweep.
-void launch_unpack_zero(const float* xb, const float* b, const double* bshift, float* x, Dims d, Stencil st,
-                        cudaStream_t s);
+void launch_zero_restrict_rows(const float* b, const double* bshift, float* x, bool full, float* bc, Dims d,
+                               Stencil st, int zc, cudaStream_t s);
 // Levels handled by the single-CTA coarse V-cycle (shared-memory resident).
 constexpr int kMaxSmallLevels = 12;
 struct CoarseLevels {
@@ -253,7 +251,9 @@ void launch_prolong8(const T* xc, T* x, Dims d, bool sweep_follows, cudaStream_t
 // field to xout (xin is left uncorrected) and returns the partial-sum count
 // as launch_rb_sweep does, or -1 without launching when it does not apply
 // (the caller then prolongs and sweeps separately). packed: xin holds the
-// black cells only (launch_rows_prolong_sweep).
+// black cells only (launch_rows_prolong_sweep). prolong_sweep_on: whether the
+// level and its tuned shapes let it apply (16-byte aligned fields given).
+bool prolong_sweep_on(Dims d);
 template <typename T>
 int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
                          Stencil st, double* part, int part_cap, cudaStream_t s);

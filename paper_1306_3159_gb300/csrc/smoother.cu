@@ -1146,24 +1146,27 @@ void launch_zero_restrict(const float* b, const double* bshift, float* x, float*
   prof_end(P_RBGS32, s, "zero_restrict", 8.0 * d.n() + 0.5 * d.n());
 }
 
+bool prolong_sweep_on(Dims d) {
+  if (!rows_sweep_ok(d) || !wait_error_flag()) return false;
+  // the row-resident sweep with the prolongation, unless a tiled sweep was
+  // chosen or the fusion was switched off for it
+  const SweepShape* tp = tuned_sweep(4, TUNE_PROLONG, d);
+  return rows_shape(tuned_sweep(4, TUNE_SWEEP, d), d) && !(tp && tp->tx == 1);
+}
+
 template <typename T>
 int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
                          Stencil st, double* part, int part_cap, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (rows_sweep_ok(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && aligned16(xc) && xin != xout &&
-        b != xout && xc != xout && wait_error_flag()) {
-      // the row-resident sweep serves this level unless a tiled shape was
-      // chosen or the fusion was switched off for it
+    if (prolong_sweep_on(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && aligned16(xc) && xin != xout &&
+        b != xout && xc != xout) {
       const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
-      const SweepShape* tp = tuned_sweep(4, TUNE_PROLONG, d);
-      if (rows_shape(tn, d) && !(tp && tp->tx == 1)) {
-        const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
-        prof_begin(P_RBGS32, s);
-        const int r = launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);
-        // x (or its black half), b and the coarse field read once, x written once
-        prof_end(P_RBGS32, s, "prolong_sweep_rows", ((packed ? 2.5 : 3.0) + 0.125) * sizeof(T) * d.n());
-        return r;
-      }
+      const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
+      prof_begin(P_RBGS32, s);
+      const int r = launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);
+      // x (or its black half), b and the coarse field read once, x written once
+      prof_end(P_RBGS32, s, "prolong_sweep_rows", ((packed ? 2.5 : 3.0) + 0.125) * sizeof(T) * d.n());
+      return r;
     }
   }
   return -1;

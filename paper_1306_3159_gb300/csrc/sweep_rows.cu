@@ -611,7 +611,9 @@ __host__ __device__ constexpr size_t zero_rows_floats(int nx) {
 // cells (b - shift) / diag, black cells from their red neighbours (the
 // arithmetic of k_rb_zero_f32v), bc = mean over the 8 children of
 // b - shift - A x, in one pass over b (HBM: read b, write the packed black
-// cells and bc; the red cells are b / diag and enter no later sweep). In exact
+// cells and bc; the red cells are b / diag and enter no later sweep). FULL: the
+// field is written in full, for cycles whose next pass is not the row sweep with
+// the prolongation. In exact
 // arithmetic the residual is off times the neighbour sum in the red cells and
 // zero in the black ones; inv = 1 / diag in FP32 leaves a common relative error
 // of up to 3e-8 in every x, which adds (1 - diag inv) diag x to every residual
@@ -626,9 +628,9 @@ __host__ __device__ constexpr size_t zero_rows_floats(int nx) {
 // adds them one step later (after the step's barrier) and writes the coarse
 // row. Chunks start on even planes and hold an even number of them, so plane
 // pairs never straddle chunks.
-template <int NS, int WPR, int NXT>
+template <int NS, int WPR, int NXT, bool FULL>
 __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
-    k_zr_rows(const __grid_constant__ RowMaps mb, float* __restrict__ xb, float* __restrict__ bc,
+    k_zr_rows(const __grid_constant__ RowMaps mb, float* __restrict__ xo, float* __restrict__ bc,
               const double* __restrict__ bshift, int nx_, int ny, int nz, int zc, float inv, float off, float slack,
               int* __restrict__ err, unsigned wait_limit) {
   constexpr int TY = kRowsTY, R = kZeroRing, XROWS = TY + 4, BROWS = TY + 2;
@@ -710,8 +712,9 @@ __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
 
   bool ok = true;
   // where this row of plane mp(2), mp(3), ... and the coarse rows go
-  const ptrdiff_t pplane = (ptrdiff_t)nxp * ny, cplane = (ptrdiff_t)nxp * (ny >> 1);
-  float* dst = xb + (ptrdiff_t)mp(2) * pplane + (ptrdiff_t)y * nxp;
+  const int nxo = FULL ? nx : nxp;  // row length of the output
+  const ptrdiff_t pplane = (ptrdiff_t)nxo * ny, cplane = (ptrdiff_t)nxp * (ny >> 1);
+  float* dst = xo + (ptrdiff_t)mp(2) * pplane + (ptrdiff_t)y * nxo;
   float* cdst = bc + (ptrdiff_t)(mp(2) >> 1) * cplane + (ptrdiff_t)(y >> 1) * nxp;
   const ptrdiff_t dstep = down ? -pplane : pplane, cstep = down ? -cplane : cplane;
   float2 held[NS];  // restriction sums of a completed plane pair (even rows)
@@ -753,7 +756,15 @@ __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
         x0[s] = mul2(fma2(off2, add2(add2(n[s], add2(u[s], d[s])), add2(rm[s], rp[s])), b0[s]), inv2);
       put_row(xbrow(P0, w), x0);
       if (interior && i >= 3) {
-        put_row(dst, xm1);
+        if constexpr (FULL) {
+#pragma unroll
+          for (int s = 0; s < NS; ++s)
+            if (row.valid(s))
+              *reinterpret_cast<float4*>(dst + 4 * row.group(s)) =
+                  a ? make_float4(rm[s].x, xm1[s].x, rm[s].y, xm1[s].y) : make_float4(xm1[s].x, rm[s].x, xm1[s].y, rm[s].y);
+        } else {
+          put_row(dst, xm1);
+        }
         dst += dstep;
         nbr_sums<NS, WPR, NXT>(n, xm1, xbrow(P1, w), !a, row);
         get_row(u, xbrow(P1, w - 1));
@@ -799,26 +810,6 @@ __global__ void __launch_bounds__(kRowsThreads<WPR>, WPR == 1 ? 2 : 1)
     march(std::false_type{});
   }
   if (ok && interior && !odd_row) combine();  // the last pair (its RY write preceded the last barrier)
-}
-
-// x = the field whose black cells are packed in xb and whose red cells are
-// (b - shift) / diag (the state after a first sweep from zero): for V-cycles
-// that need the pre-smoothed field in full (no post-smoothing sweep, or the
-// prolongation kept separate). One thread per 4-cell group.
-__global__ void __launch_bounds__(256) k_unpack_zero(const float* __restrict__ xb, const float* __restrict__ b,
-                                                     const double* __restrict__ bshift, float* __restrict__ x,
-                                                     int nx, int ny, int nz, float inv) {
-  const size_t groups = (size_t)(nx >> 2) * ny * nz;
-  const float sh = bshift ? (float)(*bshift) : 0.f;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < groups;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const size_t r = t / (nx >> 2);  // row j + ny k
-    const bool a = ((int)(r % ny) + (int)(r / ny)) & 1;
-    const float2 k = reinterpret_cast<const float2*>(xb)[t];
-    const float4 q = reinterpret_cast<const float4*>(b)[t];
-    reinterpret_cast<float4*>(x)[t] = a ? make_float4(k.x, (q.y - sh) * inv, k.y, (q.w - sh) * inv)
-                                        : make_float4((q.x - sh) * inv, k.x, (q.z - sh) * inv, k.y);
-  }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -874,6 +865,17 @@ void sweep_rows_go(dim3 g, cudaStream_t s, const RowMaps& mx, const RowMaps& mb,
   k_rbgs_rows<NS, WPR, NXT, IN><<<g, kRowsThreads<WPR>, sm, s>>>(
       mx, mb, mc, xout, bshift, d.nx, d.ny, d.nz, zc, inv, off, part, wait_error_flag(),
       wait_limit());
+}
+
+template <int NS, int WPR, int NXT, bool FULL>
+void zero_rows_go(dim3 g, cudaStream_t s, const RowMaps& mb, float* x, float* bc, const double* bshift, Dims d, int zc,
+                  float inv, float off, float slack) {
+  const size_t sm = 4 * zero_rows_floats(d.nx) + 8 * kZeroRing;
+  static std::atomic<unsigned long long> attr{0};
+  ensure_smem_attr((const void*)k_zr_rows<NS, WPR, NXT, FULL>,
+                   (int)(4 * zero_rows_floats(NXT ? NXT : 128 * NS * WPR) + 8 * kZeroRing), attr);
+  k_zr_rows<NS, WPR, NXT, FULL><<<g, kRowsThreads<WPR>, sm, s>>>(mb, x, bc, bshift, d.nx, d.ny, d.nz, zc, inv, off,
+                                                                 slack, wait_error_flag(), wait_limit());
 }
 
 // Calls f with the kernel shape of rows of nx cells (see rows_sweep_ok).
@@ -961,9 +963,9 @@ int zero_restrict_rows_default_zc(Dims d) {
   return rows_sweep_default_zc(d);  // even: plane pairs of the restriction stay inside a chunk
 }
 
-void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, float* bc, Dims d, Stencil st,
-                               int zc, cudaStream_t s) {
-  if (!zero_restrict_rows_ok(d) || !aligned16(b) || !aligned16(xb) || ((uintptr_t)bc & 7u) || b == xb)
+void launch_zero_restrict_rows(const float* b, const double* bshift, float* x, bool full, float* bc, Dims d,
+                               Stencil st, int zc, cudaStream_t s) {
+  if (!zero_restrict_rows_ok(d) || !aligned16(b) || !aligned16(x) || ((uintptr_t)bc & 7u) || b == x)
     throw CudaError{cudaErrorInvalidValue, "fused zero sweep + restriction arguments"};
   zc = clamp_zc(zc, d.nz, true);
   const RowMaps mb = row_maps(b, d.nx, d.ny, d.nz, kRowsTY, 2);
@@ -971,20 +973,11 @@ void launch_zero_restrict_rows(const float* b, const double* bshift, float* xb, 
   const float inv = (float)(1.0 / st.diag), slack = (float)((1.0 - st.diag * (double)inv) * st.diag / st.off);
   with_row_shape(d.nx, [&](auto ns, auto wpr, auto nxt) {
     constexpr int NS = ns.value, WPR = wpr.value, NXT = nxt.value;
-    const size_t sm = 4 * zero_rows_floats(d.nx) + 8 * kZeroRing;
-    static std::atomic<unsigned long long> attr{0};
-    ensure_smem_attr((const void*)k_zr_rows<NS, WPR, NXT>,
-                     (int)(4 * zero_rows_floats(NXT ? NXT : 128 * NS * WPR) + 8 * kZeroRing), attr);
-    k_zr_rows<NS, WPR, NXT><<<g, kRowsThreads<WPR>, sm, s>>>(
-        mb, xb, bc, bshift, d.nx, d.ny, d.nz, zc, inv, (float)st.off, slack, wait_error_flag(), wait_limit());
+    if (full)
+      zero_rows_go<NS, WPR, NXT, true>(g, s, mb, x, bc, bshift, d, zc, inv, (float)st.off, slack);
+    else
+      zero_rows_go<NS, WPR, NXT, false>(g, s, mb, x, bc, bshift, d, zc, inv, (float)st.off, slack);
   });
-}
-
-void launch_unpack_zero(const float* xb, const float* b, const double* bshift, float* x, Dims d, Stencil st,
-                        cudaStream_t s) {
-  const size_t groups = d.n() / 4;
-  const int blocks = (int)std::min<size_t>((groups + 255) / 256, 152 * 16);
-  k_unpack_zero<<<blocks, 256, 0, s>>>(xb, b, bshift, x, d.nx, d.ny, d.nz, (float)(1.0 / st.diag));
 }
 
 }  // namespace ibrd
