@@ -409,11 +409,14 @@ double ibrd_periodic_constant(double lx, double ly, double lz);
    handle's hierarchy, tx in {0, 32, 64} or tx = nx (0 for kind 1; 64 only
    for FP32 and when 64 divides nx, else ignored; nx selects the row-resident
    FP32 sweep on levels whose rows are 128 or 256 cells, ny a multiple of 8
-   and nz even; 0, the built-in rule, selects it wherever it serves the level),
-   zc >= 0 (0 = built-in; clamped to the level's nz).
+   and nz even; 0, the built-in rule, selects it on levels it serves where it is
+   the faster one), zc >= 0 (0 = built-in; clamped to the level's nz). For FP64
+   the built-in rule is the in-place half sweeps; tx = 32, or tx = 0 with zc > 0,
+   selects the tiled kernel.
    kind 2 (FP32 only, zc = 0) is the coarse-grid correction of the level: on
-   levels the row-resident sweep serves, the V-cycle adds the prolongation of
-   the coarse correction inside the first post-smoothing sweep (one pass over
+   levels the row-resident sweep serves (with more than one sweep before it:
+   where that is faster), the V-cycle adds the prolongation of the coarse
+   correction inside the first post-smoothing sweep (one pass over
    x instead of two; the same values bit for bit); tx = 1 keeps it a separate
    kernel, tx = 0 restores the default. Drops the handle's captured CUDA
    graphs. */

@@ -450,7 +450,7 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
   const bool rows = one_pass && zero_restrict_rows_ok(lv.d) && wait_error_flag();
   const bool tile = one_pass && zero_restrict_ok(lv.d) && lv.d.n() <= (size_t(1) << 21);
   // whether the sweep from zero leaves the black cells only, for the post-smoothing sweep with the prolongation
-  const bool packed = rows && nu2 > 0 && prolong_sweep_on(lv.d);
+  const bool packed = rows && nu2 > 0 && packed_between_halves(lv.d);
   if (zero) {
     // the cycle starts in whichever of the two fields its out-of-place passes
     // lead from to x (a copy at the end would move the level once more)
@@ -485,7 +485,7 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
   int sweep = 0;
   if (nu2 >= 1) {
     // the coarse-grid correction inside the first post-smoothing sweep
-    const int r = launch_prolong_sweep<T>(H.x[l + 1], cur, packed, oth, b, bshift, lv.d, st,
+    const int r = launch_prolong_sweep<T>(H.x[l + 1], cur, rows, packed, oth, b, bshift, lv.d, st,
                                           nu2 == 1 ? part : nullptr, part_cap, g->s);
     if (r >= 0) {
       std::swap(cur, oth);

@@ -168,7 +168,9 @@ bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b);
 // Launch shape of a red-black sweep kernel picked by the autotuner: tile width
 // tx (cells, fused sweep only: 32 or 64 for the tiled kernel, nx = 128 or 256
 // for the row-resident kernel there) and z-march depth zc (planes per
-// CTA); 0 keeps the built-in rule (the row-resident kernel where it applies).
+// CTA); 0 keeps the built-in rule (the row-resident kernel where rows_plain_ok
+// and rows_prolong_full_ok say; FP64: the in-place half sweeps, but with a
+// depth zc the tiled kernel).
 struct SweepShape {
   int tx = 0;
   int zc = 0;
@@ -191,6 +193,10 @@ unsigned wait_limit();
 // launch_rb_sweep (out of place, per-CTA partial sums of the new x when part
 // holds enough entries; returns their count or 0). zc = planes per CTA.
 bool rows_sweep_ok(Dims d);
+// Where its forms that read a full field are the faster ones: the plain sweep
+// (against the tiled one) and the sweep with the prolongation (against two passes).
+bool rows_plain_ok(Dims d);
+bool rows_prolong_full_ok(Dims d);
 int rows_sweep_default_zc(Dims d);
 int launch_rows_sweep(const float* xin, float* xout, const float* b, const double* bshift, Dims d, Stencil st,
                       int zc, double* part, int part_cap, cudaStream_t s);
@@ -246,17 +252,18 @@ void launch_zero_restrict(const float* b, const double* bshift, float* x, float*
 // sweep_follows: a red-black sweep of x comes next (it reads no red cells).
 template <typename T>
 void launch_prolong8(const T* xc, T* x, Dims d, bool sweep_follows, cudaStream_t s);
-// The prolongation of xc added to xin fused with the red-black sweep that
-// follows it, on levels the row-resident FP32 sweep serves: writes the swept
-// field to xout (xin is left uncorrected) and returns the partial-sum count
-// as launch_rb_sweep does, or -1 without launching when it does not apply
-// (the caller then prolongs and sweeps separately). packed: xin holds the
-// black cells only (launch_rows_prolong_sweep). prolong_sweep_on: whether the
-// level and its tuned shapes let it apply (16-byte aligned fields given).
-bool prolong_sweep_on(Dims d);
+// The prolongation of xc added to xin and the red-black sweep that follows it, on
+// levels where the row-resident FP32 sweep takes both: writes the swept field to
+// xout and returns the partial-sum count as launch_rb_sweep does, or -1 without
+// launching when it does not apply (the caller then prolongs and sweeps
+// separately). One pass, which leaves xin uncorrected, or, kept apart by hand, two
+// with the same result bit for bit. one_pass: the sweeps before it were
+// launch_zero_restrict_rows; packed: which then kept only the black cells.
 template <typename T>
-int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
-                         Stencil st, double* part, int part_cap, cudaStream_t s);
+int launch_prolong_sweep(const T* xc, T* xin, bool one_pass, bool packed, T* xout, const T* b, const double* bshift,
+                         Dims d, Stencil st, double* part, int part_cap, cudaStream_t s);
+// Whether launch_zero_restrict_rows may keep only the black cells for it.
+bool packed_between_halves(Dims d);
 // Coarsest exact solve x = G b with the circulant table G (dc.n() entries).
 template <typename T>
 void launch_coarse_solve(const T* table, const T* b, T* x, Dims dc, cudaStream_t s);

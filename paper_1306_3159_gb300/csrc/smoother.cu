@@ -941,12 +941,10 @@ bool rb_sweep_fused_ok(Dims d) {
 }
 
 
-// Whether a tuned shape (or none) means the row-resident kernel on a level it
-// serves: the built-in width, or the row length where it is 128 or 256 (widths
-// of 32 and 64 name the tiled kernel).
-static bool rows_shape(const SweepShape* tn, Dims d) {
-  return !tn || tn->tx == 0 || (tn->tx == d.nx && d.nx > 64);
-}
+// Whether a tuned shape names the tiled sweep (widths of 32 and 64), or the
+// row-resident one (the row length, where that is 128 or 256).
+static bool names_tile(const SweepShape* tn) { return tn && (tn->tx == 32 || tn->tx == 64); }
+static bool names_rows(const SweepShape* tn, Dims d) { return tn && tn->tx == d.nx && d.nx > 64; }
 
 template <typename T>
 bool rb_sweep_swaps(Dims d, bool zero, const T* x, const T* b) {
@@ -990,18 +988,16 @@ int launch_rb_sweep(const T* xin, T* xout, const T* b, const double* bshift, Dim
     }
   }
   if constexpr (sizeof(T) == 4) {
-    // rows of up to 512 cells: the row-resident kernel unless a tiled shape was
-    // chosen for this level
-    if (!zero && rows_sweep_ok(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && xin != xout &&
+    // rows of up to 512 cells: the row-resident kernel where it is the faster one,
+    // unless a shape was chosen for this level
+    const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
+    if (!zero && (names_rows(tn, d) || (rows_plain_ok(d) && !names_tile(tn))) && rows_sweep_ok(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && xin != xout &&
         b != xout && wait_error_flag()) {
-      const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
-      if (rows_shape(tn, d)) {
-        const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
-        prof_begin(c, s);
-        const int r = launch_rows_sweep(xin, xout, b, bshift, d, st, zc, part, part_cap, s);
-        prof_end(c, s, "rb_sweep_rows", 3.0 * sizeof(T) * d.n());
-        return r;
-      }
+      const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
+      prof_begin(c, s);
+      const int r = launch_rows_sweep(xin, xout, b, bshift, d, st, zc, part, part_cap, s);
+      prof_end(c, s, "rb_sweep_rows", 3.0 * sizeof(T) * d.n());
+      return r;
     }
   }
   if constexpr (sizeof(T) == 8) {
@@ -1146,26 +1142,35 @@ void launch_zero_restrict(const float* b, const double* bshift, float* x, float*
   prof_end(P_RBGS32, s, "zero_restrict", 8.0 * d.n() + 0.5 * d.n());
 }
 
-bool prolong_sweep_on(Dims d) {
-  if (!rows_sweep_ok(d) || !wait_error_flag()) return false;
-  // the row-resident sweep with the prolongation, unless a tiled sweep was
-  // chosen or the fusion was switched off for it
+// The level's coarse-grid correction belongs to the row-resident sweep that
+// follows it, unless a tiled sweep was chosen; it may be kept apart by hand.
+static bool rows_take_correction(Dims d, bool one_pass) {
+  return (one_pass ? rows_sweep_ok(d) : rows_prolong_full_ok(d)) && wait_error_flag() &&
+         !names_tile(tuned_sweep(4, TUNE_SWEEP, d));
+}
+static bool kept_apart(Dims d) {
   const SweepShape* tp = tuned_sweep(4, TUNE_PROLONG, d);
-  return rows_shape(tuned_sweep(4, TUNE_SWEEP, d), d) && !(tp && tp->tx == 1);
+  return tp && tp->tx == 1;
 }
 
+bool packed_between_halves(Dims d) { return rows_take_correction(d, true) && !kept_apart(d); }
+
 template <typename T>
-int launch_prolong_sweep(const T* xc, const T* xin, bool packed, T* xout, const T* b, const double* bshift, Dims d,
-                         Stencil st, double* part, int part_cap, cudaStream_t s) {
+int launch_prolong_sweep(const T* xc, T* xin, bool one_pass, bool packed, T* xout, const T* b, const double* bshift,
+                         Dims d, Stencil st, double* part, int part_cap, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (prolong_sweep_on(d) && aligned16(xin) && aligned16(xout) && aligned16(b) && aligned16(xc) && xin != xout &&
-        b != xout && xc != xout) {
+    if (rows_take_correction(d, one_pass) && aligned16(xin) && aligned16(xout) && aligned16(b) && aligned16(xc) &&
+        xin != xout && b != xout && xc != xout) {
       const SweepShape* tn = tuned_sweep(4, TUNE_SWEEP, d);
       const int zc = (tn && tn->zc >= 2) ? tn->zc : rows_sweep_default_zc(d);
+      const bool apart = kept_apart(d);
+      if (apart) launch_prolong8<T>(xc, xin, d, true, s);
       prof_begin(P_RBGS32, s);
-      const int r = launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);
+      const int r = apart ? launch_rows_sweep(xin, xout, b, bshift, d, st, zc, part, part_cap, s)
+                          : launch_rows_prolong_sweep(xc, xin, packed, xout, b, bshift, d, st, zc, part, part_cap, s);
       // x (or its black half), b and the coarse field read once, x written once
-      prof_end(P_RBGS32, s, "prolong_sweep_rows", ((packed ? 2.5 : 3.0) + 0.125) * sizeof(T) * d.n());
+      prof_end(P_RBGS32, s, apart ? "rb_sweep_rows" : "prolong_sweep_rows",
+               (apart ? 3.0 : (packed ? 2.5 : 3.0) + 0.125) * sizeof(T) * d.n());
       return r;
     }
   }
@@ -1222,7 +1227,7 @@ void launch_vcycle_small(const CoarseLevels& lv, const T* b, T* x, const double*
   template void launch_resid_restrict<T>(const T*, const T*, const double*, T*, Dims, Stencil, bool,          \
                                          cudaStream_t);                                                     \
   template void launch_prolong8<T>(const T*, T*, Dims, bool, cudaStream_t);                                 \
-  template int launch_prolong_sweep<T>(const T*, const T*, bool, T*, const T*, const double*, Dims, Stencil,   \
+  template int launch_prolong_sweep<T>(const T*, T*, bool, bool, T*, const T*, const double*, Dims, Stencil,   \
                                        double*, int, cudaStream_t);                                         \
   template bool rb_sweep_swaps<T>(Dims, bool, const T*, const T*);                                           \
   template bool rb_sweep_fused_ok<T>(Dims);

@@ -28,11 +28,13 @@
 //   from lane 31 to lane 0. Rows of other lengths (multiples of 32) leave lanes
 //   idle and take one more shuffle for the wrap; rows above 256 cells belong to
 //   two warps, whose outermost groups read their neighbour from the published
-//   row in shared memory. The tiled sweep (smoother.cu), which served these
-//   lengths, is the slower one at all of them: FP32 V-cycles of one pre- and one
-//   post-sweep at 96^3, 160^3, 224^3, 320^3 and 512^3 take 73, 117, 157, 361 and
-//   537 us, with the tiled sweep and separate transfers 88, 151, 222, 446 and
-//   1330 us (512^3 is the largest cube a CTA's shared memory holds rows of).
+//   row in shared memory. FP32 V-cycles of one pre- and one post-sweep, which
+//   run the sweep from zero and the packed sweep below, are faster with them at
+//   every length than with the tiled sweep and separate transfers: 49 and 60 us on
+//   32 x 64 x 64 cells, 73 and 88 at 96^3, 117 and 151 at 160^3, 157 and 222 at 224^3,
+//   361 and 446 at 320^3, 537 and 1330 at 512^3 (the largest cube a CTA's shared
+//   memory holds rows of). Where the other two forms, which read a full field,
+//   are slower, rows_plain_ok and rows_prolong_full_ok leave them out.
 // * A CTA owns TY rows of every plane of a z-chunk, plus one halo row on each
 //   side in y whose red cells it also updates (the black cells at the tile's
 //   edge rows need them); the neighbouring CTA computes the same red values
@@ -909,8 +911,9 @@ int sweep_rows_any(const float* xin, const float* xc, float* xout, const float* 
   const int nblk = (int)(g.x * g.y);
   if (nblk > part_cap) part = nullptr;
   with_row_shape(d.nx, [&](auto ns, auto wpr, auto nxt) {
-    sweep_rows_go<ns.value, wpr.value, nxt.value, IN>(g, s, mx, mb, mc, xout, bshift, d, zc, (float)(1.0 / st.diag),
-                                                      (float)st.off, part);
+    if constexpr (IN != IN_FULL_PRO || wpr.value == 1 || nxt.value == 512)  // (rows_prolong_full_ok)
+      sweep_rows_go<ns.value, wpr.value, nxt.value, IN>(g, s, mx, mb, mc, xout, bshift, d, zc,
+                                                        (float)(1.0 / st.diag), (float)st.off, part);
   });
   return part ? nblk : 0;
 }
@@ -924,6 +927,33 @@ int clamp_zc(int zc, int nz, bool even) {
 
 bool rows_sweep_ok(Dims d) {
   return d.nx % 32 == 0 && d.nx <= 512 && d.ny % kRowsTY == 0 && d.ny >= kRowsTY && d.nz % 2 == 0 && d.nz >= 4;
+}
+
+// The plain sweep of a full field. A march has a start of four planes and a
+// barrier per plane, 5 us at least, which the tiled sweep undercuts on few rows; and
+// rows below 96 cells leave lanes idle. Measured (us, row and tiled sweep, data
+// in L2) on 16 x 16 rows: 4.9 and 3.6 (96 cells), 5.4 and 4.1 (256), 6.7 and 4.0
+// (448); on 32 x 32: 5.0 and 4.4, 5.4 and 4.8, 7.0 and 5.7; on 32 x 64: 5.2 and 4.8,
+// 5.7 and 6.7, 7.2 and 7.2; on 64 x 64: 5.8 and 7.1, 6.8 and 8.6, 8.6 and 11.2; on
+// 256 x 256: 20.5 and 31.3, 33.1 and 62.4, 63.5 and 93.7. Rows of 32 cells: 5.7 and 4.2
+// on 64 x 64, 20.6 and 14.2 on 256 x 256; of 64: 5.3 and 4.9, 20.4 and 17.7. Rows of 128
+// and 256 cells, where tuned shapes name the row sweep by their length, keep it on
+// every level.
+bool rows_plain_ok(Dims d) {
+  return rows_sweep_ok(d) && (d.nx == 128 || d.nx == 256 || (d.nx >= 96 && d.ny * (size_t)d.nz >= 2048));
+}
+
+// The sweep with the prolongation of a full field, against the prolongation and the
+// better of the plain sweeps (us): rows of 96, 160 and 256 cells on 16 x 16: 5.8 and
+// 6.5, 7.2 and 6.9, 6.6 and 7.6; on 32 x 32: 5.9 and 7.6, 7.4 and 8.0, 6.8 and 8.0; on
+// 256 x 256: 24.6 and 30.2, 47.2 and 47.9, 38.5 and 59.3. Rows of 512: 9.0 and 6.9, 8.7
+// and 9.7, 74.4 and 121. Two warps on part of their lanes (rows of 288 to 480), one CTA
+// per SM: 9.8 and 7.2, 10.1 and 8.8 (288), 115 and 101 (384 on 256 x 256). Rows of 32:
+// 10.6 and 11.6 on 128 x 128, 24.2 and 18.8 on 256 x 256.
+bool rows_prolong_full_ok(Dims d) {
+  if (!rows_sweep_ok(d) || d.nx == 128 || d.nx == 256) return rows_sweep_ok(d);  // (as for the plain sweep)
+  const size_t rows = d.ny * (size_t)d.nz;
+  return (d.nx <= 256 || d.nx == 512) && rows >= 1024 && (d.nx >= 64 || rows <= 16384);
 }
 
 int rows_sweep_default_zc(Dims d) {
@@ -953,6 +983,7 @@ int launch_rows_prolong_sweep(const float* xc, const float* xin, bool packed, fl
     throw CudaError{cudaErrorInvalidValue, "prolongation + row sweep arguments"};
   // even chunks: fine planes 2K - 1, 2K share their coarse pair in both march directions
   zc = clamp_zc(zc, d.nz, true);
+  if (!packed && !rows_prolong_full_ok(d)) throw CudaError{cudaErrorInvalidValue, "prolongation + row sweep level"};
   return packed ? sweep_rows_any<IN_PACKED_PRO>(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s)
                 : sweep_rows_any<IN_FULL_PRO>(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s);
 }

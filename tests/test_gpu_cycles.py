@@ -43,3 +43,46 @@ def test_passes_outside_the_fused_sweep(ibrd, dims):
     assert launches(0) == fused
     assert launches(1, (2, 1)) == fused + 1
     assert launches(1, (0, 32)) == fused + 1
+
+
+# 2048 rows and more, where the row-resident sweeps of a full field are the built-in
+# ones: part of one slot, one, part of two, two; two warps with part of two
+# slots (plain sweep only) and with two
+@pytest.mark.parametrize("dims", [(96, 32, 64), (128, 64, 32), (160, 64, 32), (224, 32, 64), (256, 64, 32),
+                                  (288, 64, 32), (448, 32, 64), (512, 64, 32), (64, 48, 32), (32, 64, 64)])
+@pytest.mark.parametrize("nu,alpha,zero", [(2, 0.1, True), (1, 0.0, False), (2, 0.0, True)])
+def test_sweeps_of_a_full_field(ibrd, dims, nu, alpha, zero):
+    """Two sweeps on each side, or a guess: the cycles whose sweeps read a full
+    field (2e-5 of the definition, the bound of the other FP32 V-cycle tests)."""
+    import torch
+    rng = np.random.default_rng(dims[0] + nu)
+    b, x0 = (rng.standard_normal(dims[::-1]).astype(np.float32) for _ in (0, 1))
+    g = ibrd.Grid(*dims, alpha=alpha)
+    x = g.vcycle_f32(torch.from_numpy(b).cuda(), torch.from_numpy(x0).cuda(), zero, nu1=nu, nu2=nu)
+    want = mg.vcycle(b.astype(np.float64), 1.0, 1.0, alpha, x0=None if zero else x0.astype(np.float64), nu1=nu,
+                     nu2=nu, exact_cells=32768, exact_side=64)
+    assert rel_max(x.cpu().numpy().astype(np.float64), want) < 2e-5
+
+
+@pytest.mark.parametrize("dims", [(32, 256, 256), (64, 512, 512), (384, 16, 16), (96, 16, 16), (256, 256, 64)])
+def test_built_in_sweeps_are_not_slower(ibrd, dims):
+    """The built-in shapes of a cycle with two sweeps on each side against tiled
+    sweeps on its finest level (5 % for the clock)."""
+    import torch
+    width = 64 if dims[0] % 64 == 0 else 32
+    fields = [torch.randn(dims[::-1], device="cuda") for _ in range(3)]
+    handles = [ibrd.Grid(*dims, alpha=0.1) for _ in (0, 1)]
+    ibrd.ibrd_tune_set(handles[1].handle, 4, 0, *dims, width, 0)
+    best = [1e9, 1e9]
+    for k in range(24):
+        g = handles[k % 2]
+        for warm in (True, False):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(2 if warm else 12):
+                g.vcycle_f32(fields[0], fields[1], nu1=2, nu2=2)
+                g.vcycle_f32(fields[1], fields[2], nu1=2, nu2=2)
+            e1.record()
+            e1.synchronize()
+        best[k % 2] = min(best[k % 2], e0.elapsed_time(e1))
+    assert best[0] < 1.05 * best[1]
