@@ -367,12 +367,12 @@ ibrd_status ibrd_solve_many(int count, const ibrd_solve_item* items, int threads
 /* Autotuner (not in the paper: launch-shape selection for this library's
    kernels). For every multigrid level whose red-black sweeps (Sec. III.E) run
    as a fused one-pass sweep kernel, times candidate launch shapes of the
-   sweep -- the row-resident FP32 kernel (levels whose rows are a multiple of
-   32 of at most 512 cells; tx = nx at 128 and 256 cells, else 0) or the tiled
-   kernel with tile width 32 or 64 cells (FP32) or 32 (FP64), each with z-march depths (planes per CTA, 2 to 512) -- and
-   the z-march depth of the stencil pass that forms the first
-   sweep from a zero guess (FP32), on scratch fields of the level's size with
-   CUDA events, and keeps a shape only when it is at least 3 % faster than the
+   sweep -- z-march depths (planes per CTA, 2 to 512) of the row-resident FP32
+   kernel on levels it serves (rows of a multiple of 32 cells, at most 512; tx =
+   nx at 128 and 256 cells, else 0), elsewhere of the tiled kernel, whose tile is
+   32 or 64 cells (FP32) or 32 (FP64) wide -- and the z-march depth of the
+   stencil pass that forms the first sweep from a zero guess (FP32), on scratch
+   fields of the level's size with CUDA events, and keeps a shape only when it is at least 3 % faster than the
    built-in one. Shapes tuned before in this process for the same device and
    grid are reused without timing unless retune != 0. Every later call on the
    handle launches the kept shapes; results can change in the last bits only

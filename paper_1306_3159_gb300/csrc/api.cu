@@ -2208,7 +2208,14 @@ void autotune_levels(ibrd_grid g, bool retune, std::vector<ibrd_tune_entry>& rep
           if (kind == TUNE_SWEEP) {
             txs = {32};
             if (elem == 4 && d.nx % 64 == 0) txs.push_back(64);
-            if (elem == 4 && rows_sweep_ok(d)) txs.push_back(rows_named(d) ? d.nx : 0);
+            // a tiled shape also takes the cycle's transfers off the row-resident
+            // kernels, which costs more than a plain sweep can gain (sweep_rows.cu):
+            // levels they serve keep them, and have a depth to choose where they
+            // run the plain sweep too
+            if (elem == 4 && rows_sweep_ok(d)) {
+              txs.clear();
+              if (rows_plain_ok(d)) txs.push_back(rows_named(d) ? d.nx : 0);
+            }
           }
           static const int zcs[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
           for (int tx : txs)

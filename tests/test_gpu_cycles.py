@@ -86,3 +86,24 @@ def test_built_in_sweeps_are_not_slower(ibrd, dims):
             e1.synchronize()
         best[k % 2] = min(best[k % 2], e0.elapsed_time(e1))
     assert best[0] < 1.05 * best[1]
+
+
+@pytest.mark.parametrize("dims", [(64, 256, 256), (96, 64, 64), (160, 32, 32), (128, 64, 32)])
+def test_tuning_keeps_the_fused_cycle(ibrd, dims):
+    """Tuned shapes change depths on levels the row-resident kernels serve, not the
+    kernels: the cycle has as many launches as before."""
+    import torch
+    b = torch.randn(dims[::-1], device="cuda")
+    g = ibrd.Grid(*dims, alpha=0.1)
+
+    def launches():
+        g.vcycle_f32(b, nu1=1, nu2=1)
+        ibrd.ibrd_profile_read(g.handle)
+        g.vcycle_f32(b, nu1=1, nu2=1)
+        return ibrd.ibrd_profile_read(g.handle)["launches"]
+
+    before = launches()
+    for r in ibrd.ibrd_autotune(g.handle, 1, retune=True):
+        if r["kind"] == 0 and r["nx"] % 32 == 0 and r["nx"] <= 512 and r["ny"] % 8 == 0:
+            assert r["tx"] in (0, r["nx"] if r["nx"] in (128, 256) else 0)
+    assert launches() == before
