@@ -372,15 +372,15 @@ ibrd_status ibrd_solve_many(int count, const ibrd_solve_item* items, int threads
    nx at 128 and 256 cells, else 0), elsewhere of the tiled kernel, whose tile is
    32 or 64 cells (FP32) or 32 (FP64) wide -- and the z-march depth of the
    stencil pass that forms the first sweep from a zero guess (FP32), on scratch
-   fields of the level's size with CUDA events, and keeps a shape only when it is at least 3 % faster than the
-   built-in one. Shapes tuned before in this process for the same device and
-   grid are reused without timing unless retune != 0. Every later call on the
-   handle launches the kept shapes; results can change in the last bits only
-   (per-CTA partial sums group differently). Drops the handle's captured CUDA
-   graphs. precision: IBRD_FP64 tunes the FP64 kernels, either mixed mode the
-   FP32 ones, -1 both. out (may be NULL if cap = 0) receives up to cap
-   records; *n_out (may be NULL) the number of records. Allocates six
-   scratch fields of the finest grid for the duration of the call (two sets
+   fields of the level's size with CUDA events, and keeps a shape only when it
+   is at least 3 % faster than the built-in one. Shapes tuned before in this
+   process for the same device and grid are reused without timing unless retune
+   != 0. Every later call on the handle launches the kept shapes; results can
+   change in the last bits only (per-CTA partial sums group differently). Drops
+   the handle's captured CUDA graphs. precision: IBRD_FP64 tunes the FP64
+   kernels, either mixed mode the FP32 ones, -1 both. out (may be NULL if cap =
+   0) receives up to cap records; *n_out (may be NULL) the number of records.
+   Allocates six scratch fields of the finest grid for the duration of the call (two sets
    of x in, x out and b that consecutive timed sweeps alternate between, so
    that levels larger than half the L2 stream from DRAM as in a V-cycle).
    Synchronizes the stream. */
