@@ -88,7 +88,7 @@ __device__ void givens_step(double* __restrict__ H, int ldh, int j, double* __re
   *res = fabs(gvec[j + 1]);
 }
 
-// The Gram-Schmidt norm estimate (see k_gs_norm_estimate), by one warp.
+// The Gram-Schmidt norm estimate (DotTail), by one warp.
 __device__ void gs_norm_estimate_warp(const double* __restrict__ h, int nb, double* __restrict__ ww,
                                       double* __restrict__ hhat, double* __restrict__ hinv) {
   const int lane = threadIdx.x & 31;
@@ -105,7 +105,7 @@ __device__ void gs_norm_estimate_warp(const double* __restrict__ h, int nb, doub
   *hinv = r > 0.0 ? 1.0 / r : 0.0;
 }
 
-// The Gram-Schmidt norm fix (see k_gs_norm_fix) for rho2 = ||stored||^2. One thread.
+// The Gram-Schmidt norm fix (AxpyTail, hhat) for rho2 = ||stored||^2. One thread.
 __device__ void gs_norm_fix_one(double rho2, const double* __restrict__ hhat, double* __restrict__ hsub,
                                 double* __restrict__ vscale, double* __restrict__ sq) {
   const double r = sqrt(fmax(rho2, 0.0));

@@ -64,8 +64,9 @@ struct NaLevel {
 };
 
 // The same hierarchy rules as a grid handle: halve while every side is even
-// and >= 4; the coarse end runs in one CTA from the first level whose
-// remaining levels (x and b, FP64) fit in 160 KB of shared memory.
+// and >= 4; the coarse end runs on a thread block cluster from the first level
+// that fits one, else in one CTA from the first level whose remaining levels
+// (x and b, FP64) fit in 160 KB of shared memory (small_from).
 struct NaPlan {
   std::vector<NaLevel> lv;
   int small_from = 0;
