@@ -7,7 +7,7 @@
 // (86 us in the single-CTA kernel of smoother.cu, most of it that). Separate
 // launches over the whole chip cost about 3 us for each half-sweep of a level
 // this small. Here 16 CTAs of a cluster share the levels of 600 cells and more,
-// and its CTA 0 runs the rest in its own shared memory. 32^3 and below: 68 us,
+// and its CTA 0 runs the rest in its own shared memory. 32^3 and below: 70 us,
 // against 147 us for the separate kernels of the 32^3 level and the single-CTA
 // one of the others; 24^3 and below: 51 us, against 95.
 //
