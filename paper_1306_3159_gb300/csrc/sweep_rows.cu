@@ -845,9 +845,12 @@ CUtensorMap field_map(const float* f, int nx, int ny, int nz, int rows) {
   return m;
 }
 
+// The maps of a field whose tiles have `rows` rows: only those that load_rows
+// uses for ny rows (an encoding is most of a microsecond of host time, which
+// counts on levels whose kernels take five).
 RowMaps row_maps(const float* f, int nx, int ny, int nz, int rows, int halo) {
   RowMaps m{};
-  if (ny > rows) m.all = field_map(f, nx, ny, nz, rows + 2 * halo);
+  if (ny >= 3 * rows) m.all = field_map(f, nx, ny, nz, rows + 2 * halo);
   m.part = field_map(f, nx, ny, nz, ny >= 2 * rows ? rows + halo : rows);
   m.halo = field_map(f, nx, ny, nz, halo);
   return m;
