@@ -468,10 +468,10 @@ int vcycle_level(ibrd_grid g, int l, const T* b, const double* bshift, T* x, boo
                               g->s);
     prof_end(P_RBGS32, g->s, "zero_restrict_rows", (packed ? 6.5 : 8.5) * lv.d.n());
   } else if (tile) {
-    // rows above 512 cells: the single pre-smoothing sweep from zero and the
-    // restriction in one pass over tiles (levels of up to 2^21 cells; on larger
-    // ones the kernel is bound by its shared-memory traffic and the two
-    // streaming kernels are faster)
+    // rows above 512 cells, or few above 256: the single pre-smoothing sweep
+    // from zero and the restriction in one pass over tiles (levels of up to 2^21
+    // cells; on larger ones the kernel is bound by its shared-memory traffic and
+    // the two streaming kernels are faster)
     launch_zero_restrict(reinterpret_cast<const float*>(b), bshift, reinterpret_cast<float*>(cur),
                          reinterpret_cast<float*>(H.b[l + 1]), lv.d, st, g->s);
   } else {

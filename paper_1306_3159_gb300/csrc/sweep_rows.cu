@@ -29,12 +29,11 @@
 //   idle and take one more shuffle for the wrap; rows above 256 cells belong to
 //   two warps, whose outermost groups read their neighbour from the published
 //   row in shared memory. FP32 V-cycles of one pre- and one post-sweep, which
-//   run the sweep from zero and the packed sweep below, are faster with them at
-//   every length than with the tiled sweep and separate transfers: 49 and 60 us on
-//   32 x 64 x 64 cells, 73 and 88 at 96^3, 117 and 151 at 160^3, 157 and 222 at 224^3,
-//   361 and 446 at 320^3, 537 and 1330 at 512^3 (the largest cube a CTA's shared
-//   memory holds rows of). Where the other two forms, which read a full field,
-//   are slower, rows_plain_ok and rows_prolong_full_ok leave them out.
+//   run the sweep from zero and the packed sweep below, against ones of the tiled sweep
+//   and separate transfers: 73 and 88 us at 96^3, 117 and 151 at 160^3, 157 and 222 at
+//   224^3, 361 and 446 at 320^3, 537 and 1330 at 512^3 (the largest cube a CTA's shared
+//   memory holds rows of). Which levels take which form: zero_restrict_rows_ok,
+//   rows_plain_ok, rows_prolong_full_ok.
 // * A CTA owns TY rows of every plane of a z-chunk, plus one halo row on each
 //   side in y whose red cells it also updates (the black cells at the tile's
 //   edge rows need them); the neighbouring CTA computes the same red values
@@ -992,7 +991,15 @@ int launch_rows_prolong_sweep(const float* xc, const float* xin, bool packed, fl
                 : sweep_rows_any<IN_FULL_PRO>(xin, xc, xout, b, bshift, d, st, zc, part, part_cap, s);
 }
 
-bool zero_restrict_rows_ok(Dims d) { return rows_sweep_ok(d); }
+// The sweep from zero and the packed sweep that follows it, against the tiled sweep
+// from zero with the restriction, the prolongation and the tiled sweep (us, data in
+// L2): rows of 128 cells 10.2 and 9.9 on 8 x 8, 10.0 and 10.9 on 16 x 16; of 224
+// 11.9 and 11.5 on 16 x 16, 12.5 and 13.8 on 32 x 32 (and one launch less). Two warps
+// per row start later: of 320 15.6 and 12.0 on 16 x 16, 15.7 and 15.1 on 32 x 32, 16.4
+// and 18.2 on 32 x 64; of 512 14.2 and 11.5, 14.2 and 17.1, 14.3 and 21.3.
+bool zero_restrict_rows_ok(Dims d) {
+  return rows_sweep_ok(d) && (d.nx <= 256 || d.ny * (size_t)d.nz >= 1024);
+}
 
 int zero_restrict_rows_default_zc(Dims d) {
   return rows_sweep_default_zc(d);  // even: plane pairs of the restriction stay inside a chunk

@@ -107,3 +107,25 @@ def test_tuning_keeps_the_fused_cycle(ibrd, dims):
         if r["kind"] == 0 and r["nx"] % 32 == 0 and r["nx"] <= 512 and r["ny"] % 8 == 0:
             assert r["tx"] in (0, r["nx"] if r["nx"] in (128, 256) else 0)
     assert launches() == before
+
+
+# the packed black cells' kernels where two warps per row begin (1024 rows), and
+# one tile of rows
+@pytest.mark.parametrize("dims", [(288, 32, 32), (320, 64, 32), (448, 32, 64), (512, 32, 32), (96, 8, 8),
+                                  (256, 8, 16)])
+@pytest.mark.parametrize("nu2,alpha,zc", [(0, 0.1, 0), (1, 0.0, 0), (1, 0.1, 2), (1, 0.0, 6), (2, 0.1, 0)])
+def test_packed_cells_and_the_correction_apart(ibrd, dims, nu2, alpha, zc):
+    """One sweep before: the cycle's definition (2e-5), and bit for bit the one with
+    the correction kept apart."""
+    import torch
+    b = np.random.default_rng(dims[0] + zc).standard_normal(dims[::-1]).astype(np.float32)
+    out = []
+    for apart in (0, 1):
+        g = ibrd.Grid(*dims, alpha=alpha)
+        if zc:
+            ibrd.ibrd_tune_set(g.handle, 4, 0, *dims, 0, zc)
+        ibrd.ibrd_tune_set(g.handle, 4, 2, *dims, apart, 0)
+        out.append(g.vcycle_f32(torch.from_numpy(b).cuda(), nu1=1, nu2=nu2).cpu().numpy())
+    assert np.array_equal(out[0], out[1])
+    want = mg.vcycle(b.astype(np.float64), 1.0, 1.0, alpha, nu1=1, nu2=nu2, exact_cells=32768, exact_side=64)
+    assert rel_max(out[0].astype(np.float64), want) < 2e-5
