@@ -414,9 +414,9 @@ double ibrd_periodic_constant(double lx, double ly, double lz);
    the built-in rule is the in-place half sweeps; tx = 32, or tx = 0 with zc > 0,
    selects the tiled kernel.
    kind 2 (FP32 only, zc = 0) is the coarse-grid correction of the level: on
-   levels the row-resident sweep serves (with more than one sweep before it:
-   where that is faster), the V-cycle adds the prolongation of the coarse
-   correction inside the first post-smoothing sweep (one pass over
+   levels the row-resident sweep serves, where it is the faster form, the
+   V-cycle adds the prolongation of the coarse correction inside the first
+   post-smoothing sweep (one pass over
    x instead of two; the same values bit for bit); tx = 1 keeps it a separate
    kernel, tx = 0 restores the default. Drops the handle's captured CUDA
    graphs. */
